@@ -45,6 +45,8 @@ struct BatchPlan {
   int4* d_tiles_pair = nullptr;
   int ntiles_pair = 0;
   bool pair = false;
+  // the FP32 path's products have only the 256 x 256 form
+  bool on_pairs() const { return pair || prec == PSD_PREC_FP32; }
   int4* d_symv = nullptr;
   int nsymv = 0;
   int4* d_cast = nullptr;
@@ -364,7 +366,7 @@ psd_status_t build_bplan(BatchPlan* p) {
 }
 
 void* bpart(const BatchPlan* p, const Mat& m, int part) {
-  return p->slots + (static_cast<size_t>(m.slot) + static_cast<size_t>(part * kind_lo_step(m.kind))) * p->slot_size;
+  return p->slots + (static_cast<size_t>(m.slot) + static_cast<size_t>(part)) * p->slot_size;
 }
 
 // The chain form: run_chain's sequence recorded without launching anything
@@ -458,7 +460,9 @@ cudaError_t bgemm(BatchPlan* p, int epi, const Mat& A, const Mat& B, const Mat* 
     g.ep.Y_lo = kind_is_pair(Y->kind) ? bpart(p, *Y, 1) : nullptr;
     g.ep.ldy = p->ldm;
   }
-  g.ep.in_scale = g.ep.y_scale = g.ep.out_scale = 1.f;
+  g.ep.in_scale = 1.f / (A.scale * B.scale);
+  g.ep.y_scale = Y ? 1.f / Y->scale : 1.f;
+  g.ep.out_scale = out ? out->scale : 1.f;
   if (epi == EPI_FINAL) g.ep.cres = p->d_cres;
   const int grid = num_sms();
   const int64_t cols = p->ldm, rows = p->R;
@@ -484,7 +488,18 @@ cudaError_t bgemm(BatchPlan* p, int epi, const Mat& A, const Mat& B, const Mat* 
     g.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | (8u << 24);
     return launch_symgemm(dt, epi, ta, tb, g, grid, s, out ? kind_dtype(*out) : -1, /*many_small=*/true);
   }
-  if (route == ROUTE_NONE) return cudaErrorNotSupported;
+  if (route == ROUTE_NONE || (epi == EPI_FINAL && (route == ROUTE_X3 || route == ROUTE_X2)))
+    return cudaErrorNotSupported;
+  if (route == ROUTE_F32) {
+    const Mat* ops[2] = {&A, &B};
+    CUtensorMap tm[4];
+    for (int i = 0; i < 4; ++i)
+      if (!encode_tmap_rows(&tm[i], DT_F16X2, bpart(p, *ops[i >> 1], i & 1), cols, rows, p->ldm, 128, 64))
+        return cudaErrorInvalidValue;
+    g.num_tiles = p->ntiles_pair;
+    g.tiles = p->d_tiles_pair;
+    return launch_symgemm_f32(epi, tm, g, grid, s);
+  }
   const bool b1 = route == ROUTE_X2;
   const Mat& PA = b1 ? B : A;  // the pair operand goes first
   const Mat& PB = b1 ? A : B;
@@ -496,7 +511,7 @@ cudaError_t bgemm(BatchPlan* p, int epi, const Mat& A, const Mat& B, const Mat* 
       !encode_tmap_rows(&tm[2], dt, bpart(p, PB, 0), cols, rows, p->ldm, 256, rb) ||
       !encode_tmap_rows(&tm[3], dt, bpart(p, PB, b1 ? 0 : 1), cols, rows, p->ldm, 256, rb))
     return cudaErrorInvalidValue;
-  const int out_mode = epi == EPI_FINAL ? 2 : (kind_is_pair(out->kind) ? 0 : 1);
+  const int out_mode = kind_is_pair(out->kind) ? 0 : 1;  // the final product of these chains is a 16-bit one
   return launch_symgemm_x3(dt, b1, epi, out_mode, tm, g, grid, s);
 }
 
@@ -504,7 +519,7 @@ struct BatchOps {
   BatchPlan* p;
   cudaStream_t s;
   cudaError_t cast(const Mat& X0) {
-    BatchCast bc{bpart(p, X0, 0), kind_is_pair(X0.kind) ? bpart(p, X0, 1) : nullptr, p->ldm};
+    BatchCast bc{bpart(p, X0, 0), kind_is_pair(X0.kind) ? bpart(p, X0, 1) : nullptr, p->ldm, X0.scale};
     return enqueue_batch_cast(kind_dtype(X0), bc, p->d_bb, p->d_st, p->d_cast, p->ncast, s);
   }
   cudaError_t gemm(int epi, const Mat& A, const Mat& B, const Mat* out, const Mat* Y, float a, float b, float c,
@@ -512,7 +527,7 @@ struct BatchOps {
     return bgemm(p, epi, A, B, out, Y, a, b, c, sc, track, s);
   }
   cudaError_t finish() {
-    return enqueue_batch_finalize(p->d_bb, p->d_st, p->count, p->d_cres, p->d_cidx, p->d_crange, p->pair ? 16 : 4,
+    return enqueue_batch_finalize(p->d_bb, p->d_st, p->count, p->d_cres, p->d_cidx, p->d_crange, p->on_pairs() ? 16 : 4,
                                   p->flow ? p->d_flowctl + 1 : nullptr,
                                   s);
   }
@@ -614,14 +629,14 @@ psd_status_t tune_bplan(BatchPlan* p) {
     return PSD_ERR_CUDA;
   // each block's final-product shares, in the block's own tile order (schedule-independent
   // sums), positions in the tile list the final product runs over
-  const std::vector<int4> tf = p->pair ? pair_tiles(p->sizes) : t;
+  const std::vector<int4> tf = p->on_pairs() ? pair_tiles(p->sizes) : t;
   std::map<std::tuple<int, int, int>, int> pos;
   for (int i = 0; i < static_cast<int>(tf.size()); ++i) pos[std::make_tuple(tf[i].z, tf[i].x, tf[i].y)] = i;
   std::vector<int> cidx;
   std::vector<int2> crange(p->count);
   for (int b = 0; b < p->count; ++b) {
     crange[b].x = static_cast<int>(cidx.size());
-    const std::vector<int4> own = p->pair ? make_tile_list_pair(p->sizes[b], b, 8) : make_tile_list(p->sizes[b], b, 8);
+    const std::vector<int4> own = p->on_pairs() ? make_tile_list_pair(p->sizes[b], b, 8) : make_tile_list(p->sizes[b], b, 8);
     for (const int4& c : own) cidx.push_back(pos.at(std::make_tuple(b, c.x, c.y)));
     crange[b].y = static_cast<int>(cidx.size()) - crange[b].x;
   }

@@ -910,28 +910,25 @@ __device__ __forceinline__ void put4_16(uint16_t* H, const uint16_t (&u)[4], int
     for (int k = 0; k < valid; ++k) H[k] = u[k];
   }
 }
-__device__ __forceinline__ float tf32_round(float v) {
-  if (!isfinite(v)) return v;
-  return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);
-}
-
 template <int DT>
 __device__ __forceinline__ void bstore4(const BatchCast& c, int64_t pos, const float (&v)[4], int valid) {
-  if (DT == DT_TF32X3) {
-    float* Mh = static_cast<float*>(c.M) + pos;
-    float* Ml = static_cast<float*>(c.M_lo) + pos;
-    for (int k = 0; k < valid; ++k) {
-      const float h = tf32_round(v[k]);
-      Mh[k] = h;
-      Ml[k] = tf32_round(v[k] - h);
+  uint16_t u[4];
+  if (DT == DT_F16X2) {
+    uint16_t l[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float x = v[k] * c.scale;
+      const __half h = __float2half_rn(x);
+      u[k] = __half_as_ushort(h);
+      l[k] = __half_as_ushort(__float2half_rn(x - __half2float(h)));
     }
+    put4_16(static_cast<uint16_t*>(c.M_lo) + pos, l, valid);
   } else {
-    uint16_t u[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
       u[k] = DT == DT_BF16 ? __bfloat16_as_ushort(__float2bfloat16_rn(v[k])) : __half_as_ushort(__float2half_rn(v[k]));
-    put4_16(static_cast<uint16_t*>(c.M) + pos, u, valid);
   }
+  put4_16(static_cast<uint16_t*>(c.M) + pos, u, valid);
 }
 
 // X_0 of every block into the stacked buffers (64 x 64 upper tiles, item =
@@ -1102,7 +1099,7 @@ cudaError_t enqueue_batch_cast(int dtype, const BatchCast& c, const BatchBlock* 
   switch (dtype) {
     case DT_F16: bcast_kernel<DT_F16><<<nitems, 256, 0, s>>>(c, blk, st, items); break;
     case DT_BF16: bcast_kernel<DT_BF16><<<nitems, 256, 0, s>>>(c, blk, st, items); break;
-    case DT_TF32X3: bcast_kernel<DT_TF32X3><<<nitems, 256, 0, s>>>(c, blk, st, items); break;
+    case DT_F16X2: bcast_kernel<DT_F16X2><<<nitems, 256, 0, s>>>(c, blk, st, items); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

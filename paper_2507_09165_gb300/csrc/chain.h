@@ -24,7 +24,7 @@ namespace psd {
 // Storage of one matrix of the chain (workspace slots of n x ldm 16-bit elements).
 enum MatKind : int {
   MK_16 = 0,      // one FP16 or BF16 matrix (Mat::dt16)
-  MK_TF32X3 = 2,  // TF32 hi/lo pair in FP32 containers (4 slots)
+  MK_F32X2 = 2,   // FP32 path: FP16 hi/lo pair of the values times Mat::scale (2 slots)
   MK_E4M3 = 3,    // e4m3 values times Mat::scale (1 slot)
   MK_F16X2 = 4,   // FP16 hi/lo pair (2 slots)
 };
@@ -33,18 +33,16 @@ struct Mat {
   int kind = MK_16;
   int slot = -1;
   int dt16 = DT_F16;  // element type of an MK_16 matrix
-  float scale = 1.f;  // MK_E4M3: stored value = RN_e4m3(value * scale)
+  float scale = 1.f;  // MK_E4M3, MK_F32X2: the stored matrix holds value * scale (a power of two)
 };
 
 inline int kind_slots(int kind) {
-  return kind == MK_TF32X3 ? 4 : kind == MK_F16X2 ? 2 : 1;
+  return kind == MK_F32X2 || kind == MK_F16X2 ? 2 : 1;
 }
 inline int kind_dtype(const Mat& m) {
-  return m.kind == MK_16 ? m.dt16 : m.kind == MK_E4M3 ? DT_E4M3 : m.kind == MK_F16X2 ? DT_F16X2 : DT_TF32X3;
+  return m.kind == MK_16 ? m.dt16 : m.kind == MK_E4M3 ? DT_E4M3 : DT_F16X2;
 }
-// Slot offset of the lo part of a pair.
-inline int kind_lo_step(int kind) { return kind == MK_TF32X3 ? 2 : 1; }
-inline bool kind_is_pair(int kind) { return kind == MK_TF32X3 || kind == MK_F16X2; }
+inline bool kind_is_pair(int kind) { return kind == MK_F32X2 || kind == MK_F16X2; }
 
 // Mixed precision: P of the first kMixedPStages stages as an FP16 pair, and Y
 // of stages kMixedYFirst .. kMixedYLast (0-based) too; X_t stays FP16.  The
@@ -67,6 +65,15 @@ constexpr int kFp8Stages = 2;
 constexpr float kFp8ScaleX = 256.f;
 constexpr float kFp8ScaleY = 256.f;
 
+// FP32 path: scales of the FP16 pairs.  |X_t(i,j)|, |Y(i,j)| <= their spectral
+// norms (~1.03 in the composite's basin) and |P(i,j)| <= a_1 = 8.3; entries of
+// a spread iterate are ~1/sqrt(n).  2^13 and 2^12 leave a factor 8 and 2 below
+// FP16's 65504, and put the lo parts' smallest step at 2^-37 and 2^-36 in place
+// of an unscaled pair's 2^-24 (which at n = 10,000 is coarser than the pair's
+// own 2^-23 relative step for every entry).
+constexpr float kF32ScaleX = 8192.f;
+constexpr float kF32ScaleP = 4096.f;
+
 inline float fp8_poly_scale(const double (&c)[3]) {
   double m = 0.0;
   const double ys[3] = {0.0, 1.25, c[2] != 0.0 ? -c[1] / (2.0 * c[2]) : 0.0};
@@ -84,7 +91,7 @@ struct StageKinds {
 };
 inline StageKinds stage_kinds(psd_precision_t prec, int t, int T) {
   auto xk = [&](int s) {
-    if (prec == PSD_PREC_FP32) return static_cast<int>(MK_TF32X3);
+    if (prec == PSD_PREC_FP32) return static_cast<int>(MK_F32X2);
     if (prec == PSD_PREC_FP8_LATE && s >= T - kFp8Stages) return static_cast<int>(MK_E4M3);
     return static_cast<int>(MK_16);
   };
@@ -96,7 +103,7 @@ inline StageKinds stage_kinds(psd_precision_t prec, int t, int T) {
   } else {
     k.y = k.p = k.x;
   }
-  k.out = prec == PSD_PREC_FP32 ? static_cast<int>(MK_TF32X3) : (t + 1 < T ? xk(t + 1) : static_cast<int>(MK_16));
+  k.out = prec == PSD_PREC_FP32 ? static_cast<int>(MK_F32X2) : (t + 1 < T ? xk(t + 1) : static_cast<int>(MK_16));
   return k;
 }
 
@@ -133,31 +140,31 @@ cudaError_t run_chain(psd_precision_t prec, const Schedule& sched, int nslots, i
     }
   } hw{pool, high_water};
   const int T = sched.T;
-  auto make = [&](int kind, float scale) {
+  auto make = [&](int kind, float scale8, float scale32) {
     Mat m;
     m.kind = kind;
     m.dt16 = dt16;
-    m.scale = kind == MK_E4M3 ? scale : 1.f;
+    m.scale = kind == MK_E4M3 ? scale8 : kind == MK_F32X2 ? scale32 : 1.f;
     m.slot = pool.alloc(kind_slots(kind));
     return m;
   };
-  Mat X0 = make(stage_kinds(prec, 0, T).x, kFp8ScaleX);
+  Mat X0 = make(stage_kinds(prec, 0, T).x, kFp8ScaleX, kF32ScaleX);
   if (X0.slot < 0) return cudaErrorMemoryAllocation;
   if ((e = ops.cast(X0)) != cudaSuccess) return e;
   Mat cur = X0;
   for (int t = 0; t < T; ++t) {
     const StageKinds k = stage_kinds(prec, t, T);
-    Mat Y = make(k.y, kFp8ScaleY);
+    Mat Y = make(k.y, kFp8ScaleY, kF32ScaleX);
     if (Y.slot < 0) return cudaErrorMemoryAllocation;
     if ((e = ops.gemm(EPI_COPY, cur, cur, &Y, nullptr, 0.f, 0.f, 0.f, 1.f, false)) != cudaSuccess) return e;
-    Mat P = make(k.p, fp8_poly_scale(sched.coef[t]));
+    Mat P = make(k.p, fp8_poly_scale(sched.coef[t]), kF32ScaleP);
     if (P.slot < 0) return cudaErrorMemoryAllocation;
     if ((e = ops.gemm(EPI_POLY, Y, Y, &P, &Y, static_cast<float>(sched.coef[t][0]),
                       static_cast<float>(sched.coef[t][1]), static_cast<float>(sched.coef[t][2]), 1.f, false)) !=
         cudaSuccess)
       return e;
     pool.release(Y);
-    Mat Xn = make(k.out, kFp8ScaleX);
+    Mat Xn = make(k.out, kFp8ScaleX, kF32ScaleX);
     if (Xn.slot < 0) return cudaErrorMemoryAllocation;
     if ((e = ops.gemm(EPI_SCALE, cur, P, &Xn, nullptr, 0.f, 0.f, 0.f, static_cast<float>(1.0 / sched.post[t]),
                       t == T - 1)) != cudaSuccess)
@@ -172,14 +179,16 @@ cudaError_t run_chain(psd_precision_t prec, const Schedule& sched, int nslots, i
 
 // Which kernel forms a product of the given operand kinds:
 //   both MK_16 or both MK_E4M3: the 16-bit/e4m3 kernel (symgemm.cu);
-//   both pairs of one type:      the split kernel (symgemm_x3.cu), three products;
+//   both MK_F16X2:               the split kernel (symgemm_x3.cu), three products;
+//   both MK_F32X2:               the FP32 path's kernel (symgemm_f32.cu), three products;
 //   MK_16 A with an MK_F16X2 B:  the split kernel's single-B instance with the
 //                                operands exchanged (B A = A B: they commute),
 //                                two products.
-enum GemmRoute : int { ROUTE_16 = 0, ROUTE_X3 = 1, ROUTE_X2 = 2, ROUTE_NONE = 3 };
+enum GemmRoute : int { ROUTE_16 = 0, ROUTE_X3 = 1, ROUTE_X2 = 2, ROUTE_F32 = 3, ROUTE_NONE = 4 };
 inline GemmRoute gemm_route(const Mat& A, const Mat& B) {
   if ((A.kind == MK_16 || A.kind == MK_E4M3) && A.kind == B.kind) return ROUTE_16;
-  if (kind_is_pair(A.kind) && A.kind == B.kind) return ROUTE_X3;
+  if (A.kind == MK_F32X2 && B.kind == MK_F32X2) return ROUTE_F32;
+  if (A.kind == MK_F16X2 && B.kind == MK_F16X2) return ROUTE_X3;
   if (A.kind == MK_16 && A.dt16 == DT_F16 && B.kind == MK_F16X2) return ROUTE_X2;
   return ROUTE_NONE;
 }

@@ -53,8 +53,8 @@ struct DevState {
 // Epilogue kinds of the symmetric product (fused into the tensor-core kernel).
 enum Epi : int { EPI_COPY = 0, EPI_POLY = 1, EPI_SCALE = 2, EPI_FINAL = 3 };
 
-// Operand storage of the chain: single 16-bit or e4m3 matrices, TF32 hi/lo
-// pairs (FP32 containers), FP16 hi/lo pairs.
+// Operand storage: single 16-bit or e4m3 matrices, FP16 hi/lo pairs, and (the
+// product entry point only) TF32 hi/lo pairs in FP32 containers.
 // Element types; the X2/X3 names are hi/lo pairs (DT_F16X2: FP16 hi + FP16 lo).
 enum Dtype : int { DT_F16 = 0, DT_BF16 = 1, DT_TF32X3 = 2, DT_E4M3 = 4, DT_F16X2 = 5 };
 
@@ -94,10 +94,10 @@ struct EpiParams {
   int absmax_blocks;     // 1: atomic max of |output| into blocks[b].st->absmax_bits;
                          // 2: the same for the blocks with a nonzero `track`
   int per_block_coef;    // nonzero: a, b, c, s from each tile's block record
-  // e4m3 operands / outputs (the 16-bit kernel's FP8 instances): every e4m3
-  // matrix holds its values times a power of two; the accumulator is
+  // e4m3 operands / outputs (the 16-bit kernel's FP8 instances) and the FP32
+  // path's scaled pairs: every such matrix holds its values times a power of two; the accumulator is
   // multiplied by in_scale = 1 / (scale_A scale_B), the EPI_POLY operand Y by
-  // y_scale = 1 / scale_Y, and an e4m3 output is rounded from value * out_scale.
+  // y_scale = 1 / scale_Y, and the output is rounded from value * out_scale.
   float in_scale, y_scale, out_scale;
   unsigned* absmax;      // if set: atomic max of |output| into this word instead
   int* status;           // device status word for timeouts
@@ -294,6 +294,11 @@ cudaError_t launch_symgemm_chain(int dtype, const ChainMaps& maps, const ChainPr
 // or a single B with EPI_SCALE and an FP16 output.
 cudaError_t launch_symgemm_x3(int et, bool b_single, int epi, int out, const CUtensorMap* tm, const GemmParams& p,
                               int grid, cudaStream_t stream, bool pair = false);
+// The FP32 path's product (symgemm_f32.cu): scaled FP16 pairs on SM pairs,
+// promoted accumulation; tm = {A_hi, A_lo, B_hi, B_lo}, each with 128-row
+// boxes of 64 bytes; tiles from make_tile_list_pair; ep.in_scale / y_scale /
+// out_scale carry the operands' scales; EPI_FINAL writes 16 shares per tile.
+cudaError_t launch_symgemm_f32(int epi, const CUtensorMap* tm, const GemmParams& p, int grid, cudaStream_t stream);
 int num_sms();
 
 // --- batched projection of a block-diagonal cone (batched_kernels.cu) ---
@@ -328,6 +333,7 @@ struct BatchCast {
   void* M;                // X_0: stacked iterate buffer (hi part of a pair)
   void* M_lo;
   int64_t ldm;
+  float scale;            // pairs: the values are stored times this power of two
 };
 
 cudaError_t enqueue_batch_norm_bound(const BatchLanczos& L, int count, const int4* symv_items, int nsymv,
@@ -393,9 +399,9 @@ cudaError_t enqueue_norm_bound(const LanczosBufs& b, const DevArgs* args, DevSta
                                cudaStream_t stream, bool persistent = true);
 // Frees the cached plans of psd_project_deflate (device synchronised by the caller).
 void release_deflate_plans();
-// X_0 = X / lam~ as `dtype` (DT_F16, DT_BF16, or DT_TF32X3 with M = hi, M_lo = lo).
+// X_0 = X / lam~ as `dtype` (DT_F16, DT_BF16, or DT_F16X2 with M = hi, M_lo = lo of the values times `scale`).
 cudaError_t enqueue_scale_cast(int dtype, const DevArgs* args, const DevState* st, int64_t n,
-                               void* M, void* M_lo, int64_t ldm, cudaStream_t stream);
+                               void* M, void* M_lo, int64_t ldm, cudaStream_t stream, float scale = 1.f);
 // Argument block of one replay (and the caller fields of a one-block record, if given).
 cudaError_t enqueue_set_args(DevArgs* d_args, const DevArgs& h, cudaStream_t stream, BlockRec* blk = nullptr);
 cudaError_t enqueue_set_block(BlockRec* d_blk, const BlockRec& v, cudaStream_t stream);

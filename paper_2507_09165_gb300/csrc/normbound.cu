@@ -962,15 +962,8 @@ __global__ void __launch_bounds__(kNT, 2) nb_persistent_kernel(NBCtx c, unsigned
 #undef NB_SYNC
 }
 
-// TF32 rounding (10 explicit mantissa bits, nearest, ties away from zero) of a
-// finite value; the tensor cores read only these bits of an FP32 operand.
-__device__ __forceinline__ float tf32_round(float v) {
-  if (!isfinite(v)) return v;
-  return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);
-}
-
 // Four consecutive elements (positions pos .. pos+3 of a row) of the output
-// matrix in the chain's storage: 16-bit, or TF32 hi/lo pairs.
+// matrix in the chain's storage: 16-bit, or an FP16 hi/lo pair of v * scale.
 __device__ __forceinline__ void put16(uint16_t* H, const uint16_t (&u)[4], int valid) {
   if (valid == 4) {
     *reinterpret_cast<uint2*>(H) =
@@ -981,37 +974,29 @@ __device__ __forceinline__ void put16(uint16_t* H, const uint16_t (&u)[4], int v
 }
 
 template <int DT>
-__device__ __forceinline__ void store4(void* M, void* M_lo, int64_t pos, const float (&v)[4],
-                                       int valid) {
-  if (DT == DT_TF32X3) {
-    float h[4], l[4];
+__device__ __forceinline__ void store4(void* M, void* M_lo, int64_t pos, const float (&v)[4], int valid,
+                                       float scale) {
+  uint16_t u[4];
+  if (DT == DT_F16X2) {
+    uint16_t l[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      h[k] = tf32_round(v[k]);
-      l[k] = tf32_round(v[k] - h[k]);
+      const float x = v[k] * scale;
+      const __half h = __float2half_rn(x);
+      u[k] = __half_as_ushort(h);
+      l[k] = __half_as_ushort(__float2half_rn(x - __half2float(h)));
     }
-    float* Mh = static_cast<float*>(M) + pos;
-    float* Ml = static_cast<float*>(M_lo) + pos;
-    if (valid == 4) {
-      *reinterpret_cast<float4*>(Mh) = make_float4(h[0], h[1], h[2], h[3]);
-      *reinterpret_cast<float4*>(Ml) = make_float4(l[0], l[1], l[2], l[3]);
-    } else {
-      for (int k = 0; k < valid; ++k) {
-        Mh[k] = h[k];
-        Ml[k] = l[k];
-      }
-    }
+    put16(static_cast<uint16_t*>(M_lo) + pos, l, valid);
   } else {
-    uint16_t u[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
       u[k] = DT == DT_BF16 ? __bfloat16_as_ushort(__float2bfloat16_rn(v[k])) : __half_as_ushort(__float2half_rn(v[k]));
-    put16(static_cast<uint16_t*>(M) + pos, u, valid);
   }
+  put16(static_cast<uint16_t*>(M) + pos, u, valid);
 }
 
-// X_0 = RN(X * (1/lam~)) into a full symmetric matrix (16-bit, or TF32 hi/lo
-// pairs), from the upper triangle of X, in 64 x 64 tiles through shared memory.
+// X_0 = RN(X * (1/lam~)) into a full symmetric matrix (16-bit, or a scaled FP16
+// hi/lo pair), from the upper triangle of X, in 64 x 64 tiles through shared memory.
 // Thread (tx, ty): rows i0 + 4 tx .. +3 (one 16-byte load), columns
 // j0 + ty + 16 c, c = 0..3.  Both output positions are written with
 // row-contiguous vector stores.
@@ -1019,7 +1004,7 @@ template <int DT>
 __global__ void __launch_bounds__(256) scale_cast_kernel(const DevArgs* __restrict__ args, int n,
                                                          const DevState* __restrict__ st, void* __restrict__ M,
                                                          void* __restrict__ M_lo,
-                                                         int64_t ldm) {
+                                                         int64_t ldm, float scale) {
   __shared__ float s[64][65];
   int bi, bj;
   tile_of(blockIdx.x, bi, bj);
@@ -1072,14 +1057,14 @@ __global__ void __launch_bounds__(256) scale_cast_kernel(const DevArgs* __restri
     // position (i + j ldm): memory row j, elements i0 + 4 tx .. +3
     if (j < n && valid_i > 0) {
       const float v[4] = {s[4 * tx][jj], s[4 * tx + 1][jj], s[4 * tx + 2][jj], s[4 * tx + 3][jj]};
-      store4<DT>(M, M_lo, static_cast<int64_t>(j) * ldm + ib, v, valid_i);
+      store4<DT>(M, M_lo, static_cast<int64_t>(j) * ldm + ib, v, valid_i, scale);
     }
     // mirrored position (j + i ldm): memory row i = i0 + jj, elements j0 + 4 tx .. +3
     const int i = i0 + jj, jc = j0 + 4 * tx;
     const int valid_j = min(4, n - jc);
     if (!diag && i < n && valid_j > 0) {
       const float v[4] = {s[jj][4 * tx], s[jj][4 * tx + 1], s[jj][4 * tx + 2], s[jj][4 * tx + 3]};
-      store4<DT>(M, M_lo, static_cast<int64_t>(i) * ldm + jc, v, valid_j);
+      store4<DT>(M, M_lo, static_cast<int64_t>(i) * ldm + jc, v, valid_j, scale);
     }
   }
 }
@@ -1274,15 +1259,15 @@ cudaError_t enqueue_norm_bound(const LanczosBufs& L, const DevArgs* args, DevSta
 
 
 cudaError_t enqueue_scale_cast(int dtype, const DevArgs* args, const DevState* st, int64_t n, void* M,
-                               void* M_lo, int64_t ldm, cudaStream_t s) {
+                               void* M_lo, int64_t ldm, cudaStream_t s, float scale) {
   const int nb = static_cast<int>((n + 63) / 64);
   const int tiles = nb * (nb + 1) / 2;
   const int blk = 256;
   const int ni = static_cast<int>(n);
   switch (dtype) {
-    case DT_F16: scale_cast_kernel<DT_F16><<<tiles, blk, 0, s>>>(args, ni, st, M, M_lo, ldm); break;
-    case DT_BF16: scale_cast_kernel<DT_BF16><<<tiles, blk, 0, s>>>(args, ni, st, M, M_lo, ldm); break;
-    case DT_TF32X3: scale_cast_kernel<DT_TF32X3><<<tiles, blk, 0, s>>>(args, ni, st, M, M_lo, ldm); break;
+    case DT_F16: scale_cast_kernel<DT_F16><<<tiles, blk, 0, s>>>(args, ni, st, M, M_lo, ldm, scale); break;
+    case DT_BF16: scale_cast_kernel<DT_BF16><<<tiles, blk, 0, s>>>(args, ni, st, M, M_lo, ldm, scale); break;
+    case DT_F16X2: scale_cast_kernel<DT_F16X2><<<tiles, blk, 0, s>>>(args, ni, st, M, M_lo, ldm, scale); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -86,7 +86,7 @@ int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 int64_t internal_ld(int64_t n) { return round_up(std::max<int64_t>(n, 1), 64); }
 
 // Workspace is carved into slots of one n x ldm 16-bit matrix: a 16-bit
-// matrix takes 1 slot, an FP16 pair 2, a TF32 pair 4.
+// matrix takes 1 slot, an FP16 pair (plain or scaled) 2.
 size_t slot_bytes(int64_t n) {
   return static_cast<size_t>(round_up(static_cast<int64_t>(internal_ld(n)) * n * 2, 1024));
 }
@@ -129,7 +129,7 @@ struct Plan {
   int ntiles = 0;
   int4* d_tiles_pair = nullptr;  // 256-row tiles of the CTA-pair form of the 16-bit stage products
   int ntiles_pair = 0;
-  int ncompl = 0;  // complementarity shares the final product writes (4 per one-SM tile, 8 per pair tile)
+  int ncompl = 0;  // complementarity shares the final product writes (4 per one-SM tile, 8 per pair tile, 16 on the FP32 path)
   double* d_compl = nullptr;  // 4 per tile: shares of <out, X - out> from the final product
   cudaGraphExec_t exec = nullptr;
   bool graph_tried = false;
@@ -182,7 +182,7 @@ psd_status_t build_plan(Plan* p, void* user_ws, size_t user_bytes) {
   std::vector<int4> tiles_pair = make_tile_list_pair(n);
   p->ntiles_pair = static_cast<int>(tiles_pair.size());
   const size_t o_compl = o_tiles + round_up(sizeof(int4) * std::max<size_t>(tiles.size(), 1), 256);
-  const size_t ncompl_max = std::max<size_t>(std::max(4 * tiles.size(), 8 * tiles_pair.size()), 1);
+  const size_t ncompl_max = std::max<size_t>(std::max(4 * tiles.size(), 16 * tiles_pair.size()), 1);
   const size_t o_pair = o_compl + round_up(sizeof(double) * ncompl_max, 256);
   const size_t small = o_pair + sizeof(int4) * std::max<size_t>(tiles_pair.size(), 1);
   uint8_t* sm = nullptr;
@@ -213,7 +213,7 @@ psd_status_t build_plan(Plan* p, void* user_ws, size_t user_bytes) {
 }
 
 void* part_ptr(const Plan* p, const Mat& m, int part) {
-  return p->slots + (static_cast<size_t>(m.slot) + static_cast<size_t>(part * kind_lo_step(m.kind))) * p->slot_size;
+  return p->slots + (static_cast<size_t>(m.slot) + static_cast<size_t>(part)) * p->slot_size;
 }
 
 GemmParams base_params(const Plan* p) {
@@ -278,17 +278,27 @@ cudaError_t gemm(Plan* p, int epi, const Mat& A, const Mat& B, const Mat* out, c
     g.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | (8u << 24);  // M = 128; N per tile
     return launch_symgemm(dt, epi, ta, tb, g, grid, s, out ? kind_dtype(*out) : -1);
   }
-  if (route == ROUTE_NONE) return cudaErrorNotSupported;
+  if (route == ROUTE_NONE || (epi == EPI_FINAL && (route == ROUTE_X3 || route == ROUTE_X2)))
+    return cudaErrorNotSupported;
+  if (route == ROUTE_F32) {
+    const Mat* ops[2] = {&A, &B};
+    CUtensorMap tm[4];
+    for (int i = 0; i < 4; ++i)
+      if (!encode_tmap(&tm[i], DT_F16X2, part_ptr(p, *ops[i >> 1], i & 1), n, ldm, 128, 64)) return cudaErrorInvalidValue;
+    g.num_tiles = p->ntiles_pair;
+    g.tiles = p->d_tiles_pair;
+    if (epi == EPI_FINAL) p->ncompl = 16 * p->ntiles_pair;
+    return launch_symgemm_f32(epi, tm, g, grid, s);
+  }
   const bool b1 = route == ROUTE_X2;
   const Mat& PA = b1 ? B : A;  // the pair operand goes first
   const Mat& PB = b1 ? A : B;
   const int dt = kind_dtype(PA);
   CUtensorMap tm[4];
   const int rb = x3_row_bytes(b1);
-  const int out_mode = epi == EPI_FINAL ? 2 : (kind_is_pair(out->kind) ? 0 : 1);
+  const int out_mode = kind_is_pair(out->kind) ? 0 : 1;  // the final product of these chains is a 16-bit one
   // FP16-pair stage products on CTA pairs (M = 256, half of B in each CTA)
-  const bool pair = dt == DT_F16X2 && epi != EPI_FINAL &&
-                    (b1 ? (epi == EPI_SCALE && out_mode == 1) : out_mode == 0);
+  const bool pair = b1 ? (epi == EPI_SCALE && out_mode == 1) : out_mode == 0;
   const int brows = pair ? 128 : 256;
   if (!encode_tmap(&tm[0], dt, part_ptr(p, PA, 0), n, ldm, 128, rb) ||
       !encode_tmap(&tm[1], dt, part_ptr(p, PA, 1), n, ldm, 128, rb) ||
@@ -307,7 +317,7 @@ struct PlanOps {
   cudaStream_t s;
   cudaError_t cast(const Mat& X0) {
     return enqueue_scale_cast(kind_dtype(X0), p->d_args, p->d_state, p->n, part_ptr(p, X0, 0),
-                              kind_is_pair(X0.kind) ? part_ptr(p, X0, 1) : nullptr, p->ldm, s);
+                              kind_is_pair(X0.kind) ? part_ptr(p, X0, 1) : nullptr, p->ldm, s, X0.scale);
   }
   cudaError_t gemm(int epi, const Mat& A, const Mat& B, const Mat* out, const Mat* Y, float a, float b, float c,
                    float sc, bool track) {

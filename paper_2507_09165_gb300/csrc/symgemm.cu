@@ -27,6 +27,7 @@
 #include <cstdio>
 #include <mutex>
 
+#include "epilogue.cuh"
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -51,7 +52,6 @@ constexpr int kStageBytes16 = kABytes16 + kBBytes16;  // 48 KB
 // transposed (ST) and the prefetched Y chunk (YB), each 32 x 40 halves (80-byte
 // rows keep 16-byte accesses aligned and spread over the banks).  FP32 output:
 // 32 x 33 words, in the same space.
-constexpr int kStgWords = 33;
 constexpr int kH = 40;
 constexpr int kEpiWarpBytes = 3 * 32 * kH * 2;  // 7680 >= 32 * 33 * 4
 
@@ -80,10 +80,6 @@ __device__ __forceinline__ float from16(uint16_t u, bool bf16) {
 
 __device__ __forceinline__ uint16_t to8(float v) {
   return static_cast<uint16_t>(__nv_cvt_float_to_fp8(v, __NV_SATFINITE, __NV_E4M3));
-}
-
-__device__ __forceinline__ void raise_status(int* status, int code) {
-  if (status) atomicCAS(status, 0, code);
 }
 
 // Y chunk (r0..r0+31) x (c0..c0+31) of a symmetric 16-bit matrix, read as
@@ -297,59 +293,6 @@ __device__ __forceinline__ void epilogue_chunk16(const GemmParams& p, const Bloc
 #pragma unroll
     for (int j = 0; j < 32; ++j)
       if (c0 + j < n) amax_bits = max(amax_bits, __float_as_uint(fabsf(from16(static_cast<uint16_t>(h[j]), bf16))));
-  }
-}
-
-// One 32 x 32 chunk of the final output out = (X + lam~ acc) / 2 in FP32,
-// reading only the upper triangle of the caller's X (column-major).
-__device__ __forceinline__ void epilogue_chunk_final(const BlockRec& br, int r0, int c0,
-                                                     const uint32_t (&v)[32], uint8_t* wbuf,
-                                                     int lane, float lam, ComplAcc* ca) {
-  uint32_t* stg = reinterpret_cast<uint32_t*>(wbuf);
-  const int n = br.n;
-  const float* X = br.X;
-  const int64_t ld = br.ld;
-  float* out = br.out;
-  const int64_t ldo = br.ld_out;
-  const int r = r0 + lane;
-  const bool diag = (r0 == c0);
-  const bool row_ok = r < n;
-  float o[32];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const int c = c0 + j;
-    float x = 0.f;
-    const bool upper = !diag || j >= lane;
-    if (row_ok && c < n && upper) x = X[static_cast<int64_t>(c) * ld + r];
-    o[j] = 0.5f * fmaf(lam, __uint_as_float(v[j]), x);
-    if (ca && row_ok && c < n && upper) compl_add(*ca, o[j], x, c == r ? 1.f : 2.f);
-  }
-  float* sf = reinterpret_cast<float*>(stg);
-  if (diag) {
-#pragma unroll
-    for (int j = 0; j < 32; ++j) sf[lane * kStgWords + j] = o[j];
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < 32; ++j)
-      if (j < lane) o[j] = sf[j * kStgWords + lane];
-    __syncwarp();
-  }
-  if (row_ok) {
-#pragma unroll
-    for (int j = 0; j < 32; ++j)
-      if (c0 + j < n) out[static_cast<int64_t>(c0 + j) * ldo + r] = o[j];
-  }
-  if (!diag) {
-#pragma unroll
-    for (int j = 0; j < 32; ++j) sf[lane * kStgWords + j] = o[j];
-    __syncwarp();
-    const int c = c0 + lane;
-    if (c < n) {
-#pragma unroll 4
-      for (int rr = 0; rr < 32; ++rr)
-        if (r0 + rr < n) out[static_cast<int64_t>(r0 + rr) * ldo + c] = sf[rr * kStgWords + lane];
-    }
-    __syncwarp();
   }
 }
 
