@@ -391,7 +391,7 @@ struct LanczosBufs {
 size_t lanczos_bytes(int64_t n);
 void lanczos_carve(LanczosBufs& b, int64_t n, uint8_t* base);
 // persistent: the whole bound as one cooperative persistent kernel (grid
-// barriers between the phases); otherwise 151 launches (kNormBoundLaunches)
+// barriers between the phases); otherwise kNormBoundLaunches launches
 // that can share the GPU with other work -- the request server's preparation
 // streams run beside product kernels that leave no room for a co-resident
 // grid.  Both paths give identical results.
@@ -431,8 +431,8 @@ __device__ __forceinline__ void finalize_report(DevState* st, psd_info_t* info) 
 }
 
 // Kernel launches of one multi-launch enqueue_norm_bound: start vector (2),
-// the Lanczos steps (6 each, plus the Frobenius norm in the first), the
+// the Lanczos steps (5 each, plus the Frobenius norm in the first), the
 // tridiagonal solve, Ritz vector and residual (8).
-constexpr int kNormBoundLaunches = 2 + 6 * kMaxSteps + 1 + 8;
+constexpr int kNormBoundLaunches = 2 + 5 * kMaxSteps + 1 + 8;
 
 }  // namespace psd

@@ -26,6 +26,9 @@
 
 #include <algorithm>
 #include <cmath>
+#include <map>
+#include <mutex>
+#include <type_traits>
 
 #include "internal.h"
 #include "ptx.cuh"
@@ -213,15 +216,26 @@ __device__ __forceinline__ TileGeom tile_geom(int t) {
   return g;
 }
 
-// The thread's slices of v (rows and columns) and its 64 elements: 16
-// independent 16-byte loads of X in flight.
-__device__ __forceinline__ void tile_load(const float* __restrict__ X, int64_t ld, int n, const TileGeom& g,
-                                          const float* vh, float (&vi)[8], float (&vj)[8], float (&x)[8][8]) {
+// The thread's 8-element slices of v: rows (vi) and columns (vj); zeros past n.
+// vh holds npad (a multiple of 256) floats and the slices start at multiples of 8.
+__device__ __forceinline__ void tile_load_v(int n, const TileGeom& g, const float* vh, float (&vi)[8],
+                                            float (&vj)[8]) {
+  const float4 a0 = __ldcg(reinterpret_cast<const float4*>(vh + g.ib));
+  const float4 a1 = __ldcg(reinterpret_cast<const float4*>(vh + g.ib) + 1);
+  const float4 b0 = __ldcg(reinterpret_cast<const float4*>(vh + g.jb));
+  const float4 b1 = __ldcg(reinterpret_cast<const float4*>(vh + g.jb) + 1);
+  const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+  const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    vi[k] = (g.ib + k < n) ? __ldcg(vh + g.ib + k) : 0.f;
-    vj[k] = (g.jb + k < n) ? __ldcg(vh + g.jb + k) : 0.f;
+    vi[k] = g.ib + k < n ? a[k] : 0.f;
+    vj[k] = g.jb + k < n ? b[k] : 0.f;
   }
+}
+
+// The thread's 64 elements: 16 independent 16-byte loads of X in flight.
+__device__ __forceinline__ void tile_load_x(const float* __restrict__ X, int64_t ld, int n, const TileGeom& g,
+                                            float (&x)[8][8]) {
   const bool full = (g.ib + 7 < n) && (g.jb + 7 < n);
   const bool vec = full && ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
 #pragma unroll
@@ -240,9 +254,10 @@ __device__ __forceinline__ void tile_load(const float* __restrict__ X, int64_t l
 }
 
 // Per-thread row and column dot products of the 8 x 8 block (8-term FP32 FMA runs).
-template <bool STATS, bool DIAG>
+// `col(c, x)` gives column c of the block.
+template <bool STATS, bool DIAG, class Col>
 __device__ __forceinline__ void tile_fma(int n, const TileGeom& g, const float (&vi)[8], const float (&vj)[8],
-                                         const float (&x)[8][8], float (&rsum)[8], float (&csum)[8], float& fro,
+                                         const Col& col, float (&rsum)[8], float (&csum)[8], float& fro,
                                          unsigned& mdiag) {
   fro = 0.f;
   mdiag = 0;
@@ -250,21 +265,38 @@ __device__ __forceinline__ void tile_fma(int n, const TileGeom& g, const float (
   for (int k = 0; k < 8; ++k) rsum[k] = 0.f;
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
+    float x[8];
+    col(c, x);
     csum[c] = 0.f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      float xr = x[c][k], xc = x[c][k];
+      float xr = x[k], xc = x[k];
       if (DIAG) {
         const int i = g.ib + k, j = g.jb + c;
         xr = (i <= j) ? xr : 0.f;
         xc = (i < j) ? xc : 0.f;
-        if (STATS && i == j && i < n) mdiag = max(mdiag, __float_as_uint(fabsf(x[c][k])));
+        if (STATS && i == j && i < n) mdiag = max(mdiag, __float_as_uint(fabsf(x[k])));
       }
       rsum[k] = fmaf(xr, vj[c], rsum[k]);
       csum[c] = fmaf(xc, vi[k], csum[c]);
       if (STATS) fro = fmaf(xr, xc + xr, fro);  // x^2 on the diagonal, 2 x^2 above it
     }
   }
+}
+
+// tile_fma of a tile held in registers.
+template <bool STATS>
+__device__ __forceinline__ void tile_fma_reg(int n, const TileGeom& g, const float (&vi)[8], const float (&vj)[8],
+                                             const float (&x)[8][8], float (&rsum)[8], float (&csum)[8], float& fro,
+                                             unsigned& mdiag) {
+  auto col = [&](int c, float (&o)[8]) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) o[k] = x[c][k];
+  };
+  if (g.diag)
+    tile_fma<STATS, true>(n, g, vi, vj, col, rsum, csum, fro, mdiag);
+  else
+    tile_fma<STATS, false>(n, g, vi, vj, col, rsum, csum, fro, mdiag);
 }
 
 // Combines the threads' sums in a fixed order (double-float) into the tile's
@@ -346,11 +378,9 @@ __device__ __forceinline__ void ph_symv(const NBCtx& c, const float* X, int64_t 
   const TileGeom g = tile_geom(t);
   float vi[8], vj[8], x[8][8], rsum[8], csum[8], fro;
   unsigned mdiag;
-  tile_load(X, ld, c.n, g, c.vh, vi, vj, x);
-  if (g.diag)
-    tile_fma<STATS, true>(c.n, g, vi, vj, x, rsum, csum, fro, mdiag);
-  else
-    tile_fma<STATS, false>(c.n, g, vi, vj, x, rsum, csum, fro, mdiag);
+  tile_load_v(c.n, g, c.vh, vi, vj);
+  tile_load_x(X, ld, c.n, g, x);
+  tile_fma_reg<STATS>(c.n, g, vi, vj, x, rsum, csum, fro, mdiag);
   tile_reduce_store<STATS>(c.n, g, rsum, csum, fro, mdiag, c.P1, c.P2, c.npad, c.tile_fro, c.st, sh, t);
 }
 
@@ -367,17 +397,18 @@ __device__ __forceinline__ void ph_symv_run(const NBCtx& c, const float* X, int6
   int r = first;
   int buf = 0;
   TileGeom g = tile_geom(tile_at(r));
-  tile_load(X, ld, c.n, g, c.vh, vi, vj, x);
+  tile_load_v(c.n, g, c.vh, vi, vj);
+  tile_load_x(X, ld, c.n, g, x);
   while (true) {
     float rsum[8], csum[8], fro;
     unsigned mdiag;
-    if (g.diag)
-      tile_fma<STATS, true>(c.n, g, vi, vj, x, rsum, csum, fro, mdiag);
-    else
-      tile_fma<STATS, false>(c.n, g, vi, vj, x, rsum, csum, fro, mdiag);
+    tile_fma_reg<STATS>(c.n, g, vi, vj, x, rsum, csum, fro, mdiag);
     const int rn = r + stride;
     const TileGeom gn = tile_geom(tile_at(rn < c.ntiles ? rn : r));
-    if (rn < c.ntiles) tile_load(X, ld, c.n, gn, c.vh, vi, vj, x);  // in flight during the reduction
+    if (rn < c.ntiles) {  // in flight during the reduction
+      tile_load_v(c.n, gn, c.vh, vi, vj);
+      tile_load_x(X, ld, c.n, gn, x);
+    }
     tile_reduce_store<STATS>(c.n, g, rsum, csum, fro, mdiag, c.P1, c.P2, c.npad, c.tile_fro, c.st, sh,
                              tile_at(r), buf, false);
     if (rn >= c.ntiles) break;
@@ -385,6 +416,35 @@ __device__ __forceinline__ void ph_symv_run(const NBCtx& c, const float* X, int6
     g = gn;
     buf ^= 1;
   }
+}
+
+// The product over a CTA's resident tiles: tile b0 in registers (x), tile b0 +
+// stride (if any) in shared memory, each thread's own 16 float4 of it at
+// xs[256 q + thread] (read and written by that thread only).
+template <bool STATS>
+__device__ __forceinline__ void ph_symv_resident(const NBCtx& c, int b0, int stride, const float (&x)[8][8],
+                                                 const float4* xs, NBShared& sh) {
+  if (b0 >= c.ntiles) return;
+  float vi[8], vj[8], rsum[8], csum[8], fro;
+  unsigned mdiag;
+  const TileGeom g = tile_geom(b0);
+  tile_load_v(c.n, g, c.vh, vi, vj);
+  tile_fma_reg<STATS>(c.n, g, vi, vj, x, rsum, csum, fro, mdiag);
+  const int t1 = b0 + stride;
+  const TileGeom g1 = tile_geom(t1 < c.ntiles ? t1 : b0);
+  if (t1 < c.ntiles) tile_load_v(c.n, g1, c.vh, vi, vj);
+  tile_reduce_store<STATS>(c.n, g, rsum, csum, fro, mdiag, c.P1, c.P2, c.npad, c.tile_fro, c.st, sh, b0, 0, false);
+  if (t1 >= c.ntiles) return;
+  auto col = [&](int k, float (&o)[8]) {
+    const float4 a = xs[kNT * (2 * k) + threadIdx.x], b = xs[kNT * (2 * k + 1) + threadIdx.x];
+    o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
+    o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
+  };
+  if (g1.diag)
+    tile_fma<STATS, true>(c.n, g1, vi, vj, col, rsum, csum, fro, mdiag);
+  else
+    tile_fma<STATS, false>(c.n, g1, vi, vj, col, rsum, csum, fro, mdiag);
+  tile_reduce_store<STATS>(c.n, g1, rsum, csum, fro, mdiag, c.P1, c.P2, c.npad, c.tile_fro, c.st, sh, t1, 1, false);
 }
 
 // State reset and the start vector q_0 (unit SplitMix64 vector, before scaling).
@@ -459,12 +519,12 @@ __device__ __forceinline__ double reduce_partials(const NBCtx& c, int ch, NBShar
   F2 a{0.f, 0.f}, d{0.f, 0.f};
   if (e < c.n) {
     const int b = e / kSymvTile;
-#pragma unroll 4
+#pragma unroll 8
     for (int bj = b + hw; bj < c.nb; bj += 4) {
       const float2 t = __ldcg(c.P1 + static_cast<int64_t>(bj) * c.npad + e);
       a = f2_add(a, F2{t.x, t.y});
     }
-#pragma unroll 4
+#pragma unroll 8
     for (int bi = hw; bi <= b; bi += 4) {
       const float2 t = __ldcg(c.P2 + static_cast<int64_t>(bi) * c.npad + e);
       d = f2_add(d, F2{t.x, t.y});
@@ -484,28 +544,80 @@ __device__ __forceinline__ double reduce_partials(const NBCtx& c, int ch, NBShar
   return y;
 }
 
-// u = X v (first product of X (X v)); split u for the second product.  Chunk pair cp.
-__device__ __forceinline__ void ph_reduce_split(const NBCtx& c, int cp, double* u, NBShared& sh) {
-  const int ch = chunk_of_half(cp);
-  const double y = reduce_partials(c, ch, sh);
-  const int e = ch * 32 + (threadIdx.x & 31);
-  if (half_lead_warp() && e < c.n) {
-    u[e] = y;
-    split_d(y, c.vh[e], c.vl[e]);
-  }
-}
-
-// ---- Lanczos step j after the second product: Gram-Schmidt and q_{j+1}.
-// Element work is done per chunk of 32 elements by one warp (lane =
-// element), FP64.  Sums over the chunks (the dot products q_k . w and ||w||^2)
-// go through per-chunk partials stored as double-float pairs (FP32 hi + lo,
-// about 48 bits): every CTA adds them up itself in FP32 arithmetic, in the same
-// order, because this GPU issues FP64 at a small fraction of its FP32 rate.
-
 __device__ __forceinline__ float2 d_to_f2(double v) {
   const float h = __double2float_rn(v);
   return make_float2(h, __double2float_rn(v - static_cast<double>(h)));
 }
+
+// Warp sum of one FP64 value per lane as a double-float pair (fixed order;
+// every lane): FP32 shuffles and adds, this GPU's FP64 adds being far slower.
+__device__ __forceinline__ F2 warp_sum_f2(double v) {
+  const int lane = threadIdx.x & 31;
+  const float2 p = d_to_f2(v);
+  F2 t{p.x, p.y};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const F2 other = shfl_xor_f2(t, o);
+    t = (lane & o) ? f2_add(other, t) : f2_add(t, other);
+  }
+  return t;
+}
+
+// Sum of nch double-float partials by one warp (lanes stride over them, 8 loads
+// in flight, then a butterfly; fixed order), as FP64 in every lane.
+__device__ __forceinline__ double warp_sum_chunks(const float2* part, int nch) {
+  const int lane = threadIdx.x & 31;
+  F2 acc{0.f, 0.f};
+  for (int c0 = 0; c0 < nch; c0 += 8 * 32) {
+    float2 t[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int ch = c0 + 32 * i + lane;
+      t[i] = ch < nch ? __ldcg(part + ch) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc = f2_add(acc, F2{t[i].x, t[i].y});
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const F2 other = shfl_xor_f2(acc, o);
+    acc = (lane & o) ? f2_add(other, acc) : f2_add(acc, other);
+  }
+  return f2_to_d(acc);
+}
+
+// u = X v (first product of X (X v)); split u for the second product; the
+// chunk's share of ||u||^2 (= alpha_j, q_j being a unit vector).  Chunk pair cp.
+__device__ __forceinline__ void ph_reduce_split(const NBCtx& c, int cp, double* u, NBShared& sh) {
+  const int ch = chunk_of_half(cp);
+  const double y = reduce_partials(c, ch, sh);
+  if (!half_lead_warp() || ch >= c.npart) return;
+  const int e = ch * 32 + (threadIdx.x & 31);
+  if (e < c.n) {
+    u[e] = y;
+    split_d(y, c.vh[e], c.vl[e]);
+  }
+  const F2 t = warp_sum_f2(e < c.n ? y * y : 0.0);
+  if ((threadIdx.x & 31) == 0) c.norms2[ch] = make_float2(t.h, t.l);
+}
+
+// ---- Lanczos step j after the second product: w = X u, the three-term
+// recurrence, one full Gram-Schmidt pass and q_{j+1}.
+//
+// alpha_j = q_j . X u = ||u||^2 is known from the first product, so the
+// recurrence w' = w - alpha_j q_j - beta_{j-1} q_{j-1} is applied as soon as w
+// is reduced.  In exact arithmetic w' is orthogonal to every Lanczos vector; in
+// this one its components along them are at the mat-vec's rounding level, and a
+// single Gram-Schmidt pass over all of them takes those out down to the FP64
+// rounding of w' (two passes are only needed where the first cancels most of
+// the vector).  The pass's coefficient along q_j is added to alpha_j.  Two
+// passes on w itself took a phase and a grid barrier more per step.
+//
+// Element work is done per chunk of 32 elements by one warp (lane =
+// element), FP64.  Sums over the chunks (the dot products q_k . w' and ||w'||^2)
+// go through per-chunk partials stored as double-float pairs (FP32 hi + lo,
+// about 48 bits): every CTA adds them up itself in FP32 arithmetic, in the same
+// order, because this GPU issues FP64 at a small fraction of its FP32 rate.
 
 // S[k] = sum over the chunks of part[k * nch + ch] (slot-major: a warp's 32
 // lanes read 256 contiguous bytes) for the slots k with (want >> k) & 1,
@@ -536,100 +648,104 @@ __device__ __forceinline__ void chunk_sums(const float2* part, int nch, uint32_t
   }
 }
 
-// w = X u (the second product, reduced); partial dots q_k . w (k <= j) of the
-// chunk into slot k of dots.  Chunk pair cp.
+// w' = w - alpha_j q_j - beta_{j-1} q_{j-1}; the chunk's shares of q_k . w'
+// (k <= j) and ||w'||^2 (slot 31) into dots.  Chunk pair cp.
 __device__ __forceinline__ void ph_reduce_dots(const NBCtx& c, int cp, int j, NBShared& sh) {
   const int ch = chunk_of_half(cp);
-  const double y = reduce_partials(c, ch, sh);
-  if (!half_lead_warp() || ch >= c.npart) return;
   const int lane = threadIdx.x & 31;
   const int e = ch * 32 + lane;
+  const bool lead = half_lead_warp() && ch < c.npart;
+  // alpha_j by a warp of the other half of the CTA's work; loads before the partial sums'
+  if (threadIdx.x >= 32 && threadIdx.x < 64) {
+    const double a = warp_sum_chunks(c.norms2, c.npart);
+    if (lane == 0) sh.scalar[0] = a;
+  }
+  double qk[kMaxSteps];
+  double beta = 0.0;
+#pragma unroll
+  for (int k = 0; k < kMaxSteps; ++k)
+    qk[k] = (lead && k <= j && e < c.n) ? __ldcg(c.Qv + static_cast<int64_t>(k) * c.npad + e) : 0.0;
+  if (lead && j > 0) beta = __ldcg(&c.st->beta[j - 1]);
+  double y = reduce_partials(c, ch, sh);  // its barriers publish sh.scalar[0]
+  const double alpha = sh.scalar[0];
+  if (cp == 0 && threadIdx.x == 0) c.st->alpha[j] = alpha;
+  if (!lead) return;
+  double qj = 0.0, qp = 0.0;
+#pragma unroll
+  for (int k = 0; k < kMaxSteps; ++k) {
+    if (k == j) qj = qk[k];
+    if (k == j - 1) qp = qk[k];
+  }
+  y = (y - alpha * qj) - beta * qp;
   if (e < c.n) c.w[e] = y;
   double v[32];
 #pragma unroll
-  for (int k = 0; k < 32; ++k)
-    v[k] = (k <= j && e < c.n) ? __ldcg(c.Qv + static_cast<int64_t>(k) * c.npad + e) * y : 0.0;
+  for (int k = 0; k < 32; ++k) v[k] = k < kMaxSteps ? qk[k < kMaxSteps ? k : 0] * y : 0.0;
+  v[31] = e < c.n ? y * y : 0.0;
   c.dots[static_cast<int64_t>(lane) * c.npart + ch] = d_to_f2(warp_multi_sum(v, lane));
 }
 
-// First Gram-Schmidt pass (every CTA first sums the chunks' dots: h, and
-// alpha_j = h_j), then per chunk: w -= sum_k h_k q_k, and the partials of the
-// second pass, q_k . w (k <= j) and ||w||^2 (slot 31), into dots2.
-// Chunks ch = cta + ncta * warp, ... (warp 0 only while there are no more
-// chunks than CTAs: the FP64 work spreads over the SMs).
-__device__ __forceinline__ void ph_orth1(const NBCtx& c, int cta, int ncta, int j, NBShared& sh) {
-  chunk_sums(c.dots, c.npart, (2u << j) - 1u, sh.u.orth.h);
-  __syncthreads();
-  if (cta == 0 && threadIdx.x == 0) c.st->alpha[j] = sh.u.orth.h[j];
+// The Gram-Schmidt pass and the next Lanczos vector.  Every CTA sums the
+// chunks' dots h and ||w'||^2; w'' = w' - Q h is orthogonal to Q and (Q
+// orthonormal) ||w''||^2 = ||w'||^2 - ||h||^2, so beta_j = ||w''|| needs no
+// further reduction (h is at the mat-vec's rounding level: no cancellation
+// until w' itself is down there).  Stops on breakdown (beta_j <= 1e-12
+// ||X||_F^2) or after the last step; otherwise q_{j+1} = w'' / beta_j per chunk.
+// The chunks' warps form w'' (four independent chains: an FP64 operation's
+// latency is 64 cycles) while the last warp forms beta_j.  Returns `stop` (the
+// same in every CTA).
+__device__ __forceinline__ bool ph_orth_next(const NBCtx& c, int cta, int ncta, int j, NBShared& sh) {
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  for (int ch = cta + ncta * wp; ch < c.npart; ch += ncta * (kNT / 32)) {
+  constexpr int kW = kNT / 32;
+  const double fro = __ldcg(&c.st->fro);
+  chunk_sums(c.dots, c.npart, ((2u << j) - 1u) | 0x80000000u, sh.u.orth.h);
+  __syncthreads();
+  if (wp == kW - 1) {
+    double h2 = lane <= j ? sh.u.orth.h[lane] * sh.u.orth.h[lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) h2 += __shfl_xor_sync(0xffffffffu, h2, o);
+    if (lane == 0) {
+      const double b2 = sh.u.orth.h[31] - h2;
+      const double r = rsqrt(b2);
+      sh.scalar[0] = b2 > 0.0 ? b2 * r : (b2 <= 0.0 ? 0.0 : b2);  // NaN stays NaN
+      sh.scalar[1] = r;
+    }
+  }
+  auto next = [&](int ch) {  // w'' of the lane's element
     const int e = ch * 32 + lane;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
     double qk[kMaxSteps];
 #pragma unroll
     for (int k = 0; k < kMaxSteps; ++k)
       qk[k] = (k <= j && e < c.n) ? __ldcg(c.Qv + static_cast<int64_t>(k) * c.npad + e) : 0.0;
-    double we = 0.0;
-    if (e < c.n) {
-      we = __ldcg(c.w + e);
+    const double we = e < c.n ? __ldcg(c.w + e) : 0.0;
 #pragma unroll
-      for (int k = 0; k < kMaxSteps; ++k)
-        if (k <= j) we -= sh.u.orth.h[k] * qk[k];
-      c.w[e] = we;
-    }
-    double v[32];
-#pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = (k < kMaxSteps && k <= j) ? qk[k < kMaxSteps ? k : 0] * we : 0.0;
-    v[31] = we * we;
-    c.dots2[static_cast<int64_t>(lane) * c.npart + ch] = d_to_f2(warp_multi_sum(v, lane));
-  }
+    for (int k = 0; k < kMaxSteps; ++k)
+      if (k <= j) a[k & 3] += sh.u.orth.h[k] * qk[k];
+    return we - ((a[0] + a[1]) + (a[2] + a[3]));
+  };
+  const int ch0 = cta + ncta * wp;  // most CTAs have one chunk, on warp 0
+  const double w0 = ch0 < c.npart ? next(ch0) : 0.0;
   __syncthreads();
-}
-
-// Second Gram-Schmidt pass and the next Lanczos vector.  Every CTA sums the
-// second pass's dots h2 and ||w||^2; w' = w - Q h2 is orthogonal to Q and
-// (Q orthonormal) ||w'||^2 = ||w||^2 - ||h2||^2, so beta_j = ||w'|| needs no
-// further reduction (h2 is at the rounding level of w after the first pass:
-// no cancellation).  Stops on breakdown (beta_j <= 1e-12 ||X||_F^2) or after
-// the last step; otherwise q_{j+1} = w' / beta_j per chunk.  Returns `stop`
-// (the same in every CTA) and beta_j.
-__device__ __forceinline__ bool ph_orth2_next(const NBCtx& c, int cta, int ncta, int j, NBShared& sh,
-                                              double& beta) {
-  chunk_sums(c.dots2, c.npart, ((2u << j) - 1u) | 0x80000000u, sh.u.orth.h);
-  __syncthreads();
-  if (threadIdx.x == 0) {  // FP64 scalar work once per CTA
-    double h2 = 0.0;
-    for (int k = 0; k <= j; ++k) h2 += sh.u.orth.h[k] * sh.u.orth.h[k];
-    const double b = sqrt(fmax(sh.u.orth.h[31] - h2, 0.0));
-    sh.scalar[0] = b;
-    sh.scalar[1] = 1.0 / b;
-  }
-  __syncthreads();
-  beta = sh.scalar[0];
-  const double fro = __ldcg(&c.st->fro);
+  const double beta = sh.scalar[0];
   const bool stop = !(beta > kBreakdown * (fro * fro)) || j == kMaxSteps - 1;  // also true for NaN
   if (cta == 0 && threadIdx.x == 0) {
+    c.st->alpha[j] = __ldcg(&c.st->alpha[j]) + sh.u.orth.h[j];
     c.st->beta[j] = beta;
     c.st->m = j + 1;
     if (stop) c.st->done = 1;
   }
   if (!stop) {
     const double inv = sh.scalar[1];
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    for (int ch = cta + ncta * wp; ch < c.npart; ch += ncta * (kNT / 32)) {
+    auto put = [&](int ch, double w) {
       const int e = ch * 32 + lane;
-      if (e >= c.n) continue;
-      double qk[kMaxSteps];
-#pragma unroll
-      for (int k = 0; k < kMaxSteps; ++k)
-        qk[k] = k <= j ? __ldcg(c.Qv + static_cast<int64_t>(k) * c.npad + e) : 0.0;
-      double we = __ldcg(c.w + e);
-#pragma unroll
-      for (int k = 0; k < kMaxSteps; ++k)
-        if (k <= j) we -= sh.u.orth.h[k] * qk[k];
-      const double q = we * inv;
+      if (e >= c.n) return;
+      const double q = w * inv;
       c.Qv[static_cast<int64_t>(j + 1) * c.npad + e] = q;
       split_d(q, c.vh[e], c.vl[e]);
-    }
+    };
+    if (ch0 < c.npart) put(ch0, w0);
+    for (int ch = ch0 + ncta * kW; ch < c.npart; ch += ncta * kW) put(ch, next(ch));
   }
   __syncthreads();
   return stop;
@@ -669,13 +785,7 @@ __device__ __forceinline__ void ph_ritz(const NBCtx& c, int cta, int ncta, NBSha
         if (k < m) s += yk[k] * qk[k];
       c.q[e] = s;
     }
-    F2 t = {__double2float_rn(s * s), 0.f};
-    t.l = __double2float_rn(s * s - static_cast<double>(t.h));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const F2 other = shfl_xor_f2(t, o);
-      t = (lane & o) ? f2_add(other, t) : f2_add(t, other);
-    }
+    const F2 t = warp_sum_f2(s * s);
     if (lane == 0) c.norms2[ch] = make_float2(t.h, t.l);
   }
 }
@@ -684,27 +794,8 @@ __device__ __forceinline__ void ph_ritz(const NBCtx& c, int cta, int ncta, NBSha
 // (fixed order; 0 for a zero sum); every thread of the CTA receives it.
 __device__ __forceinline__ double inv_norm_of_sum(const NBCtx& c, NBShared& sh) {
   if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    F2 acc{0.f, 0.f};
-    for (int c0 = 0; c0 < c.npart; c0 += 8 * 32) {
-      float2 t[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int ch = c0 + 32 * i + lane;
-        t[i] = ch < c.npart ? __ldcg(c.norms2 + ch) : make_float2(0.f, 0.f);
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) acc = f2_add(acc, F2{t[i].x, t[i].y});
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const F2 other = shfl_xor_f2(acc, o);
-      acc = (lane & o) ? f2_add(other, acc) : f2_add(acc, other);
-    }
-    if (lane == 0) {
-      const double s2 = f2_to_d(acc);
-      sh.scalar[0] = s2 > 0.0 ? 1.0 / sqrt(s2) : 0.0;
-    }
+    const double s2 = warp_sum_chunks(c.norms2, c.npart);
+    if (threadIdx.x == 0) sh.scalar[0] = s2 > 0.0 ? 1.0 / sqrt(s2) : 0.0;
   }
   __syncthreads();
   const double r = sh.scalar[0];
@@ -731,27 +822,13 @@ __device__ __forceinline__ void ph_resid(const NBCtx& c, int cp, NBShared& sh) {
   const int e = ch * 32 + lane;
   double r = 0.0;
   if (e < c.n) r = y - __ldcg(&c.st->sigma) * __ldcg(c.q + e);
-  F2 t = {__double2float_rn(r * r), 0.f};
-  t.l = __double2float_rn(r * r - static_cast<double>(t.h));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const F2 other = shfl_xor_f2(t, o);
-    t = (lane & o) ? f2_add(other, t) : f2_add(t, other);
-  }
+  const F2 t = warp_sum_f2(r * r);
   if (lane == 0) c.norms2[ch] = make_float2(t.h, t.l);
 }
 
 // lam~ = max(sqrt(sigma + r), ||X||_F / sqrt n, max |X_ii|); report.  One warp.
 __device__ __forceinline__ void ph_final(const NBCtx& c) {
-  const int lane = threadIdx.x;
-  F2 acc{0.f, 0.f};
-  for (int ch = lane; ch < c.npart; ch += 32) acc = f2_add(acc, F2{__ldcg(c.norms2 + ch).x, __ldcg(c.norms2 + ch).y});
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const F2 other = shfl_xor_f2(acc, o);
-    acc = (lane & o) ? f2_add(other, acc) : f2_add(acc, other);
-  }
-  const double r2 = f2_to_d(acc);
+  const double r2 = warp_sum_chunks(c.norms2, c.npart);
   if (threadIdx.x != 0) return;
   DevState* st = c.st;
   const double r = sqrt(r2);
@@ -818,16 +895,10 @@ __global__ void __launch_bounds__(kNT) nb_reduce_dots_kernel(NBCtx c, int j) {
   __shared__ NBShared sh;
   ph_reduce_dots(c, blockIdx.x, j, sh);
 }
-__global__ void __launch_bounds__(kNT) nb_orth1_kernel(NBCtx c, int j) {
+__global__ void __launch_bounds__(kNT) nb_orth_kernel(NBCtx c, int j) {
   if (c.st->done) return;
   __shared__ NBShared sh;
-  ph_orth1(c, blockIdx.x, gridDim.x, j, sh);
-}
-__global__ void __launch_bounds__(kNT) nb_orth2_kernel(NBCtx c, int j) {
-  if (c.st->done) return;
-  __shared__ NBShared sh;
-  double beta;
-  ph_orth2_next(c, blockIdx.x, gridDim.x, j, sh, beta);
+  ph_orth_next(c, blockIdx.x, gridDim.x, j, sh);
 }
 __global__ void nb_tridiag_kernel(NBCtx c) {
   __shared__ NBShared sh;
@@ -848,32 +919,39 @@ __global__ void __launch_bounds__(kNT) nb_resid_kernel(NBCtx c) {
 __global__ void nb_final_kernel(NBCtx c) { ph_final(c); }
 
 // ----------------------------------------------------- persistent kernel
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ void red_release_add_u32(unsigned* p, unsigned v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // Grid-wide barrier of a cooperative launch: every CTA adds 1 to sync[0]
-// (zeroed before the launch); the k-th barrier is passed when it reaches
-// k * gridDim.x.  The wait is bounded: after kWaitLimitNs the CTA raises
-// PSD_ERR_TIMEOUT and sync[1], and every CTA that sees sync[1] leaves the
-// kernel at its next barrier.  Thread 0 keeps the count of barriers.
+// (zeroed before the launch) with release semantics, which the CTA barrier in
+// front extends to all its threads' writes; the k-th barrier is passed when it
+// reaches k * gridDim.x.  A poll is one 64-bit acquire load of the count and
+// the abort word sync[1] next to it; the clock is read on every 32nd poll only.
+// The wait is bounded: after the limit the CTA raises PSD_ERR_TIMEOUT and
+// sync[1], and every CTA that sees sync[1] leaves the kernel at its next
+// barrier.  Thread 0 keeps the count of barriers.
 struct GridBarrier {
-  unsigned* sync;
+  unsigned* sync;  // 8-byte aligned
+  unsigned long long limit;
   unsigned epoch;
   __device__ __forceinline__ bool wait(int* status, volatile int* ok_sh) {
     __syncthreads();
     if (threadIdx.x == 0) {
       ++epoch;
       const unsigned target = epoch * gridDim.x;
-      __threadfence();
-      atomicAdd(sync, 1u);
+      red_release_add_u32(sync, 1u);
       int ok = 1;
-      const unsigned long long limit = g_debug_barrier_limit_ns;
-      const unsigned long long t0 = globaltimer_ns();
-      while (ld_acquire_u32(sync) < target) {
-        if (ld_acquire_u32(sync + 1) != 0u) {
+      unsigned long long t0 = 0;
+      for (unsigned poll = 0;; ++poll) {
+        const unsigned long long v = ld_acquire_u64(reinterpret_cast<const unsigned long long*>(sync));
+        if (static_cast<unsigned>(v) >= target) break;
+        if (static_cast<unsigned>(v >> 32) != 0u) {
           // another CTA gave up; record it too: the first phase resets the
           // status word in CTA 0, which may run after that CTA's record, and
           // every CTA (CTA 0 included) leaves through a barrier after its own
@@ -882,14 +960,17 @@ struct GridBarrier {
           ok = 0;
           break;
         }
-        if (globaltimer_ns() - t0 >= limit) {  // >=: a zero limit gives up on the first poll
-          atomicExch(sync + 1, 1u);
-          atomicCAS(status, 0, PSD_ERR_TIMEOUT);
-          ok = 0;
-          break;
+        if ((poll & 31u) == 0u) {
+          const unsigned long long now = globaltimer_ns();
+          if (poll == 0u) t0 = now;
+          if (now - t0 >= limit) {  // >=: a zero limit gives up on the first poll
+            atomicExch(sync + 1, 1u);
+            atomicCAS(status, 0, PSD_ERR_TIMEOUT);
+            ok = 0;
+            break;
+          }
         }
       }
-      __threadfence();
       *ok_sh = ok;
     }
     __syncthreads();
@@ -901,15 +982,41 @@ struct GridBarrier {
 // same order, separated by grid barriers instead of kernel boundaries (about
 // 150 of them, each a few microseconds shorter than a kernel boundary, and no
 // launch of a small FP64 vector kernel waits on an empty GPU).
+//
+// RESIDENT: at most two tiles per CTA, loaded once -- the first into registers,
+// the second into shared memory (64 KB, dynamic; not allocated when no CTA has
+// two) -- so X is read from global memory once instead of 42 times.
+template <bool RESIDENT>
 __global__ void __launch_bounds__(kNT, 2) nb_persistent_kernel(NBCtx c, unsigned* sync) {
+  extern __shared__ float4 xs[];
   __shared__ NBShared sh;
   __shared__ volatile int ok_sh;
-  GridBarrier gb{sync, 0u};
+  GridBarrier gb{sync, g_debug_barrier_limit_ns, 0u};
   int* status = &c.st->status;
   const int G = gridDim.x, b0 = blockIdx.x;
   const int npair = (c.npart + 1) / 2;  // chunk pairs of the reducing phases
   const float* X = c.args->X;
   const int64_t ld = c.args->ld;
+  float x[8][8];
+  if (RESIDENT) {
+    if (b0 + G < c.ntiles) {
+      tile_load_x(X, ld, c.n, tile_geom(b0 + G), x);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        xs[kNT * (2 * k) + threadIdx.x] = make_float4(x[k][0], x[k][1], x[k][2], x[k][3]);
+        xs[kNT * (2 * k + 1) + threadIdx.x] = make_float4(x[k][4], x[k][5], x[k][6], x[k][7]);
+      }
+    }
+    if (b0 < c.ntiles) tile_load_x(X, ld, c.n, tile_geom(b0), x);
+  }
+  int pass = 0;
+  auto product = [&](auto stats) {
+    constexpr bool kStats = decltype(stats)::value;
+    if constexpr (RESIDENT)
+      ph_symv_resident<kStats>(c, b0, G, x, xs, sh);
+    else
+      ph_symv_run<kStats>(c, X, ld, b0, G, (pass++ & 1) != 0, sh);
+  };
 #define NB_SYNC()                           \
   do {                                      \
     if (!gb.wait(status, &ok_sh)) return;   \
@@ -918,26 +1025,21 @@ __global__ void __launch_bounds__(kNT, 2) nb_persistent_kernel(NBCtx c, unsigned
   NB_SYNC();
   for (int vb = b0; vb < c.nv; vb += G) ph_norm0(c, vb, sh);
   NB_SYNC();
-  int pass = 0;
   for (int j = 0; j < kMaxSteps; ++j) {
-    const bool rev = (pass++ & 1) != 0;
     if (j == 0)
-      ph_symv_run<true>(c, X, ld, b0, G, rev, sh);
+      product(std::true_type{});
     else
-      ph_symv_run<false>(c, X, ld, b0, G, rev, sh);
+      product(std::false_type{});
     NB_SYNC();
     if (j == 0 && b0 == 0 && threadIdx.x < 32) ph_fro(c);
     double* u = c.zsave ? c.zsave + j * c.npad : c.u;
     for (int cp = b0; cp < npair; cp += G) ph_reduce_split(c, cp, u, sh);
     NB_SYNC();
-    ph_symv_run<false>(c, X, ld, b0, G, (pass++ & 1) != 0, sh);
+    product(std::false_type{});
     NB_SYNC();
     for (int cp = b0; cp < npair; cp += G) ph_reduce_dots(c, cp, j, sh);
     NB_SYNC();
-    ph_orth1(c, b0, G, j, sh);
-    NB_SYNC();
-    double beta;
-    if (ph_orth2_next(c, b0, G, j, sh, beta)) break;  // the same decision in every CTA
+    if (ph_orth_next(c, b0, G, j, sh)) break;  // the same decision in every CTA
     NB_SYNC();
   }
   __syncthreads();  // thread 0's record of the last step, for warp 0
@@ -950,11 +1052,11 @@ __global__ void __launch_bounds__(kNT, 2) nb_persistent_kernel(NBCtx c, unsigned
     for (int vb = b0; vb < c.nv; vb += G) ph_ritz_norm(c, vb, inv);
   }
   NB_SYNC();
-  ph_symv_run<false>(c, X, ld, b0, G, (pass++ & 1) != 0, sh);
+  product(std::false_type{});
   NB_SYNC();
   for (int cp = b0; cp < npair; cp += G) ph_reduce_split(c, cp, c.u, sh);
   NB_SYNC();
-  ph_symv_run<false>(c, X, ld, b0, G, (pass++ & 1) != 0, sh);
+  product(std::false_type{});
   NB_SYNC();
   for (int cp = b0; cp < npair; cp += G) ph_resid(c, cp, sh);
   NB_SYNC();
@@ -1191,16 +1293,56 @@ NBCtx make_ctx(const LanczosBufs& L, const DevArgs* args, DevState* st) {
   return c;
 }
 
-// CTAs of the persistent kernel: as many as can be resident at once (a
-// cooperative launch needs every CTA resident), no more than the largest
-// phase has virtual blocks.  0 if the device cannot run it.
-int persistent_grid(const NBCtx& c) {
-  int dev = 0, sms = 0, occ = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, nb_persistent_kernel, kNT, 0) != cudaSuccess) return 0;
-  const int work = std::max(std::max(c.ntiles, c.npart), c.nv);
-  return std::min(occ * sms, std::max(work, 1));
+constexpr int kTileSmem = static_cast<int>(sizeof(float)) * kSymvTile * kSymvTile;  // one resident tile
+
+// Form and grid of the persistent kernel.  A cooperative launch needs every CTA
+// resident: up to 2 per SM (128 registers; 64 KB + 17 KB of shared memory
+// each), no more than the largest phase has virtual blocks.  RESIDENT when two
+// tiles per CTA hold the whole triangle (304 CTAs: 608 tiles, n <= 4352).
+// grid 0: the device cannot run it.
+struct PersistentForm {
+  int grid = 0;
+  bool resident = false;
+  int smem = 0;
+};
+PersistentForm persistent_form(const NBCtx& c) {
+  // occupancies by device, looked up once (callers on several threads and streams)
+  struct Occ {
+    int sms = 0, stream = 0, one = 0, two = 0;
+  };
+  static std::mutex mu;
+  static std::map<int, Occ> known;
+  PersistentForm f;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return f;
+  Occ o;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = known.find(dev);
+    if (it != known.end()) {
+      o = it->second;
+    } else {
+      if (cudaDeviceGetAttribute(&o.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+          cudaFuncSetAttribute(nb_persistent_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem) !=
+              cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o.stream, nb_persistent_kernel<false>, kNT, 0) !=
+              cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o.one, nb_persistent_kernel<true>, kNT, 0) != cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o.two, nb_persistent_kernel<true>, kNT, kTileSmem) !=
+              cudaSuccess)
+        return f;
+      known[dev] = o;
+    }
+  }
+  const int work = std::max(std::max(std::max(c.ntiles, c.npart), c.nv), 1);
+  if (c.ntiles <= o.one * o.sms) {
+    f = PersistentForm{std::min(o.one * o.sms, work), true, 0};
+  } else if (c.ntiles <= 2 * o.two * o.sms) {
+    f = PersistentForm{std::min(o.two * o.sms, work), true, kTileSmem};
+  } else {
+    f = PersistentForm{std::min(o.stream * o.sms, work), false, 0};
+  }
+  return f;
 }
 
 }  // namespace
@@ -1209,21 +1351,26 @@ cudaError_t enqueue_norm_bound(const LanczosBufs& L, const DevArgs* args, DevSta
                                bool persistent) {
   const NBCtx c = make_ctx(L, args, st);
   if (persistent) {
-    const int G = persistent_grid(c);
-    if (G > 0) {
+    const PersistentForm f = persistent_form(c);
+    if (f.grid > 0) {
       cudaError_t e = cudaMemsetAsync(L.sync, 0, 2 * sizeof(unsigned), s);
       if (e != cudaSuccess) return e;
       cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3(G);
+      cfg.gridDim = dim3(f.grid);
       cfg.blockDim = dim3(kNT);
-      cfg.dynamicSmemBytes = 0;
+      if (f.smem > 0) {  // on every call: a device reset drops it
+        e = cudaFuncSetAttribute(nb_persistent_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, f.smem);
+        if (e != cudaSuccess) return e;
+      }
+      cfg.dynamicSmemBytes = f.smem;
       cfg.stream = s;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeCooperative;
       attr[0].val.cooperative = 1;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
-      return cudaLaunchKernelEx(&cfg, nb_persistent_kernel, c, L.sync);
+      return f.resident ? cudaLaunchKernelEx(&cfg, nb_persistent_kernel<true>, c, L.sync)
+                        : cudaLaunchKernelEx(&cfg, nb_persistent_kernel<false>, c, L.sync);
     }
   }
   const int vb = c.nv, rb = c.npart, pb = (c.npart + 1) / 2;  // pb: chunk pairs
@@ -1241,8 +1388,7 @@ cudaError_t enqueue_norm_bound(const LanczosBufs& L, const DevArgs* args, DevSta
     nb_reduce_split_kernel<<<pb, kNT, 0, s>>>(c, u, 1);
     nb_symv_kernel<false><<<c.ntiles, kNT, 0, s>>>(c, 1, pass++ & 1);
     nb_reduce_dots_kernel<<<pb, kNT, 0, s>>>(c, j);
-    nb_orth1_kernel<<<rb, kNT, 0, s>>>(c, j);
-    nb_orth2_kernel<<<rb, kNT, 0, s>>>(c, j);
+    nb_orth_kernel<<<rb, kNT, 0, s>>>(c, j);
   }
   nb_tridiag_kernel<<<1, 32, 0, s>>>(c);
   nb_ritz_kernel<<<rb, kNT, 0, s>>>(c);
