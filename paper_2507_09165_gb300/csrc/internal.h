@@ -159,7 +159,9 @@ struct GemmParams {
   const int4* tiles;     // (m0, n0, block, ncols) of each 128-row output tile, upper triangle
   const BlockRec* blocks;
   uint32_t idesc;        // instruction descriptor without its N field
+  int tile_w;            // pair form: columns of a full tile (0: 256); B's boxes have half as many rows
   EpiParams ep;
+  __host__ __device__ int b_rows() const { return tile_w > 0 ? tile_w / 2 : 128; }
 };
 
 // A tile and the fields of its block that the producer and MMA roles need.
@@ -251,7 +253,9 @@ cudaError_t launch_symgemm(int dtype, int epi, const CUtensorMap& tmA, const CUt
 // with a 16-bit (out_dtype = dtype or -1) or FP16-pair output, and EPI_FINAL
 // (cres: 8 shares per tile; 16 with many_small).  many_small: 8 epilogue warps
 // per CTA and a 5-stage ring (16-bit outputs and EPI_FINAL).
-std::vector<int4> make_tile_list_pair(int64_t n, int block = 0, int group = 8);
+std::vector<int4> make_tile_list_pair(int64_t n, int block = 0, int group = 8, int width = 256);
+// Tile width of a single matrix's pair-form launches (GemmParams::tile_w).
+int pair_tile_width(int64_t n);
 cudaError_t launch_symgemm_pair(int dtype, int epi, const CUtensorMap& tmA, const CUtensorMap& tmB,
                                 const GemmParams& p, int grid, cudaStream_t stream, int out_dtype = -1,
                                 bool many_small = false);

@@ -127,8 +127,11 @@ struct Plan {
   BlockRec* d_block = nullptr;   // the one block of a single projection
   int4* d_tiles = nullptr;
   int ntiles = 0;
-  int4* d_tiles_pair = nullptr;  // 256-row tiles of the CTA-pair form of the 16-bit stage products
+  int4* d_tiles_pair = nullptr;  // 256 x 256 tiles of the final product of the 16-bit chains on CTA pairs
   int ntiles_pair = 0;
+  int4* d_tiles_bal = nullptr;  // 256 x tile_w tiles of every other product on CTA pairs (pair_tile_width)
+  int ntiles_bal = 0;
+  int tile_w = 0;
   int ncompl = 0;  // complementarity shares the final product writes (4 per one-SM tile, 8 per pair tile, 16 on the FP32 path)
   double* d_compl = nullptr;  // 4 per tile: shares of <out, X - out> from the final product
   cudaGraphExec_t exec = nullptr;
@@ -181,10 +184,14 @@ psd_status_t build_plan(Plan* p, void* user_ws, size_t user_bytes) {
   const size_t o_tiles = o_block + round_up(sizeof(BlockRec), 256);
   std::vector<int4> tiles_pair = make_tile_list_pair(n);
   p->ntiles_pair = static_cast<int>(tiles_pair.size());
+  p->tile_w = pair_tile_width(n);
+  std::vector<int4> tiles_bal = make_tile_list_pair(n, 0, 8, p->tile_w);
+  p->ntiles_bal = static_cast<int>(tiles_bal.size());
   const size_t o_compl = o_tiles + round_up(sizeof(int4) * std::max<size_t>(tiles.size(), 1), 256);
-  const size_t ncompl_max = std::max<size_t>(std::max(4 * tiles.size(), 16 * tiles_pair.size()), 1);
+  const size_t ncompl_max = std::max({4 * tiles.size(), 8 * tiles_pair.size(), 16 * tiles_bal.size(), size_t{1}});
   const size_t o_pair = o_compl + round_up(sizeof(double) * ncompl_max, 256);
-  const size_t small = o_pair + sizeof(int4) * std::max<size_t>(tiles_pair.size(), 1);
+  const size_t o_bal = o_pair + round_up(sizeof(int4) * std::max<size_t>(tiles_pair.size(), 1), 256);
+  const size_t small = o_bal + sizeof(int4) * std::max<size_t>(tiles_bal.size(), 1);
   uint8_t* sm = nullptr;
   if (cudaMalloc(&sm, small) != cudaSuccess) {
     cudaGetLastError();
@@ -198,11 +205,15 @@ psd_status_t build_plan(Plan* p, void* user_ws, size_t user_bytes) {
   p->d_tiles = reinterpret_cast<int4*>(sm + o_tiles);
   p->d_compl = reinterpret_cast<double*>(sm + o_compl);
   p->d_tiles_pair = reinterpret_cast<int4*>(sm + o_pair);
+  p->d_tiles_bal = reinterpret_cast<int4*>(sm + o_bal);
   if (!tiles.empty() &&
       cudaMemcpy(p->d_tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice) != cudaSuccess)
     return PSD_ERR_CUDA;
   if (!tiles_pair.empty() && cudaMemcpy(p->d_tiles_pair, tiles_pair.data(), sizeof(int4) * tiles_pair.size(),
                                         cudaMemcpyHostToDevice) != cudaSuccess)
+    return PSD_ERR_CUDA;
+  if (!tiles_bal.empty() && cudaMemcpy(p->d_tiles_bal, tiles_bal.data(), sizeof(int4) * tiles_bal.size(),
+                                       cudaMemcpyHostToDevice) != cudaSuccess)
     return PSD_ERR_CUDA;
   BlockRec br{};
   br.off = 0;
@@ -223,6 +234,12 @@ GemmParams base_params(const Plan* p) {
   g.blocks = p->d_block;
   g.ep.status = &p->d_state->status;
   return g;
+}
+
+void use_balanced_tiles(const Plan* p, GemmParams& g) {
+  g.num_tiles = p->ntiles_bal;
+  g.tiles = p->d_tiles_bal;
+  g.tile_w = p->tile_w;
 }
 
 // One product C = epi(A * B) (routes: chain.h gemm_route); `out` is the
@@ -262,11 +279,18 @@ cudaError_t gemm(Plan* p, int epi, const Mat& A, const Mat& B, const Mat* out, c
         (epi == EPI_FINAL || odt == dt || (odt == DT_F16X2 && dt == DT_F16))) {
       // 16-bit products on CTA pairs: M = 256, half of B in each CTA (128-row boxes)
       CUtensorMap ta, tb;
-      if (!encode_tmap(&ta, dt, part_ptr(p, A, 0), n, ldm, 128) || !encode_tmap(&tb, dt, part_ptr(p, B, 0), n, ldm, 128))
+      if (epi == EPI_FINAL) {
+        // 256-wide tiles at any order: the shares of <out, X - out> are per tile,
+        // and a served request's list is the same
+        g.num_tiles = p->ntiles_pair;
+        g.tiles = p->d_tiles_pair;
+      } else {
+        use_balanced_tiles(p, g);
+      }
+      if (!encode_tmap(&ta, dt, part_ptr(p, A, 0), n, ldm, 128) ||
+          !encode_tmap(&tb, dt, part_ptr(p, B, 0), n, ldm, g.b_rows()))
         return cudaErrorInvalidValue;
       const uint32_t fmt = dt == DT_BF16 ? 1u : 0u;
-      g.num_tiles = p->ntiles_pair;
-      g.tiles = p->d_tiles_pair;
       g.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | (16u << 24);  // M = 256; N per tile
       if (epi == EPI_FINAL) p->ncompl = 8 * p->ntiles_pair;
       return launch_symgemm_pair(dt, epi, ta, tb, g, grid, s, epi == EPI_FINAL ? -1 : odt);
@@ -283,11 +307,11 @@ cudaError_t gemm(Plan* p, int epi, const Mat& A, const Mat& B, const Mat* out, c
   if (route == ROUTE_F32) {
     const Mat* ops[2] = {&A, &B};
     CUtensorMap tm[4];
+    use_balanced_tiles(p, g);
     for (int i = 0; i < 4; ++i)
-      if (!encode_tmap(&tm[i], DT_F16X2, part_ptr(p, *ops[i >> 1], i & 1), n, ldm, 128, 64)) return cudaErrorInvalidValue;
-    g.num_tiles = p->ntiles_pair;
-    g.tiles = p->d_tiles_pair;
-    if (epi == EPI_FINAL) p->ncompl = 16 * p->ntiles_pair;
+      if (!encode_tmap(&tm[i], DT_F16X2, part_ptr(p, *ops[i >> 1], i & 1), n, ldm, i < 2 ? 128 : g.b_rows(), 64))
+        return cudaErrorInvalidValue;
+    if (epi == EPI_FINAL) p->ncompl = 16 * p->ntiles_bal;
     return launch_symgemm_f32(epi, tm, g, grid, s);
   }
   const bool b1 = route == ROUTE_X2;
@@ -299,16 +323,13 @@ cudaError_t gemm(Plan* p, int epi, const Mat& A, const Mat& B, const Mat* out, c
   const int out_mode = kind_is_pair(out->kind) ? 0 : 1;  // the final product of these chains is a 16-bit one
   // FP16-pair stage products on CTA pairs (M = 256, half of B in each CTA)
   const bool pair = b1 ? (epi == EPI_SCALE && out_mode == 1) : out_mode == 0;
-  const int brows = pair ? 128 : 256;
+  if (pair) use_balanced_tiles(p, g);
+  const int brows = pair ? g.b_rows() : 256;
   if (!encode_tmap(&tm[0], dt, part_ptr(p, PA, 0), n, ldm, 128, rb) ||
       !encode_tmap(&tm[1], dt, part_ptr(p, PA, 1), n, ldm, 128, rb) ||
       !encode_tmap(&tm[2], dt, part_ptr(p, PB, 0), n, ldm, brows, rb) ||
       !encode_tmap(&tm[3], dt, part_ptr(p, PB, b1 ? 0 : 1), n, ldm, brows, rb))
     return cudaErrorInvalidValue;
-  if (pair) {
-    g.num_tiles = p->ntiles_pair;
-    g.tiles = p->d_tiles_pair;
-  }
   return launch_symgemm_x3(dt, b1, epi, out_mode, tm, g, grid, s, pair);
 }
 

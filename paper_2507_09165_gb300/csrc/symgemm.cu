@@ -24,6 +24,8 @@
 #include <cuda_fp8.h>
 
 #include <algorithm>
+#include <climits>
+#include <cstdint>
 #include <cstdio>
 #include <mutex>
 
@@ -620,6 +622,7 @@ __global__ void __launch_bounds__(threads16(EW), 1)
     if (lane == 0) {
       uint32_t s = 0, ph = 0;
       bool ok = true, issued = false;
+      const uint32_t stage_tx = 2 * (kABytes16 + p.b_rows() * kRowBytes16);
       for (TileStream ts(p, cl, ncl); ok && ts.valid(); ts.advance()) {
         ts.prefetch();
         const TileMeta& m = ts.cur();
@@ -633,7 +636,7 @@ __global__ void __launch_bounds__(threads16(EW), 1)
             ok = false;
             break;
           }
-          if (leader) mbar_arrive_expect_tx(full_bar(s), 2 * kStageBytesP);  // both CTAs' copies
+          if (leader) mbar_arrive_expect_tx(full_bar(s), stage_tx);  // both CTAs' copies
           const uint32_t dst = smem_u32(stages + s * kStageBytesP);
           const uint32_t fb = mapa_shared(full_bar(s), 0);
           tma_load_2d_pair(dst, &tmA, kb * kBK16, ya, fb);
@@ -1240,8 +1243,20 @@ std::vector<int4> make_tile_list(int64_t n, int block, int group) {
 // tile, in the same grouped raster; widths trimmed to the columns below n,
 // rounded up to 32 (N/2 rows of B per CTA; the extra columns read zero-filled
 // rows and are not written).
-std::vector<int4> make_tile_list_pair(int64_t n, int block, int group) {
+std::vector<int4> make_tile_list_pair(int64_t n, int block, int group, int width) {
   std::vector<int4> tiles;
+  if (width < kBN) {
+    // block row I from its diagonal block on in steps of `width`; the trimmed
+    // last tiles of the rows go to the end of the list
+    std::vector<int4> last;
+    for (int m0 = 0; m0 < n; m0 += kBN)
+      for (int n0 = m0; n0 < n; n0 += width) {
+        const int w = std::min(width, static_cast<int>((n - n0 + 31) / 32 * 32));
+        (w == width ? tiles : last).push_back(make_int4(m0, n0, block, w));
+      }
+    tiles.insert(tiles.end(), last.begin(), last.end());
+    return tiles;
+  }
   const int nb = static_cast<int>((n + kBN - 1) / kBN);
   const int G = group > 0 ? group : 8;
   for (int g0 = 0; g0 < nb; g0 += G)
@@ -1251,6 +1266,33 @@ std::vector<int4> make_tile_list_pair(int64_t n, int block, int group) {
         tiles.push_back(make_int4(I * kBN, J * kBN, block, std::min(kBN, static_cast<int>((n - J * kBN + 31) / 32 * 32))));
     }
   return tiles;
+}
+
+// Columns per tile of one matrix's pair-form launches: the width (a multiple of
+// 32) with the least rounds x (290 + width).  A round is one tile per SM pair;
+// its time is a K loop that does not get shorter than ~290 columns' worth of
+// MMAs (operand loads through L2) plus a part in proportion to the width, as
+// measured on GB300 over n = 256-5000 and widths 32-256 (22 products, BF16):
+//   n = 256    256 -> 32 columns   261 -> 123 us     (1 tile -> 8)
+//   n = 1000   256 -> 64           394 -> 279 us     (10 -> 40 tiles)
+//   n = 2000   256 -> 128          493 -> 415 us     (36 -> 72)
+//   n = 3001   256 -> 160          908 -> 881 us     (two rounds either way)
+//   n = 4096   256 stays           1216 us (224: 1548, three rounds)
+// Elements do not depend on the width.
+int pair_tile_width(int64_t n) {
+  const int64_t clusters = std::max(1, num_sms() / 2);
+  int best = kBN;
+  int64_t best_cost = INT64_MAX;
+  for (int w = kBN; w >= 32; w -= 32) {
+    int64_t tiles = 0;
+    for (int64_t m0 = 0; m0 < n; m0 += kBN) tiles += (n - m0 + w - 1) / w;
+    const int64_t cost = (tiles + clusters - 1) / clusters * (290 + w);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = w;
+    }
+  }
+  return best;
 }
 
 cudaError_t launch_symgemm_pair(int dtype, int epi, const CUtensorMap& tmA, const CUtensorMap& tmB,

@@ -246,6 +246,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       if (lane == 0) {
         uint32_t s = 0, ph = 0;
         bool ok = true, issued = false;
+        const uint32_t stage_tx = 4 * (kOpBytes + p.b_rows() * kRowBytesF);
         for (TileStream ts(p, cl, ncl); ok && ts.valid(); ts.advance()) {
           ts.prefetch();
           const TileMeta& m = ts.cur();
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
               ok = false;
               break;
             }
-            if (leader) mbar_arrive_expect_tx(full_bar(s), 2 * kStageBytesF);  // both CTAs' copies
+            if (leader) mbar_arrive_expect_tx(full_bar(s), stage_tx);  // both CTAs' copies
             const uint32_t dst = smem_u32(stages + s * kStageBytesF);
             const uint32_t fb = mapa_shared(full_bar(s), 0);
             tma_load_2d_pair(dst, &tmAh, kb * kKElems, ya, fb);

@@ -410,6 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       int last_parity[kStages];
       for (int s = 0; s < kStages; ++s) last_parity[s] = -1;
+      const uint32_t stage_tx = 2 * (2 * kABytes + (B1 ? 1 : 2) * p.b_rows() * X3Cfg<B1, PAIR>::kRowBytes);  // pair form
       uint32_t s = 0, ph = 0;
       bool ok = true;
       for (TileStream ts(p, cl, ncl); ok && ts.valid(); ts.advance()) {
@@ -427,7 +428,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           const uint32_t base = smem_u32(stages + s * kStageBytes);
           if (PAIR) {
-            if (leader) mbar_arrive_expect_tx(full_bar(s), 2 * kStageBytes);  // both CTAs' copies
+            if (leader) mbar_arrive_expect_tx(full_bar(s), stage_tx);  // both CTAs' copies
             const uint32_t fb = mapa_shared(full_bar(s), 0);
             tma_load_2d_pair(base, &tmAh, kb * kKElems, ya, fb);
             tma_load_2d_pair(base + kABytes, &tmAl, kb * kKElems, ya, fb);
