@@ -28,17 +28,17 @@
 #include <cmath>
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <type_traits>
 
 #include "internal.h"
+#include "normbound.cuh"
 #include "ptx.cuh"
 #include "tridiag.cuh"
 
 namespace psd {
 
 namespace {
-
-constexpr uint64_t kSeed = 0x243F6A8885A308D3ull;  // Lanczos start vector seed
 
 // Host-side fault injection (psd_debug_set): a factor applied to lam~ (1.0:
 // none; a factor below 1 drives the chain past the composite's basin and
@@ -48,49 +48,6 @@ constexpr uint64_t kSeed = 0x243F6A8885A308D3ull;  // Lanczos start vector seed
 // captured graphs see the current values.
 __device__ double g_debug_bound_scale = 1.0;
 __device__ unsigned long long g_debug_barrier_limit_ns = kWaitLimitNs;
-constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ull;
-
-// ------------------------------------------------------- double-float helpers
-struct F2 {
-  float h, l;
-};
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float z = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
-}
-__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
-  float s, e;
-  two_sum(a.h, b.h, s, e);
-  return F2{s, __fadd_rn(__fadd_rn(a.l, b.l), e)};
-}
-__device__ __forceinline__ double f2_to_d(F2 a) { return static_cast<double>(a.h) + static_cast<double>(a.l); }
-__device__ __forceinline__ void split_d(double v, float& h, float& l) {
-  h = __double2float_rn(v);
-  l = __double2float_rn(v - static_cast<double>(h));
-}
-__device__ __forceinline__ F2 shfl_xor_f2(F2 a, int m) {
-  return F2{__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
-}
-
-// --------------------------------------------------------------- SplitMix64
-__device__ __forceinline__ uint64_t splitmix64(uint64_t seed, uint64_t i) {
-  uint64_t z = seed + (i + 1) * kGolden;
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  return z ^ (z >> 31);
-}
-
-// The FP32 estimate (FP64 runs at a small fraction of the FP32 rate on this GPU,
-// and every thread of a tile's CTA evaluates this) is corrected exactly by the
-// integer loops.
-__device__ __forceinline__ void tile_of(int t, int& bi, int& bj) {
-  int j = static_cast<int>((sqrtf(8.f * static_cast<float>(t) + 1.f) - 1.f) * 0.5f);
-  while ((j + 1) * (j + 2) / 2 <= t) ++j;
-  while (j * (j + 1) / 2 > t) --j;
-  bj = j;
-  bi = t - j * (j + 1) / 2;
-}
 
 // ------------------------------------------------------------------ phases
 //
@@ -103,7 +60,6 @@ __device__ __forceinline__ void tile_of(int t, int& bi, int& bj) {
 // Vectors an earlier phase wrote are read with ld.global.cg (through L2): in
 // the persistent kernel they change while it runs, which the non-coherent
 // read-only path must not be used for.
-constexpr int kNT = 256;
 static_assert(kVecThreads == kNT, "vector phases: one element per thread of a 256-thread block");
 
 // Shared memory of one CTA, reused by the phases (each virtual block ends
@@ -179,43 +135,6 @@ __device__ __forceinline__ double warp_sum_array(const double* a, int cnt, int s
   return s;
 }
 
-// Recursive-halving sum of cnt (<= 32) FP64 values over a warp; on return
-// lane l holds the warp total of value l.  Values live in v[0..31].
-__device__ __forceinline__ double warp_multi_sum(double (&v)[32], int lane) {
-#pragma unroll
-  for (int half = 16, m = 16; half >= 1; half >>= 1, m >>= 1) {
-    const bool upper = (lane & m) != 0;
-#pragma unroll
-    for (int i = 0; i < half; ++i) {
-      const double send = upper ? v[i] : v[i + half];
-      const double keep = upper ? v[i + half] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
-    }
-  }
-  return v[0];
-}
-
-// One tile of y = X v over the upper triangle (see file comment), in three
-// pieces so that the persistent kernel can load the next tile while it
-// reduces the current one.  Thread (tr, tc) = (lane & 15, 2 warp + lane / 16)
-// owns rows i0 + 8 tr .. +7 and columns j0 + 8 tc .. +7: each column's 128
-// rows are read by a half-warp as 512 contiguous bytes.  DIAG tiles mask to
-// i <= j (rows) and i < j (columns).  STATS adds the tile's share of
-// ||X||_F^2 and max |X_ii|.
-struct TileGeom {
-  int bi, bj, ib, jb;
-  bool diag;
-};
-__device__ __forceinline__ TileGeom tile_geom(int t) {
-  TileGeom g;
-  tile_of(t, g.bi, g.bj);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  g.ib = g.bi * kSymvTile + 8 * (lane & 15);
-  g.jb = g.bj * kSymvTile + 8 * (2 * warp + (lane >> 4));
-  g.diag = g.bi == g.bj;
-  return g;
-}
-
 // The thread's 8-element slices of v: rows (vi) and columns (vj); zeros past n.
 // vh holds npad (a multiple of 256) floats and the slices start at multiples of 8.
 __device__ __forceinline__ void tile_load_v(int n, const TileGeom& g, const float* vh, float (&vi)[8],
@@ -233,144 +152,17 @@ __device__ __forceinline__ void tile_load_v(int n, const TileGeom& g, const floa
   }
 }
 
-// The thread's 64 elements: 16 independent 16-byte loads of X in flight.
-__device__ __forceinline__ void tile_load_x(const float* __restrict__ X, int64_t ld, int n, const TileGeom& g,
-                                            float (&x)[8][8]) {
-  const bool full = (g.ib + 7 < n) && (g.jb + 7 < n);
-  const bool vec = full && ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const float* col = X + static_cast<int64_t>(g.jb + c) * ld + g.ib;
-    if (vec) {
-      const float4 a4 = __ldg(reinterpret_cast<const float4*>(col));
-      const float4 b4 = __ldg(reinterpret_cast<const float4*>(col + 4));
-      x[c][0] = a4.x; x[c][1] = a4.y; x[c][2] = a4.z; x[c][3] = a4.w;
-      x[c][4] = b4.x; x[c][5] = b4.y; x[c][6] = b4.z; x[c][7] = b4.w;
-    } else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) x[c][k] = (g.jb + c < n && g.ib + k < n) ? __ldg(col + k) : 0.f;
-    }
-  }
-}
-
-// Per-thread row and column dot products of the 8 x 8 block (8-term FP32 FMA runs).
-// `col(c, x)` gives column c of the block.
-template <bool STATS, bool DIAG, class Col>
-__device__ __forceinline__ void tile_fma(int n, const TileGeom& g, const float (&vi)[8], const float (&vj)[8],
-                                         const Col& col, float (&rsum)[8], float (&csum)[8], float& fro,
-                                         unsigned& mdiag) {
-  fro = 0.f;
-  mdiag = 0;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) rsum[k] = 0.f;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    float x[8];
-    col(c, x);
-    csum[c] = 0.f;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      float xr = x[k], xc = x[k];
-      if (DIAG) {
-        const int i = g.ib + k, j = g.jb + c;
-        xr = (i <= j) ? xr : 0.f;
-        xc = (i < j) ? xc : 0.f;
-        if (STATS && i == j && i < n) mdiag = max(mdiag, __float_as_uint(fabsf(x[k])));
-      }
-      rsum[k] = fmaf(xr, vj[c], rsum[k]);
-      csum[c] = fmaf(xc, vi[k], csum[c]);
-      if (STATS) fro = fmaf(xr, xc + xr, fro);  // x^2 on the diagonal, 2 x^2 above it
-    }
-  }
-}
-
-// tile_fma of a tile held in registers.
-template <bool STATS>
-__device__ __forceinline__ void tile_fma_reg(int n, const TileGeom& g, const float (&vi)[8], const float (&vj)[8],
-                                             const float (&x)[8][8], float (&rsum)[8], float (&csum)[8], float& fro,
-                                             unsigned& mdiag) {
-  auto col = [&](int c, float (&o)[8]) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) o[k] = x[c][k];
-  };
-  if (g.diag)
-    tile_fma<STATS, true>(n, g, vi, vj, col, rsum, csum, fro, mdiag);
-  else
-    tile_fma<STATS, false>(n, g, vi, vj, col, rsum, csum, fro, mdiag);
-}
-
-// Combines the threads' sums in a fixed order (double-float) into the tile's
-// row partials P1[bj][rows] and column partials P2[bi][columns], through row
-// buffer `buf`.  Ends with a CTA barrier unless `sync_after` is false: a run
-// of tiles alternates the two buffers instead, since a tile two ahead writes a
-// buffer only after every thread has passed the barrier of the tile between
-// (and so finished reading it); the run is followed by a CTA barrier.
-template <bool STATS>
-__device__ __forceinline__ void tile_reduce_store(int n, const TileGeom& g, const float (&rsum)[8],
-                                                  const float (&csum)[8], float fro, unsigned mdiag, float2* P1,
-                                                  float2* P2, int64_t ps, double* tile_fro, DevState* st,
-                                                  NBShared& sh, int tile, int buf = 0,
-                                                  bool sync_after = true) {
-  float2 (*red)[kSymvTile] = sh.u.mv.red[buf];
-  const int i0 = g.bi * kSymvTile;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tr = lane & 15;
-  // rows: the two column groups of a warp (exact TwoSum), then the 8 warps
-  F2 rs[8], cs[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const float o = __shfl_xor_sync(0xffffffffu, rsum[k], 16);
-    float h, e;
-    if (lane < 16) two_sum(rsum[k], o, h, e); else two_sum(o, rsum[k], h, e);
-    rs[k] = F2{h, e};
-    cs[k] = F2{csum[k], 0.f};
-  }
-  if (lane < 16) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) red[warp][8 * tr + k] = make_float2(rs[k].h, rs[k].l);
-  }
-  // columns: recursive halving over the 16 row groups of a half-warp
-#pragma unroll
-  for (int half = 4, m = 8; half >= 1; half >>= 1, m >>= 1) {
-    const bool upper = (tr & m) != 0;
-#pragma unroll
-    for (int i = 0; i < half; ++i) {
-      const F2 send = upper ? cs[i] : cs[i + half];
-      const F2 keep = upper ? cs[i + half] : cs[i];
-      cs[i] = f2_add(keep, shfl_xor_f2(send, m));
-    }
-  }
-  {
-    const F2 o = shfl_xor_f2(cs[0], 1);
-    cs[0] = (tr & 1) ? f2_add(o, cs[0]) : f2_add(cs[0], o);
-    const int j = g.jb + (tr >> 1);
-    if ((tr & 1) == 0 && j < n) P2[static_cast<int64_t>(g.bi) * ps + j] = make_float2(cs[0].h, cs[0].l);
-  }
-  __syncthreads();
-  if (threadIdx.x < kSymvTile) {
-    const int r = threadIdx.x;
-    F2 a{red[0][r].x, red[0][r].y};
-#pragma unroll
-    for (int w = 1; w < 8; ++w) a = f2_add(a, F2{red[w][r].x, red[w][r].y});
-    if (i0 + r < n) P1[static_cast<int64_t>(g.bj) * ps + i0 + r] = make_float2(a.h, a.l);
-  }
-  if (STATS) {
-    double f = static_cast<double>(fro);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-    if (lane == 0) sh.u.mv.fro[warp] = f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mdiag = max(mdiag, __shfl_xor_sync(0xffffffffu, mdiag, o));
-    if (lane == 0 && mdiag) atomicMax(&st->maxdiag_bits, mdiag);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double sum = 0.0;
-      for (int w = 0; w < 8; ++w) sum += sh.u.mv.fro[w];
-      tile_fro[tile] = sum;
-    }
-  }
-  if (sync_after) __syncthreads();
-}
+// Tile `t` = (bi, bj)'s results in global memory: row partials P1[bj][rows],
+// column partials P2[bi][columns], ||X||_F^2 share, max |X_ii|.
+struct GlobalSink {
+  const NBCtx& c;
+  const TileGeom& g;
+  int tile;
+  __device__ __forceinline__ void row(int i, float2 v) const { c.P1[static_cast<int64_t>(g.bj) * c.npad + i] = v; }
+  __device__ __forceinline__ void col(int j, float2 v) const { c.P2[static_cast<int64_t>(g.bi) * c.npad + j] = v; }
+  __device__ __forceinline__ void diag(unsigned m) const { atomicMax(&c.st->maxdiag_bits, m); }
+  __device__ __forceinline__ void fro(double f) const { c.tile_fro[tile] = f; }
+};
 
 // Tile t of a product over X (t in [0, ntiles)), one tile per call.
 template <bool STATS>
@@ -381,7 +173,7 @@ __device__ __forceinline__ void ph_symv(const NBCtx& c, const float* X, int64_t 
   tile_load_v(c.n, g, c.vh, vi, vj);
   tile_load_x(X, ld, c.n, g, x);
   tile_fma_reg<STATS>(c.n, g, vi, vj, x, rsum, csum, fro, mdiag);
-  tile_reduce_store<STATS>(c.n, g, rsum, csum, fro, mdiag, c.P1, c.P2, c.npad, c.tile_fro, c.st, sh, t);
+  tile_reduce<STATS>(c.n, g, rsum, csum, fro, mdiag, sh.u.mv.red[0], sh.u.mv.fro, GlobalSink{c, g, t}, true);
 }
 
 // Tiles r = first, first + stride, ... < ntiles of a product (in the
@@ -409,8 +201,8 @@ __device__ __forceinline__ void ph_symv_run(const NBCtx& c, const float* X, int6
       tile_load_v(c.n, gn, c.vh, vi, vj);
       tile_load_x(X, ld, c.n, gn, x);
     }
-    tile_reduce_store<STATS>(c.n, g, rsum, csum, fro, mdiag, c.P1, c.P2, c.npad, c.tile_fro, c.st, sh,
-                             tile_at(r), buf, false);
+    tile_reduce<STATS>(c.n, g, rsum, csum, fro, mdiag, sh.u.mv.red[buf], sh.u.mv.fro, GlobalSink{c, g, tile_at(r)},
+                       false);
     if (rn >= c.ntiles) break;
     r = rn;
     g = gn;
@@ -433,7 +225,7 @@ __device__ __forceinline__ void ph_symv_resident(const NBCtx& c, int b0, int str
   const int t1 = b0 + stride;
   const TileGeom g1 = tile_geom(t1 < c.ntiles ? t1 : b0);
   if (t1 < c.ntiles) tile_load_v(c.n, g1, c.vh, vi, vj);
-  tile_reduce_store<STATS>(c.n, g, rsum, csum, fro, mdiag, c.P1, c.P2, c.npad, c.tile_fro, c.st, sh, b0, 0, false);
+  tile_reduce<STATS>(c.n, g, rsum, csum, fro, mdiag, sh.u.mv.red[0], sh.u.mv.fro, GlobalSink{c, g, b0}, false);
   if (t1 >= c.ntiles) return;
   auto col = [&](int k, float (&o)[8]) {
     const float4 a = xs[kNT * (2 * k) + threadIdx.x], b = xs[kNT * (2 * k + 1) + threadIdx.x];
@@ -444,18 +236,14 @@ __device__ __forceinline__ void ph_symv_resident(const NBCtx& c, int b0, int str
     tile_fma<STATS, true>(c.n, g1, vi, vj, col, rsum, csum, fro, mdiag);
   else
     tile_fma<STATS, false>(c.n, g1, vi, vj, col, rsum, csum, fro, mdiag);
-  tile_reduce_store<STATS>(c.n, g1, rsum, csum, fro, mdiag, c.P1, c.P2, c.npad, c.tile_fro, c.st, sh, t1, 1, false);
+  tile_reduce<STATS>(c.n, g1, rsum, csum, fro, mdiag, sh.u.mv.red[1], sh.u.mv.fro, GlobalSink{c, g1, t1}, false);
 }
 
 // State reset and the start vector q_0 (unit SplitMix64 vector, before scaling).
 __device__ __forceinline__ void ph_init(const NBCtx& c, int vb, NBShared& sh) {
   const int e = vb * kNT + threadIdx.x;
   double v = 0.0;
-  if (e < c.n) {
-    const uint64_t z = splitmix64(kSeed, static_cast<uint64_t>(e));
-    const double u = static_cast<double>(z >> 11) * 0x1.0p-53;
-    v = 2.0 * u - 1.0;
-  }
+  if (e < c.n) v = lanczos_start(e);
   const double s = block_sum64(v * v, sh.bs);
   if (threadIdx.x == 0) c.norms[vb] = s;
   if (e < c.n) c.Qv[e] = v;  // unnormalised; ph_norm0 scales it
@@ -544,48 +332,6 @@ __device__ __forceinline__ double reduce_partials(const NBCtx& c, int ch, NBShar
   return y;
 }
 
-__device__ __forceinline__ float2 d_to_f2(double v) {
-  const float h = __double2float_rn(v);
-  return make_float2(h, __double2float_rn(v - static_cast<double>(h)));
-}
-
-// Warp sum of one FP64 value per lane as a double-float pair (fixed order;
-// every lane): FP32 shuffles and adds, this GPU's FP64 adds being far slower.
-__device__ __forceinline__ F2 warp_sum_f2(double v) {
-  const int lane = threadIdx.x & 31;
-  const float2 p = d_to_f2(v);
-  F2 t{p.x, p.y};
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const F2 other = shfl_xor_f2(t, o);
-    t = (lane & o) ? f2_add(other, t) : f2_add(t, other);
-  }
-  return t;
-}
-
-// Sum of nch double-float partials by one warp (lanes stride over them, 8 loads
-// in flight, then a butterfly; fixed order), as FP64 in every lane.
-__device__ __forceinline__ double warp_sum_chunks(const float2* part, int nch) {
-  const int lane = threadIdx.x & 31;
-  F2 acc{0.f, 0.f};
-  for (int c0 = 0; c0 < nch; c0 += 8 * 32) {
-    float2 t[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int ch = c0 + 32 * i + lane;
-      t[i] = ch < nch ? __ldcg(part + ch) : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) acc = f2_add(acc, F2{t[i].x, t[i].y});
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const F2 other = shfl_xor_f2(acc, o);
-    acc = (lane & o) ? f2_add(other, acc) : f2_add(acc, other);
-  }
-  return f2_to_d(acc);
-}
-
 // u = X v (first product of X (X v)); split u for the second product; the
 // chunk's share of ||u||^2 (= alpha_j, q_j being a unit vector).  Chunk pair cp.
 __device__ __forceinline__ void ph_reduce_split(const NBCtx& c, int cp, double* u, NBShared& sh) {
@@ -619,35 +365,6 @@ __device__ __forceinline__ void ph_reduce_split(const NBCtx& c, int cp, double* 
 // about 48 bits): every CTA adds them up itself in FP32 arithmetic, in the same
 // order, because this GPU issues FP64 at a small fraction of its FP32 rate.
 
-// S[k] = sum over the chunks of part[k * nch + ch] (slot-major: a warp's 32
-// lanes read 256 contiguous bytes) for the slots k with (want >> k) & 1,
-// double-float in a fixed order (lanes stride over the chunks, then a
-// butterfly), into shared memory as FP64.  Warp w takes the slots k = w,
-// w + 8, ...  The loads of a lane are issued 8 at a time.
-__device__ __forceinline__ void chunk_sums(const float2* part, int nch, uint32_t want, double* S) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int k = w; k < 32; k += kNT / 32) {
-    if (!((want >> k) & 1u)) continue;
-    F2 acc{0.f, 0.f};
-    for (int c0 = 0; c0 < nch; c0 += 8 * 32) {
-      float2 t[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int ch = c0 + 32 * i + lane;
-        t[i] = ch < nch ? __ldcg(part + static_cast<int64_t>(k) * nch + ch) : make_float2(0.f, 0.f);
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) acc = f2_add(acc, F2{t[i].x, t[i].y});
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const F2 other = shfl_xor_f2(acc, o);
-      acc = (lane & o) ? f2_add(other, acc) : f2_add(acc, other);
-    }
-    if (lane == 0) S[k] = f2_to_d(acc);
-  }
-}
-
 // w' = w - alpha_j q_j - beta_{j-1} q_{j-1}; the chunk's shares of q_k . w'
 // (k <= j) and ||w'||^2 (slot 31) into dots.  Chunk pair cp.
 __device__ __forceinline__ void ph_reduce_dots(const NBCtx& c, int cp, int j, NBShared& sh) {
@@ -657,7 +374,7 @@ __device__ __forceinline__ void ph_reduce_dots(const NBCtx& c, int cp, int j, NB
   const bool lead = half_lead_warp() && ch < c.npart;
   // alpha_j by a warp of the other half of the CTA's work; loads before the partial sums'
   if (threadIdx.x >= 32 && threadIdx.x < 64) {
-    const double a = warp_sum_chunks(c.norms2, c.npart);
+    const double a = warp_sum_chunks(c.norms2, c.npart, LoadCg());
     if (lane == 0) sh.scalar[0] = a;
   }
   double qk[kMaxSteps];
@@ -676,7 +393,7 @@ __device__ __forceinline__ void ph_reduce_dots(const NBCtx& c, int cp, int j, NB
     if (k == j) qj = qk[k];
     if (k == j - 1) qp = qk[k];
   }
-  y = (y - alpha * qj) - beta * qp;
+  y = lanczos_recur(y, alpha, qj, beta, qp);
   if (e < c.n) c.w[e] = y;
   double v[32];
 #pragma unroll
@@ -698,31 +415,26 @@ __device__ __forceinline__ bool ph_orth_next(const NBCtx& c, int cta, int ncta, 
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   constexpr int kW = kNT / 32;
   const double fro = __ldcg(&c.st->fro);
-  chunk_sums(c.dots, c.npart, ((2u << j) - 1u) | 0x80000000u, sh.u.orth.h);
+  chunk_sums(c.dots, c.npart, ((2u << j) - 1u) | 0x80000000u, sh.u.orth.h, LoadCg());
   __syncthreads();
   if (wp == kW - 1) {
     double h2 = lane <= j ? sh.u.orth.h[lane] * sh.u.orth.h[lane] : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) h2 += __shfl_xor_sync(0xffffffffu, h2, o);
     if (lane == 0) {
-      const double b2 = sh.u.orth.h[31] - h2;
-      const double r = rsqrt(b2);
-      sh.scalar[0] = b2 > 0.0 ? b2 * r : (b2 <= 0.0 ? 0.0 : b2);  // NaN stays NaN
-      sh.scalar[1] = r;
+      double b, inv;
+      lanczos_beta(sh.u.orth.h[31] - h2, b, inv);
+      sh.scalar[0] = b;
+      sh.scalar[1] = inv;
     }
   }
   auto next = [&](int ch) {  // w'' of the lane's element
     const int e = ch * 32 + lane;
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
     double qk[kMaxSteps];
 #pragma unroll
     for (int k = 0; k < kMaxSteps; ++k)
       qk[k] = (k <= j && e < c.n) ? __ldcg(c.Qv + static_cast<int64_t>(k) * c.npad + e) : 0.0;
-    const double we = e < c.n ? __ldcg(c.w + e) : 0.0;
-#pragma unroll
-    for (int k = 0; k < kMaxSteps; ++k)
-      if (k <= j) a[k & 3] += sh.u.orth.h[k] * qk[k];
-    return we - ((a[0] + a[1]) + (a[2] + a[3]));
+    return lanczos_orth(e < c.n ? __ldcg(c.w + e) : 0.0, sh.u.orth.h, qk, j);
   };
   const int ch0 = cta + ncta * wp;  // most CTAs have one chunk, on warp 0
   const double w0 = ch0 < c.npart ? next(ch0) : 0.0;
@@ -780,9 +492,7 @@ __device__ __forceinline__ void ph_ritz(const NBCtx& c, int cta, int ncta, NBSha
         qk[k] = k < m ? __ldcg(c.Qv + static_cast<int64_t>(k) * c.npad + e) : 0.0;
         yk[k] = k < m ? __ldcg(&c.st->y[k]) : 0.0;
       }
-#pragma unroll
-      for (int k = 0; k < kMaxSteps; ++k)
-        if (k < m) s += yk[k] * qk[k];
+      s = lanczos_ritz(yk, qk, m);
       c.q[e] = s;
     }
     const F2 t = warp_sum_f2(s * s);
@@ -794,7 +504,7 @@ __device__ __forceinline__ void ph_ritz(const NBCtx& c, int cta, int ncta, NBSha
 // (fixed order; 0 for a zero sum); every thread of the CTA receives it.
 __device__ __forceinline__ double inv_norm_of_sum(const NBCtx& c, NBShared& sh) {
   if (threadIdx.x < 32) {
-    const double s2 = warp_sum_chunks(c.norms2, c.npart);
+    const double s2 = warp_sum_chunks(c.norms2, c.npart, LoadCg());
     if (threadIdx.x == 0) sh.scalar[0] = s2 > 0.0 ? 1.0 / sqrt(s2) : 0.0;
   }
   __syncthreads();
@@ -826,20 +536,17 @@ __device__ __forceinline__ void ph_resid(const NBCtx& c, int cp, NBShared& sh) {
   if (lane == 0) c.norms2[ch] = make_float2(t.h, t.l);
 }
 
-// lam~ = max(sqrt(sigma + r), ||X||_F / sqrt n, max |X_ii|); report.  One warp.
-__device__ __forceinline__ void ph_final(const NBCtx& c) {
-  const double r2 = warp_sum_chunks(c.norms2, c.npart);
-  if (threadIdx.x != 0) return;
-  DevState* st = c.st;
+// lam~ = max(sqrt(sigma + r), ||X||_F / sqrt n, max |X_ii|) times `scale` (1.0
+// unless a test injects a bound that is too small) into the state and the
+// report.  One thread; r2 = r^2.
+__device__ void record_bound(DevState* st, psd_info_t* info, int n, double r2, double fro, double md, double sigma,
+                             int m, double scale) {
   const double r = sqrt(r2);
-  const double fro = __ldcg(&st->fro);
   const double fro2 = fro * fro;
-  const double md = static_cast<double>(__uint_as_float(__ldcg(&st->maxdiag_bits)));
-  const double sigma = __ldcg(&st->sigma);
   double lam = sqrt(fmax(sigma + r, 0.0));
-  lam = fmax(lam, fro / sqrt(static_cast<double>(c.n)));
+  lam = fmax(lam, fro / sqrt(static_cast<double>(n)));
   lam = fmax(lam, md);
-  lam *= g_debug_bound_scale;  // 1.0 unless a test injects a bound that is too small
+  lam *= scale;
   st->resid = r;
   st->maxdiag = md;
   const bool finite = isfinite(fro2) && isfinite(lam) && isfinite(sigma);
@@ -849,17 +556,26 @@ __device__ __forceinline__ void ph_final(const NBCtx& c) {
   }
   st->lambda = lam;
   st->inv_lambda = lam > 0.0 ? 1.0 / lam : 0.0;
-  psd_info_t* info = c.args->info;
   if (info) {
     info->lambda_bound = lam;
     info->lanczos_sigma = sigma;
     info->lanczos_resid = r;
     info->fro_X = fro;
     info->max_diag = md;
-    info->lanczos_steps = __ldcg(&st->m);
+    info->lanczos_steps = m;
     info->status = __ldcg(&st->status);
     info->compl_resid = __longlong_as_double(0x7ff8000000000000ll);  // set by a projection's last step
   }
+}
+
+// The bound from the residual's partials.  One warp.
+__device__ __forceinline__ void ph_final(const NBCtx& c) {
+  const double r2 = warp_sum_chunks(c.norms2, c.npart, LoadCg());
+  if (threadIdx.x != 0) return;
+  DevState* st = c.st;
+  record_bound(st, c.args->info, c.n, r2, __ldcg(&st->fro),
+               static_cast<double>(__uint_as_float(__ldcg(&st->maxdiag_bits))), __ldcg(&st->sigma), __ldcg(&st->m),
+               g_debug_bound_scale);
 }
 
 // ------------------------------------------------- multi-launch kernels
@@ -1063,6 +779,8 @@ __global__ void __launch_bounds__(kNT, 2) nb_persistent_kernel(NBCtx c, unsigned
   if (b0 == 0 && threadIdx.x < 32) ph_final(c);
 #undef NB_SYNC
 }
+
+#include "normbound_cluster.cuh"
 
 // Four consecutive elements (positions pos .. pos+3 of a row) of the output
 // matrix in the chain's storage: 16-bit, or an FP16 hi/lo pair of v * scale.
@@ -1345,11 +1063,89 @@ PersistentForm persistent_form(const NBCtx& c) {
   return f;
 }
 
+// Whether the current device runs clusters of `csize` CTAs with `smem` bytes
+// each (looked up once per device and shape).
+bool cluster_fits(int csize, int smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, int>, bool> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> lk(mu);
+  const auto key = std::make_tuple(dev, csize, smem);
+  auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(csize);
+  cfg.blockDim = dim3(kNT);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = csize;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int num = 0;
+  const bool ok =
+      cudaFuncSetAttribute(nb_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448) ==
+          cudaSuccess &&
+      cudaFuncSetAttribute(nb_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+          cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&num, nb_cluster_kernel, &cfg) == cudaSuccess && num > 0;
+  cudaGetLastError();
+  known[key] = ok;
+  return ok;
+}
+
+// The shape of a launch for a matrix of nb tile rows.
+ClusterJob cluster_job(int nb, int& smem) {
+  ClusterJob jb{};
+  cluster_shape(nb * (nb + 1) / 2, jb.csize, jb.extra);
+  jb.nbmax = nb;
+  jb.own = (4 * nb + jb.csize - 1) / jb.csize;
+  smem = cluster_carve(nullptr, nullptr, jb.extra, jb.own, nb);
+  return jb;
+}
+
+cudaError_t launch_cluster(const ClusterJob& jb, int smem, cudaStream_t s) {
+  cudaError_t e;  // the attributes on every call: a device reset drops them
+  if ((e = cudaFuncSetAttribute(nb_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448)) !=
+      cudaSuccess)
+    return e;
+  if ((e = cudaFuncSetAttribute(nb_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) !=
+      cudaSuccess)
+    return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(jb.csize);
+  cfg.blockDim = dim3(kNT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = jb.csize;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, nb_cluster_kernel, jb);
+}
+
 }  // namespace
 
 cudaError_t enqueue_norm_bound(const LanczosBufs& L, const DevArgs* args, DevState* st, cudaStream_t s,
                                bool persistent) {
   const NBCtx c = make_ctx(L, args, st);
+  if (persistent && c.nb <= kClusterMaxNb) {
+    int smem = 0;
+    ClusterJob jb = cluster_job(c.nb, smem);
+    if (cluster_fits(jb.csize, smem)) {
+      jb.args = args;
+      jb.n = c.n;
+      jb.st = st;
+      jb.Qv = c.Qv;
+      jb.zsave = c.zsave;
+      jb.npad = c.npad;
+      return launch_cluster(jb, smem, s);
+    }
+  }
   if (persistent) {
     const PersistentForm f = persistent_form(c);
     if (f.grid > 0) {
