@@ -389,6 +389,9 @@ struct LanczosBufs {
   float2* dots2;         // npart x 32 (second Gram-Schmidt pass; slot 31: ||w||^2)
   double* norms;         // max(npart, nvec_ctas) partial squared norms
   double* tile_fro;      // ntiles
+  // if set (16-byte aligned): room for ntiles packed 64 KB tiles, used by the
+  // persistent kernel when X's rows do not take 16-byte loads
+  float* pack = nullptr;
   double* zsave = nullptr;  // if set: X q_j of Lanczos step j kept at zsave + j npad (kMaxSteps x npad)
   unsigned* sync;        // 2 words: grid barrier of the persistent kernel (zeroed before each launch)
 };

@@ -97,6 +97,7 @@ struct NBCtx {
   double* norms;         // per 256-element block: FP64 partial of ||q_0||^2
   float2* norms2;        // per chunk: double-float partial of a squared norm (same storage as norms)
   double* tile_fro;
+  float4* pack;          // room for the packed tiles, or null
 };
 
 // Block-wide FP64 sum of one value per thread (kNT threads), fixed order;
@@ -180,17 +181,40 @@ __device__ __forceinline__ void ph_symv(const NBCtx& c, const float* X, int64_t 
 // opposite order of the tile list if `rev`), each loaded while the previous
 // one is reduced: the same arithmetic per tile as ph_symv.  The caller ends
 // the run with a CTA barrier (the grid barrier after the phase).
+// pack: the first product (STATS) also stores the tiles there, each thread's 16
+// float4 at [tile][q][thread], and the later ones read them from there; null:
+// all products read X.
 template <bool STATS>
-__device__ __forceinline__ void ph_symv_run(const NBCtx& c, const float* X, int64_t ld, int first, int stride,
-                                            bool rev, NBShared& sh) {
+__device__ __forceinline__ void ph_symv_run(const NBCtx& c, const float* X, int64_t ld, float4* pack, int first,
+                                            int stride, bool rev, NBShared& sh) {
   if (first >= c.ntiles) return;
   auto tile_at = [&](int r) { return rev ? c.ntiles - 1 - r : r; };
   float vi[8], vj[8], x[8][8];
   int r = first;
   int buf = 0;
   TileGeom g = tile_geom(tile_at(r));
+  auto load_x = [&](int tile, const TileGeom& tg) {
+    float4* p = pack ? pack + static_cast<int64_t>(tile) * (16 * kNT) + threadIdx.x : nullptr;
+    if (STATS || !pack) {
+      tile_load_x(X, ld, c.n, tg, x);
+      if (STATS && pack) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          p[kNT * (2 * k)] = make_float4(x[k][0], x[k][1], x[k][2], x[k][3]);
+          p[kNT * (2 * k + 1)] = make_float4(x[k][4], x[k][5], x[k][6], x[k][7]);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float4 a = __ldcg(p + kNT * (2 * k)), b = __ldcg(p + kNT * (2 * k + 1));
+        x[k][0] = a.x; x[k][1] = a.y; x[k][2] = a.z; x[k][3] = a.w;
+        x[k][4] = b.x; x[k][5] = b.y; x[k][6] = b.z; x[k][7] = b.w;
+      }
+    }
+  };
   tile_load_v(c.n, g, c.vh, vi, vj);
-  tile_load_x(X, ld, c.n, g, x);
+  load_x(tile_at(r), g);
   while (true) {
     float rsum[8], csum[8], fro;
     unsigned mdiag;
@@ -199,7 +223,7 @@ __device__ __forceinline__ void ph_symv_run(const NBCtx& c, const float* X, int6
     const TileGeom gn = tile_geom(tile_at(rn < c.ntiles ? rn : r));
     if (rn < c.ntiles) {  // in flight during the reduction
       tile_load_v(c.n, gn, c.vh, vi, vj);
-      tile_load_x(X, ld, c.n, gn, x);
+      load_x(tile_at(rn), gn);
     }
     tile_reduce<STATS>(c.n, g, rsum, csum, fro, mdiag, sh.u.mv.red[buf], sh.u.mv.fro, GlobalSink{c, g, tile_at(r)},
                        false);
@@ -713,6 +737,8 @@ __global__ void __launch_bounds__(kNT, 2) nb_persistent_kernel(NBCtx c, unsigned
   const int npair = (c.npart + 1) / 2;  // chunk pairs of the reducing phases
   const float* X = c.args->X;
   const int64_t ld = c.args->ld;
+  // rows that 16-byte loads cannot take: 41 of the 42 products read a packed copy
+  float4* pack = (ld & 3) != 0 || (reinterpret_cast<uintptr_t>(X) & 15) != 0 ? c.pack : nullptr;
   float x[8][8];
   if (RESIDENT) {
     if (b0 + G < c.ntiles) {
@@ -731,7 +757,7 @@ __global__ void __launch_bounds__(kNT, 2) nb_persistent_kernel(NBCtx c, unsigned
     if constexpr (RESIDENT)
       ph_symv_resident<kStats>(c, b0, G, x, xs, sh);
     else
-      ph_symv_run<kStats>(c, X, ld, b0, G, (pass++ & 1) != 0, sh);
+      ph_symv_run<kStats>(c, X, ld, pack, b0, G, (pass++ & 1) != 0, sh);
   };
 #define NB_SYNC()                           \
   do {                                      \
@@ -952,6 +978,7 @@ size_t lanczos_bytes(int64_t n) {
 
 void lanczos_carve(LanczosBufs& L, int64_t n, uint8_t* base) {
   L.zsave = nullptr;
+  L.pack = nullptr;
   L.n = n;
   L.npad = (n + 255) / 256 * 256;
   L.nb = static_cast<int>((n + kSymvTile - 1) / kSymvTile);
@@ -1008,6 +1035,7 @@ NBCtx make_ctx(const LanczosBufs& L, const DevArgs* args, DevState* st) {
   c.norms = L.norms;
   c.norms2 = reinterpret_cast<float2*>(L.norms);
   c.tile_fro = L.tile_fro;
+  c.pack = reinterpret_cast<float4*>(L.pack);
   return c;
 }
 

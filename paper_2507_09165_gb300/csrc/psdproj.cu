@@ -174,6 +174,9 @@ psd_status_t build_plan(Plan* p, void* user_ws, size_t user_bytes) {
   p->nslots = slots_needed(p->prec);
   p->slots = base;
   lanczos_carve(p->L, n, base + p->nslots * p->slot_size);
+  // the iterate slots are free while the norm bound runs: room for a packed copy of X's tiles
+  if (static_cast<size_t>(p->L.ntiles) * kSymvTile * kSymvTile * sizeof(float) <= p->nslots * p->slot_size)
+    p->L.pack = reinterpret_cast<float*>(base);
 
   // small library-owned records: args | state | info | tiles
   std::vector<int4> tiles = make_tile_list(n);
