@@ -139,7 +139,7 @@ psd_status_t psd_norm_bound(int64_t n, const float *X, int64_t ld, psd_info_t *d
  * or a latency-critical loop that cannot take the implicit synchronisation of
  * cudaMalloc.  Same computation and report as psd_norm_bound, for
  * 1 <= n <= 4096 (larger n: PSD_ERR_INVALID_ARG); the scratch lives in a
- * static device array of about 3 MB that every GPU loading the library holds
+ * static device array of about 3.6 MB that every GPU loading the library holds
  * until exit.  The first call on a device looks the array's address up
  * (cudaGetSymbolAddress) with that device current; make it before any stream
  * capture.  The address is kept with the CUDA context it was found in and

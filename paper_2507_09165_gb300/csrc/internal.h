@@ -378,15 +378,13 @@ struct LanczosBufs {
   int nvec_ctas;         // CTAs of the vector kernels (kVecThreads elements each)
   int npart;             // CTAs of the partial-sum reductions (32 elements each)
   double* Qv;            // (kMaxSteps + 1) x npad Lanczos vectors
-  double* u;             // npad
+  float2* Qf;            // kMaxSteps x npad Lanczos vectors as double-float pairs
   double* w;             // npad
   double* q;             // npad  Ritz vector
-  float* vh;             // npad  hi part of the mat-vec input
-  float* vl;             // npad  lo part
+  float* vh;             // npad  the mat-vec input (FP32)
   float2* P1;            // nb x npad row partials
   float2* P2;            // nb x npad column partials
-  float2* dots;          // npart x 32 double-float partial dot products (one chunk of 32 elements each)
-  float2* dots2;         // npart x 32 (second Gram-Schmidt pass; slot 31: ||w||^2)
+  float2* dots;          // npart x 32 double-float partial dot products (one chunk of 32 elements each; slot 31: ||w'||^2)
   double* norms;         // max(npart, nvec_ctas) partial squared norms
   double* tile_fro;      // ntiles
   // if set (16-byte aligned): room for ntiles packed 64 KB tiles, used by the

@@ -10,7 +10,7 @@
 // input and report buffers.
 //
 // The array g_noalloc_scratch holds the argument block, the device state and
-// the Lanczos buffers for orders up to kNoAllocMaxOrder (about 3 MB); every
+// the Lanczos buffers for orders up to kNoAllocMaxOrder (about 3.6 MB); every
 // GPU that loads the library holds it until the process exits.  In host code
 // the array's name is only a host-side stand-in, so the device address is
 // looked up with cudaGetSymbolAddress on the first call made with a device
@@ -44,8 +44,8 @@ constexpr size_t lanczos_bound_bytes(int64_t n) {
   const size_t ntiles = nb * (nb + 1) / 2;
   const size_t nctas = static_cast<size_t>((n + kVecThreads - 1) / kVecThreads);
   const size_t npart = static_cast<size_t>((n + 31) / 32);
-  return round256(8 * 21 * npad) + round256(8 * 3 * npad) + round256(4 * 2 * npad) +
-         round256(8 * 2 * nb * npad) + round256(8 * 32 * npart) + round256(8 * 32 * npart) +
+  return round256(8 * 21 * npad) + round256(8 * 20 * npad) + round256(8 * 2 * npad) + round256(4 * npad) +
+         round256(8 * 2 * nb * npad) + round256(8 * 32 * npart) +
          round256(8 * (npart > nctas ? npart : nctas)) + round256(8 * ntiles) + round256(4 * 2);
 }
 

@@ -67,13 +67,12 @@ static_assert(kVecThreads == kNT, "vector phases: one element per thread of a 25
 struct NBShared {
   union {
     struct {
-      float2 red[2][8][kSymvTile];  // two buffers: consecutive tiles of a run alternate
+      float2 red[2][8][kRedStride];  // two buffers: consecutive tiles of a run alternate
       double fro[8];
     } mv;
     float2 part[8][32];
     struct {
-      double h[32];
-      double w[8][32];
+      float2 s[32];
     } orth;
     struct {
       double y[kMaxSteps];
@@ -90,10 +89,11 @@ struct NBCtx {
   int64_t npad;
   const DevArgs* args;
   DevState* st;
-  double *Qv, *u, *w, *q, *zsave;
-  float *vh, *vl;
+  double *Qv, *w, *q, *zsave;
+  float2* Qf;            // Lanczos vectors as double-float pairs (for the dot products), kMaxSteps x npad
+  float* vh;             // mat-vec input (the vector rounded to FP32)
   float2 *P1, *P2;
-  float2 *dots, *dots2;  // per chunk: 32 double-float partials (dot products, slot 31 ||w||^2)
+  float2* dots;          // per chunk: 32 double-float partials (dot products, slot 31 ||w'||^2)
   double* norms;         // per 256-element block: FP64 partial of ||q_0||^2
   float2* norms2;        // per chunk: double-float partial of a squared norm (same storage as norms)
   double* tile_fro;
@@ -234,20 +234,19 @@ __device__ __forceinline__ void ph_symv_run(const NBCtx& c, const float* X, int6
   }
 }
 
-// The product over a CTA's resident tiles: tile b0 in registers (x), tile b0 +
-// stride (if any) in shared memory, each thread's own 16 float4 of it at
-// xs[256 q + thread] (read and written by that thread only).
+// The product over a CTA's resident tiles: tile b0 in registers (x, geometry
+// g), tile b0 + stride (if any; g1) in shared memory, each thread's own 16 float4
+// of it at xs[256 q + thread] (read and written by that thread only).
 template <bool STATS>
-__device__ __forceinline__ void ph_symv_resident(const NBCtx& c, int b0, int stride, const float (&x)[8][8],
-                                                 const float4* xs, NBShared& sh) {
+__device__ __forceinline__ void ph_symv_resident(const NBCtx& c, int b0, int stride, const TileGeom& g,
+                                                 const TileGeom& g1, const float (&x)[8][8], const float4* xs,
+                                                 NBShared& sh) {
   if (b0 >= c.ntiles) return;
   float vi[8], vj[8], rsum[8], csum[8], fro;
   unsigned mdiag;
-  const TileGeom g = tile_geom(b0);
   tile_load_v(c.n, g, c.vh, vi, vj);
   tile_fma_reg<STATS>(c.n, g, vi, vj, x, rsum, csum, fro, mdiag);
   const int t1 = b0 + stride;
-  const TileGeom g1 = tile_geom(t1 < c.ntiles ? t1 : b0);
   if (t1 < c.ntiles) tile_load_v(c.n, g1, c.vh, vi, vj);
   tile_reduce<STATS>(c.n, g, rsum, csum, fro, mdiag, sh.u.mv.red[0], sh.u.mv.fro, GlobalSink{c, g, b0}, false);
   if (t1 >= c.ntiles) return;
@@ -256,10 +255,7 @@ __device__ __forceinline__ void ph_symv_resident(const NBCtx& c, int b0, int str
     o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
     o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
   };
-  if (g1.diag)
-    tile_fma<STATS, true>(c.n, g1, vi, vj, col, rsum, csum, fro, mdiag);
-  else
-    tile_fma<STATS, false>(c.n, g1, vi, vj, col, rsum, csum, fro, mdiag);
+  tile_fma<STATS>(c.n, g1, vi, vj, col, rsum, csum, fro, mdiag);
   tile_reduce<STATS>(c.n, g1, rsum, csum, fro, mdiag, sh.u.mv.red[1], sh.u.mv.fro, GlobalSink{c, g1, t1}, false);
 }
 
@@ -291,6 +287,14 @@ __device__ __forceinline__ double bcast(double v, NBShared& sh, int k) {
   return r;
 }
 
+// Element e of Lanczos vector k: FP64, double-float pair and mat-vec input.
+__device__ __forceinline__ void put_lanczos(const NBCtx& c, int k, int e, double q) {
+  const float2 p = d_to_f2(q);
+  c.Qv[static_cast<int64_t>(k) * c.npad + e] = q;
+  c.Qf[static_cast<int64_t>(k) * c.npad + e] = p;
+  c.vh[e] = p.x;
+}
+
 // q_0 /= ||v||, split.
 __device__ __forceinline__ void ph_norm0(const NBCtx& c, int vb, NBShared& sh) {
   double s = 0.0;
@@ -299,9 +303,7 @@ __device__ __forceinline__ void ph_norm0(const NBCtx& c, int vb, NBShared& sh) {
   const double inv = bcast(s, sh, 0);
   const int e = vb * kNT + threadIdx.x;
   if (e < c.n) {
-    const double q = __ldcg(c.Qv + e) * inv;
-    c.Qv[e] = q;
-    split_d(q, c.vh[e], c.vl[e]);
+    put_lanczos(c, 0, e, __ldcg(c.Qv + e) * inv);
   }
 }
 
@@ -323,9 +325,9 @@ __device__ __forceinline__ bool half_lead_warp() { return (threadIdx.x & 127) < 
 // elements e of chunk `ch`, by the 4 warps of this thread's half of the CTA:
 // warp h (0-3 in the half) adds the blocks congruent to h mod 4 in
 // double-float, then the half's first warp combines the 4 warp sums in a fixed
-// order.  Returns y_e (FP64) in that warp; other warps return 0.  Both halves
+// order.  Returns y_e (a normalised pair) in that warp; other warps return 0.  Both halves
 // call it together (CTA barriers).
-__device__ __forceinline__ double reduce_partials(const NBCtx& c, int ch, NBShared& sh) {
+__device__ __forceinline__ F2 reduce_partials(const NBCtx& c, int ch, NBShared& sh) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, hw = w & 3;
   const int e = ch * 32 + lane;
   F2 a{0.f, 0.f}, d{0.f, 0.f};
@@ -345,29 +347,30 @@ __device__ __forceinline__ double reduce_partials(const NBCtx& c, int ch, NBShar
   const F2 t = f2_add(a, d);
   sh.u.part[w][lane] = make_float2(t.h, t.l);
   __syncthreads();
-  double y = 0.0;
+  F2 y{0.f, 0.f};
   if (hw == 0) {
     F2 acc{sh.u.part[w][lane].x, sh.u.part[w][lane].y};
 #pragma unroll
     for (int q = 1; q < 4; ++q) acc = f2_add(acc, F2{sh.u.part[w + q][lane].x, sh.u.part[w + q][lane].y});
-    y = f2_to_d(acc);
+    y = f2_norm(acc);
   }
   __syncthreads();
   return y;
 }
 
-// u = X v (first product of X (X v)); split u for the second product; the
-// chunk's share of ||u||^2 (= alpha_j, q_j being a unit vector).  Chunk pair cp.
+// u = X v (first product of X (X v)): the second product's input, the chunk's
+// share of ||u||^2 (= alpha_j, q_j being a unit vector), and u itself if asked
+// for.  Chunk pair cp.
 __device__ __forceinline__ void ph_reduce_split(const NBCtx& c, int cp, double* u, NBShared& sh) {
   const int ch = chunk_of_half(cp);
-  const double y = reduce_partials(c, ch, sh);
+  const F2 y = reduce_partials(c, ch, sh);
   if (!half_lead_warp() || ch >= c.npart) return;
   const int e = ch * 32 + (threadIdx.x & 31);
   if (e < c.n) {
-    u[e] = y;
-    split_d(y, c.vh[e], c.vl[e]);
+    if (u) u[e] = f2_to_d(y);
+    c.vh[e] = y.h;
   }
-  const F2 t = warp_sum_f2(e < c.n ? y * y : 0.0);
+  const F2 t = warp_sum_f2(f2_mul(y, y));  // y is 0 past n
   if ((threadIdx.x & 31) == 0) c.norms2[ch] = make_float2(t.h, t.l);
 }
 
@@ -384,10 +387,10 @@ __device__ __forceinline__ void ph_reduce_split(const NBCtx& c, int cp, double* 
 // passes on w itself took a phase and a grid barrier more per step.
 //
 // Element work is done per chunk of 32 elements by one warp (lane =
-// element), FP64.  Sums over the chunks (the dot products q_k . w' and ||w'||^2)
-// go through per-chunk partials stored as double-float pairs (FP32 hi + lo,
-// about 48 bits): every CTA adds them up itself in FP32 arithmetic, in the same
-// order, because this GPU issues FP64 at a small fraction of its FP32 rate.
+// element): the vectors and their updates in FP64, the dot products (q_k . w'
+// and ||w'||^2) and their sums over the chunks as double-float pairs (FP32 hi +
+// lo, about 48 bits), because this GPU issues FP64 at a small fraction of its
+// FP32 rate.  Every CTA adds the chunks' partials itself, in the same order.
 
 // w' = w - alpha_j q_j - beta_{j-1} q_{j-1}; the chunk's shares of q_k . w'
 // (k <= j) and ||w'||^2 (slot 31) into dots.  Chunk pair cp.
@@ -401,29 +404,24 @@ __device__ __forceinline__ void ph_reduce_dots(const NBCtx& c, int cp, int j, NB
     const double a = warp_sum_chunks(c.norms2, c.npart, LoadCg());
     if (lane == 0) sh.scalar[0] = a;
   }
-  double qk[kMaxSteps];
-  double beta = 0.0;
+  float2 qf[kMaxSteps];
+  double beta = 0.0, qj = 0.0, qp = 0.0;
 #pragma unroll
   for (int k = 0; k < kMaxSteps; ++k)
-    qk[k] = (lead && k <= j && e < c.n) ? __ldcg(c.Qv + static_cast<int64_t>(k) * c.npad + e) : 0.0;
-  if (lead && j > 0) beta = __ldcg(&c.st->beta[j - 1]);
-  double y = reduce_partials(c, ch, sh);  // its barriers publish sh.scalar[0]
+    qf[k] = (lead && k <= j && e < c.n) ? __ldcg(c.Qf + static_cast<int64_t>(k) * c.npad + e) : make_float2(0.f, 0.f);
+  if (lead && e < c.n) qj = __ldcg(c.Qv + static_cast<int64_t>(j) * c.npad + e);
+  if (lead && j > 0) {
+    beta = __ldcg(&c.st->beta[j - 1]);
+    if (e < c.n) qp = __ldcg(c.Qv + static_cast<int64_t>(j - 1) * c.npad + e);
+  }
+  const F2 y = reduce_partials(c, ch, sh);  // its barriers publish sh.scalar[0]
   const double alpha = sh.scalar[0];
   if (cp == 0 && threadIdx.x == 0) c.st->alpha[j] = alpha;
   if (!lead) return;
-  double qj = 0.0, qp = 0.0;
-#pragma unroll
-  for (int k = 0; k < kMaxSteps; ++k) {
-    if (k == j) qj = qk[k];
-    if (k == j - 1) qp = qk[k];
-  }
-  y = lanczos_recur(y, alpha, qj, beta, qp);
-  if (e < c.n) c.w[e] = y;
-  double v[32];
-#pragma unroll
-  for (int k = 0; k < 32; ++k) v[k] = k < kMaxSteps ? qk[k < kMaxSteps ? k : 0] * y : 0.0;
-  v[31] = e < c.n ? y * y : 0.0;
-  c.dots[static_cast<int64_t>(lane) * c.npart + ch] = d_to_f2(warp_multi_sum(v, lane));
+  const double w = lanczos_recur(f2_to_d(y), alpha, qj, beta, qp);
+  if (e < c.n) c.w[e] = w;
+  c.dots[static_cast<int64_t>(lane) * c.npart + ch] =
+      chunk_dots(f2_of(e < c.n ? w : 0.0), j, [&](int k) { return F2{qf[k].x, qf[k].y}; });
 }
 
 // The Gram-Schmidt pass and the next Lanczos vector.  Every CTA sums the
@@ -438,35 +436,26 @@ __device__ __forceinline__ void ph_reduce_dots(const NBCtx& c, int cp, int j, NB
 __device__ __forceinline__ bool ph_orth_next(const NBCtx& c, int cta, int ncta, int j, NBShared& sh) {
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   constexpr int kW = kNT / 32;
+  const int ch0 = cta + ncta * wp;  // most CTAs have one chunk, on warp 0
   const double fro = __ldcg(&c.st->fro);
-  chunk_sums(c.dots, c.npart, ((2u << j) - 1u) | 0x80000000u, sh.u.orth.h, LoadCg());
+  chunk_sums(c.dots, c.npart, c.npart, j, sh.u.orth.s, LoadCg());
   __syncthreads();
-  if (wp == kW - 1) {
-    double h2 = lane <= j ? sh.u.orth.h[lane] * sh.u.orth.h[lane] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) h2 += __shfl_xor_sync(0xffffffffu, h2, o);
-    if (lane == 0) {
-      double b, inv;
-      lanczos_beta(sh.u.orth.h[31] - h2, b, inv);
-      sh.scalar[0] = b;
-      sh.scalar[1] = inv;
-    }
-  }
+  if (wp == kW - 1) beta_of_sums(sh.u.orth.s, j, sh.scalar);
+  const double h = ch0 < c.npart && lane <= j ? f2_to_d(F2{sh.u.orth.s[lane].x, sh.u.orth.s[lane].y}) : 0.0;
   auto next = [&](int ch) {  // w'' of the lane's element
     const int e = ch * 32 + lane;
     double qk[kMaxSteps];
 #pragma unroll
     for (int k = 0; k < kMaxSteps; ++k)
       qk[k] = (k <= j && e < c.n) ? __ldcg(c.Qv + static_cast<int64_t>(k) * c.npad + e) : 0.0;
-    return lanczos_orth(e < c.n ? __ldcg(c.w + e) : 0.0, sh.u.orth.h, qk, j);
+    return lanczos_orth(e < c.n ? __ldcg(c.w + e) : 0.0, h, qk, j);
   };
-  const int ch0 = cta + ncta * wp;  // most CTAs have one chunk, on warp 0
   const double w0 = ch0 < c.npart ? next(ch0) : 0.0;
   __syncthreads();
   const double beta = sh.scalar[0];
   const bool stop = !(beta > kBreakdown * (fro * fro)) || j == kMaxSteps - 1;  // also true for NaN
   if (cta == 0 && threadIdx.x == 0) {
-    c.st->alpha[j] = __ldcg(&c.st->alpha[j]) + sh.u.orth.h[j];
+    c.st->alpha[j] = __ldcg(&c.st->alpha[j]) + f2_to_d(F2{sh.u.orth.s[j].x, sh.u.orth.s[j].y});
     c.st->beta[j] = beta;
     c.st->m = j + 1;
     if (stop) c.st->done = 1;
@@ -476,9 +465,7 @@ __device__ __forceinline__ bool ph_orth_next(const NBCtx& c, int cta, int ncta, 
     auto put = [&](int ch, double w) {
       const int e = ch * 32 + lane;
       if (e >= c.n) return;
-      const double q = w * inv;
-      c.Qv[static_cast<int64_t>(j + 1) * c.npad + e] = q;
-      split_d(q, c.vh[e], c.vl[e]);
+      put_lanczos(c, j + 1, e, w * inv);
     };
     if (ch0 < c.npart) put(ch0, w0);
     for (int ch = ch0 + ncta * kW; ch < c.npart; ch += ncta * kW) put(ch, next(ch));
@@ -519,7 +506,7 @@ __device__ __forceinline__ void ph_ritz(const NBCtx& c, int cta, int ncta, NBSha
       s = lanczos_ritz(yk, qk, m);
       c.q[e] = s;
     }
-    const F2 t = warp_sum_f2(s * s);
+    const F2 t = warp_sum_f2(f2_of(s * s));
     if (lane == 0) c.norms2[ch] = make_float2(t.h, t.l);
   }
 }
@@ -543,20 +530,20 @@ __device__ __forceinline__ void ph_ritz_norm(const NBCtx& c, int vb, double inv)
   if (e < c.n) {
     const double v = __ldcg(c.q + e) * inv;
     c.q[e] = v;
-    split_d(v, c.vh[e], c.vl[e]);
+    c.vh[e] = __double2float_rn(v);
   }
 }
 
 // r = X (X q) - sigma q, partial ||r||^2 of the chunk into norms2[ch].
 __device__ __forceinline__ void ph_resid(const NBCtx& c, int cp, NBShared& sh) {
   const int ch = chunk_of_half(cp);
-  const double y = reduce_partials(c, ch, sh);
+  const F2 y = reduce_partials(c, ch, sh);
   if (!half_lead_warp() || ch >= c.npart) return;
   const int lane = threadIdx.x & 31;
   const int e = ch * 32 + lane;
   double r = 0.0;
-  if (e < c.n) r = y - __ldcg(&c.st->sigma) * __ldcg(c.q + e);
-  const F2 t = warp_sum_f2(r * r);
+  if (e < c.n) r = fma(-__ldcg(&c.st->sigma), __ldcg(c.q + e), f2_to_d(y));
+  const F2 t = warp_sum_f2(f2_of(r * r));
   if (lane == 0) c.norms2[ch] = make_float2(t.h, t.l);
 }
 
@@ -740,22 +727,23 @@ __global__ void __launch_bounds__(kNT, 2) nb_persistent_kernel(NBCtx c, unsigned
   // rows that 16-byte loads cannot take: 41 of the 42 products read a packed copy
   float4* pack = (ld & 3) != 0 || (reinterpret_cast<uintptr_t>(X) & 15) != 0 ? c.pack : nullptr;
   float x[8][8];
+  const TileGeom g0 = tile_geom(b0 < c.ntiles ? b0 : 0), g1 = tile_geom(b0 + G < c.ntiles ? b0 + G : 0);
   if (RESIDENT) {
     if (b0 + G < c.ntiles) {
-      tile_load_x(X, ld, c.n, tile_geom(b0 + G), x);
+      tile_load_x(X, ld, c.n, g1, x);
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         xs[kNT * (2 * k) + threadIdx.x] = make_float4(x[k][0], x[k][1], x[k][2], x[k][3]);
         xs[kNT * (2 * k + 1) + threadIdx.x] = make_float4(x[k][4], x[k][5], x[k][6], x[k][7]);
       }
     }
-    if (b0 < c.ntiles) tile_load_x(X, ld, c.n, tile_geom(b0), x);
+    if (b0 < c.ntiles) tile_load_x(X, ld, c.n, g0, x);
   }
   int pass = 0;
   auto product = [&](auto stats) {
     constexpr bool kStats = decltype(stats)::value;
     if constexpr (RESIDENT)
-      ph_symv_resident<kStats>(c, b0, G, x, xs, sh);
+      ph_symv_resident<kStats>(c, b0, G, g0, g1, x, xs, sh);
     else
       ph_symv_run<kStats>(c, X, ld, pack, b0, G, (pass++ & 1) != 0, sh);
   };
@@ -774,7 +762,7 @@ __global__ void __launch_bounds__(kNT, 2) nb_persistent_kernel(NBCtx c, unsigned
       product(std::false_type{});
     NB_SYNC();
     if (j == 0 && b0 == 0 && threadIdx.x < 32) ph_fro(c);
-    double* u = c.zsave ? c.zsave + j * c.npad : c.u;
+    double* u = c.zsave ? c.zsave + j * c.npad : nullptr;
     for (int cp = b0; cp < npair; cp += G) ph_reduce_split(c, cp, u, sh);
     NB_SYNC();
     product(std::false_type{});
@@ -796,7 +784,7 @@ __global__ void __launch_bounds__(kNT, 2) nb_persistent_kernel(NBCtx c, unsigned
   NB_SYNC();
   product(std::false_type{});
   NB_SYNC();
-  for (int cp = b0; cp < npair; cp += G) ph_reduce_split(c, cp, c.u, sh);
+  for (int cp = b0; cp < npair; cp += G) ph_reduce_split(c, cp, nullptr, sh);
   NB_SYNC();
   product(std::false_type{});
   NB_SYNC();
@@ -965,11 +953,11 @@ size_t lanczos_bytes(int64_t n) {
   size_t b = 0;
   auto add = [&](size_t bytes) { b += (bytes + 255) / 256 * 256; };
   add(sizeof(double) * (kMaxSteps + 1) * npad);  // Qv
-  add(sizeof(double) * npad * 3);                // u, w, q
-  add(sizeof(float) * npad * 2);                 // vh, vl
+  add(sizeof(float2) * kMaxSteps * npad);        // Qf
+  add(sizeof(double) * npad * 2);                // w, q
+  add(sizeof(float) * npad);                     // vh
   add(sizeof(float2) * nb * npad * 2);           // P1, P2
   add(sizeof(float2) * npart * 32);              // dots
-  add(sizeof(float2) * npart * 32);              // dots2
   add(sizeof(double) * std::max(npart, nctas));  // norms
   add(sizeof(double) * ntiles);                  // tile_fro
   add(sizeof(unsigned) * 2);                     // grid barrier of the persistent kernel
@@ -992,18 +980,15 @@ void lanczos_carve(LanczosBufs& L, int64_t n, uint8_t* base) {
     return p;
   };
   L.Qv = reinterpret_cast<double*>(take(sizeof(double) * (kMaxSteps + 1) * L.npad));
-  double* v3 = reinterpret_cast<double*>(take(sizeof(double) * L.npad * 3));
-  L.u = v3;
-  L.w = v3 + L.npad;
-  L.q = v3 + 2 * L.npad;
-  float* f2 = reinterpret_cast<float*>(take(sizeof(float) * L.npad * 2));
-  L.vh = f2;
-  L.vl = f2 + L.npad;
+  L.Qf = reinterpret_cast<float2*>(take(sizeof(float2) * kMaxSteps * L.npad));
+  double* v2 = reinterpret_cast<double*>(take(sizeof(double) * L.npad * 2));
+  L.w = v2;
+  L.q = v2 + L.npad;
+  L.vh = reinterpret_cast<float*>(take(sizeof(float) * L.npad));
   float2* P = reinterpret_cast<float2*>(take(sizeof(float2) * L.nb * L.npad * 2));
   L.P1 = P;
   L.P2 = P + static_cast<int64_t>(L.nb) * L.npad;
   L.dots = reinterpret_cast<float2*>(take(sizeof(float2) * L.npart * 32));
-  L.dots2 = reinterpret_cast<float2*>(take(sizeof(float2) * L.npart * 32));
   L.norms = reinterpret_cast<double*>(take(sizeof(double) * std::max(L.npart, L.nvec_ctas)));
   L.tile_fro = reinterpret_cast<double*>(take(sizeof(double) * L.ntiles));
   L.sync = reinterpret_cast<unsigned*>(take(sizeof(unsigned) * 2));
@@ -1022,16 +1007,14 @@ NBCtx make_ctx(const LanczosBufs& L, const DevArgs* args, DevState* st) {
   c.args = args;
   c.st = st;
   c.Qv = L.Qv;
-  c.u = L.u;
   c.w = L.w;
   c.q = L.q;
   c.zsave = L.zsave;
   c.vh = L.vh;
-  c.vl = L.vl;
+  c.Qf = L.Qf;
   c.P1 = L.P1;
   c.P2 = L.P2;
   c.dots = L.dots;
-  c.dots2 = L.dots2;
   c.norms = L.norms;
   c.norms2 = reinterpret_cast<float2*>(L.norms);
   c.tile_fro = L.tile_fro;
@@ -1208,7 +1191,7 @@ cudaError_t enqueue_norm_bound(const LanczosBufs& L, const DevArgs* args, DevSta
     } else {
       nb_symv_kernel<false><<<c.ntiles, kNT, 0, s>>>(c, 1, pass++ & 1);
     }
-    double* u = L.zsave ? L.zsave + j * L.npad : L.u;
+    double* u = L.zsave ? L.zsave + j * L.npad : nullptr;
     nb_reduce_split_kernel<<<pb, kNT, 0, s>>>(c, u, 1);
     nb_symv_kernel<false><<<c.ntiles, kNT, 0, s>>>(c, 1, pass++ & 1);
     nb_reduce_dots_kernel<<<pb, kNT, 0, s>>>(c, j);
@@ -1220,7 +1203,7 @@ cudaError_t enqueue_norm_bound(const LanczosBufs& L, const DevArgs* args, DevSta
   // (after a breakdown the remaining steps' products do no work, so these two
   // may not continue the alternation; results do not depend on the direction)
   nb_symv_kernel<false><<<c.ntiles, kNT, 0, s>>>(c, 0, pass++ & 1);
-  nb_reduce_split_kernel<<<pb, kNT, 0, s>>>(c, L.u, 0);
+  nb_reduce_split_kernel<<<pb, kNT, 0, s>>>(c, nullptr, 0);
   nb_symv_kernel<false><<<c.ntiles, kNT, 0, s>>>(c, 0, pass++ & 1);
   nb_resid_kernel<<<pb, kNT, 0, s>>>(c);
   nb_final_kernel<<<1, 32, 0, s>>>(c);

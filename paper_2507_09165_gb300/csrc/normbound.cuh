@@ -31,12 +31,22 @@ __device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
   return F2{s, __fadd_rn(__fadd_rn(a.l, b.l), e)};
 }
 __device__ __forceinline__ double f2_to_d(F2 a) { return static_cast<double>(a.h) + static_cast<double>(a.l); }
-__device__ __forceinline__ void split_d(double v, float& h, float& l) {
-  h = __double2float_rn(v);
-  l = __double2float_rn(v - static_cast<double>(h));
-}
 __device__ __forceinline__ F2 shfl_xor_f2(F2 a, int m) {
   return F2{__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
+}
+
+// Normalised pair: h = RN(h + l).
+__device__ __forceinline__ F2 f2_norm(F2 a) {
+  const float s = __fadd_rn(a.h, a.l);
+  return F2{s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
+}
+// Product of two normalised pairs (Dekker's, with fma; error ~2^-47 relative).
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  const float p = __fmul_rn(a.h, b.h);
+  float e = fmaf(a.h, b.h, -p);
+  e = fmaf(a.h, b.l, e);
+  e = fmaf(a.l, b.h, e);
+  return F2{p, e};
 }
 
 // --------------------------------------------------------------- SplitMix64
@@ -58,17 +68,19 @@ __device__ __forceinline__ void tile_of(int t, int& bi, int& bj) {
   bi = t - j * (j + 1) / 2;
 }
 
-// Recursive-halving sum of cnt (<= 32) FP64 values over a warp; on return
-// lane l holds the warp total of value l.  Values live in v[0..31].
-__device__ __forceinline__ double warp_multi_sum(double (&v)[32], int lane) {
+// Recursive-halving sum of 32 double-float values over a warp; on return lane l
+// holds the warp total of value l.  The dot products of a chunk are formed and
+// added in FP32 pairs (~48 bits, what their partial sums are stored in): the
+// same sums in FP64 cost ~4,000 cycles per chunk on this GPU's FP64 unit.
+__device__ __forceinline__ F2 warp_multi_sum(F2 (&v)[32], int lane) {
 #pragma unroll
   for (int half = 16, m = 16; half >= 1; half >>= 1, m >>= 1) {
     const bool upper = (lane & m) != 0;
 #pragma unroll
     for (int i = 0; i < half; ++i) {
-      const double send = upper ? v[i] : v[i + half];
-      const double keep = upper ? v[i + half] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+      const F2 send = upper ? v[i] : v[i + half];
+      const F2 keep = upper ? v[i + half] : v[i];
+      v[i] = f2_add(keep, shfl_xor_f2(send, m));
     }
   }
   return v[0];
@@ -83,19 +95,28 @@ __device__ __forceinline__ double warp_multi_sum(double (&v)[32], int lane) {
 // ||X||_F^2 and max |X_ii|.
 struct TileGeom {
   int bi, bj, ib, jb;
-  bool diag;
+  bool diag;    // the tile lies on the diagonal
+  bool ondiag;  // the thread's block does
 };
-__device__ __forceinline__ TileGeom tile_geom(int t) {
+__device__ __forceinline__ TileGeom tile_geom_at(int bi, int bj) {
   TileGeom g;
-  tile_of(t, g.bi, g.bj);
+  g.bi = bi;
+  g.bj = bj;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   g.ib = g.bi * kSymvTile + 8 * (lane & 15);
   g.jb = g.bj * kSymvTile + 8 * (2 * warp + (lane >> 4));
   g.diag = g.bi == g.bj;
+  g.ondiag = g.ib == g.jb;
   return g;
 }
+__device__ __forceinline__ TileGeom tile_geom(int t) {
+  int bi, bj;
+  tile_of(t, bi, bj);
+  return tile_geom_at(bi, bj);
+}
 
-// The thread's 64 elements: 16 independent 16-byte loads of X in flight.
+// The thread's 64 elements: 16 independent 16-byte loads of X in flight; zeros
+// below the diagonal of a diagonal tile (those entries of X are not read for use).
 __device__ __forceinline__ void tile_load_x(const float* __restrict__ X, int64_t ld, int n, const TileGeom& g,
                                             float (&x)[8][8]) {
   const bool full = (g.ib + 7 < n) && (g.jb + 7 < n);
@@ -113,11 +134,20 @@ __device__ __forceinline__ void tile_load_x(const float* __restrict__ X, int64_t
       for (int k = 0; k < 8; ++k) x[c][k] = (g.jb + c < n && g.ib + k < n) ? __ldg(col + k) : 0.f;
     }
   }
+  if (g.diag) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (g.ib + k > g.jb + c) x[c][k] = 0.f;
+  }
 }
 
 // Per-thread row and column dot products of the 8 x 8 block (8-term FP32 FMA runs).
-// `col(c, x)` gives column c of the block.
-template <bool STATS, bool DIAG, class Col>
+// `col(c, x)` gives column c of the block (zeros below the diagonal).  Row sums
+// take i <= j, column sums i < j: only a block on the diagonal has elements
+// (c == k) that the two treat differently.
+template <bool STATS, class Col>
 __device__ __forceinline__ void tile_fma(int n, const TileGeom& g, const float (&vi)[8], const float (&vj)[8],
                                          const Col& col, float (&rsum)[8], float (&csum)[8], float& fro,
                                          unsigned& mdiag) {
@@ -132,13 +162,8 @@ __device__ __forceinline__ void tile_fma(int n, const TileGeom& g, const float (
     csum[c] = 0.f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      float xr = x[k], xc = x[k];
-      if (DIAG) {
-        const int i = g.ib + k, j = g.jb + c;
-        xr = (i <= j) ? xr : 0.f;
-        xc = (i < j) ? xc : 0.f;
-        if (STATS && i == j && i < n) mdiag = max(mdiag, __float_as_uint(fabsf(x[k])));
-      }
+      const float xr = x[k], xc = (k == c && g.ondiag) ? 0.f : x[k];
+      if (STATS && k == c && g.ondiag && g.ib + k < n) mdiag = max(mdiag, __float_as_uint(fabsf(x[k])));
       rsum[k] = fmaf(xr, vj[c], rsum[k]);
       csum[c] = fmaf(xc, vi[k], csum[c]);
       if (STATS) fro = fmaf(xr, xc + xr, fro);  // x^2 on the diagonal, 2 x^2 above it
@@ -155,11 +180,12 @@ __device__ __forceinline__ void tile_fma_reg(int n, const TileGeom& g, const flo
 #pragma unroll
     for (int k = 0; k < 8; ++k) o[k] = x[c][k];
   };
-  if (g.diag)
-    tile_fma<STATS, true>(n, g, vi, vj, col, rsum, csum, fro, mdiag);
-  else
-    tile_fma<STATS, false>(n, g, vi, vj, col, rsum, csum, fro, mdiag);
+  tile_fma<STATS>(n, g, vi, vj, col, rsum, csum, fro, mdiag);
 }
+
+// The warps' row sums lie at red[warp][17 k + tr] for row 8 tr + k: the stores (a
+// half-warp along tr) and the reads (a warp along k and tr) spread over the banks.
+constexpr int kRedStride = 8 * 17;
 
 // Combines the threads' sums in a fixed order (double-float) into the tile's
 // row partials (sink.row(i, v): row i's dot product with this tile) and column
@@ -171,7 +197,7 @@ __device__ __forceinline__ void tile_fma_reg(int n, const TileGeom& g, const flo
 // (and so finished reading it); the run is followed by a CTA barrier.
 template <bool STATS, class Sink>
 __device__ __forceinline__ void tile_reduce(int n, const TileGeom& g, const float (&rsum)[8], const float (&csum)[8],
-                                            float fro, unsigned mdiag, float2 (*red)[kSymvTile], double* fro_sh,
+                                            float fro, unsigned mdiag, float2 (*red)[kRedStride], double* fro_sh,
                                             const Sink& sink, bool sync_after) {
   const int i0 = g.bi * kSymvTile;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -188,7 +214,7 @@ __device__ __forceinline__ void tile_reduce(int n, const TileGeom& g, const floa
   }
   if (lane < 16) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) red[warp][8 * tr + k] = make_float2(rs[k].h, rs[k].l);
+    for (int k = 0; k < 8; ++k) red[warp][17 * k + tr] = make_float2(rs[k].h, rs[k].l);
   }
   // columns: recursive halving over the 16 row groups of a half-warp
 #pragma unroll
@@ -210,9 +236,15 @@ __device__ __forceinline__ void tile_reduce(int n, const TileGeom& g, const floa
   __syncthreads();
   if (threadIdx.x < kSymvTile) {
     const int r = threadIdx.x;
-    F2 a{red[0][r].x, red[0][r].y};
+    const int at = 17 * (r & 7) + (r >> 3);
+    F2 p[8];
 #pragma unroll
-    for (int w = 1; w < 8; ++w) a = f2_add(a, F2{red[w][r].x, red[w][r].y});
+    for (int w = 0; w < 8; ++w) p[w] = F2{red[w][at].x, red[w][at].y};
+#pragma unroll
+    for (int h = 1; h < 8; h *= 2)
+#pragma unroll
+      for (int w = 0; w < 8; w += 2 * h) p[w] = f2_add(p[w], p[w + h]);
+    const F2 a = p[0];
     if (i0 + r < n) sink.row(i0 + r, make_float2(a.h, a.l));
   }
   if (STATS) {
@@ -238,18 +270,19 @@ __device__ __forceinline__ float2 d_to_f2(double v) {
   return make_float2(h, __double2float_rn(v - static_cast<double>(h)));
 }
 
-// Warp sum of one FP64 value per lane as a double-float pair (fixed order;
-// every lane): FP32 shuffles and adds, this GPU's FP64 adds being far slower.
-__device__ __forceinline__ F2 warp_sum_f2(double v) {
+// Warp sum of one double-float value per lane (fixed order; every lane).
+__device__ __forceinline__ F2 warp_sum_f2(F2 t) {
   const int lane = threadIdx.x & 31;
-  const float2 p = d_to_f2(v);
-  F2 t{p.x, p.y};
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const F2 other = shfl_xor_f2(t, o);
     t = (lane & o) ? f2_add(other, t) : f2_add(t, other);
   }
   return t;
+}
+__device__ __forceinline__ F2 f2_of(double v) {
+  const float2 p = d_to_f2(v);
+  return F2{p.x, p.y};
 }
 
 // Loads of the double-float partials: through L2 (vectors other CTAs wrote), or plain (shared memory).
@@ -284,34 +317,88 @@ __device__ __forceinline__ double warp_sum_chunks(const float2* part, int nch, c
   return f2_to_d(acc);
 }
 
-// S[k] = sum over the chunks of part[k * nch + ch] (slot-major: a warp's 32
-// lanes read 256 contiguous bytes) for the slots k with (want >> k) & 1,
-// double-float in a fixed order (lanes stride over the chunks, then a
-// butterfly), into shared memory as FP64.  Warp w takes the slots k = w,
-// w + 8, ...  The loads of a lane are issued 8 at a time.
+// S[k] = sum over the chunks of part[k * stride + ch] (slot-major: a warp's 32
+// lanes read 256 contiguous bytes) for the slots k <= j and 31, double-float in a
+// fixed order (lanes stride over the chunks, then a butterfly), into shared
+// memory.  Warp w takes the slots w, w + 8, w + 16, w + 24 together: four
+// independent chains of loads and adds.
 template <class Load>
-__device__ __forceinline__ void chunk_sums(const float2* part, int nch, uint32_t want, double* S, const Load& load) {
+__device__ __forceinline__ void chunk_sums(const float2* part, int nch, int stride, int j, float2* S, const Load& load) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int k = w; k < 32; k += kNT / 32) {
-    if (!((want >> k) & 1u)) continue;
-    F2 acc{0.f, 0.f};
-    for (int c0 = 0; c0 < nch; c0 += 8 * 32) {
-      float2 t[8];
+  F2 acc[4];
+  bool use[4];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int ch = c0 + 32 * i + lane;
-        t[i] = ch < nch ? load(part + static_cast<int64_t>(k) * nch + ch) : make_float2(0.f, 0.f);
+  for (int i = 0; i < 4; ++i) {
+    const int k = w + 8 * i;
+    use[i] = k <= j || k == 31;
+    acc[i] = F2{0.f, 0.f};
+  }
+  for (int c0 = 0; c0 < nch; c0 += 2 * 32) {
+    float2 t[4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int ch = c0 + 32 * q + lane;
+        t[i][q] = use[i] && ch < nch ? load(part + static_cast<int64_t>(w + 8 * i) * stride + ch) : make_float2(0.f, 0.f);
       }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) acc = f2_add(acc, F2{t[i].x, t[i].y});
-    }
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const F2 other = shfl_xor_f2(acc, o);
-      acc = (lane & o) ? f2_add(other, acc) : f2_add(acc, other);
-    }
-    if (lane == 0) S[k] = f2_to_d(acc);
+      for (int q = 0; q < 2; ++q) acc[i] = f2_add(acc[i], F2{t[i][q].x, t[i][q].y});
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const F2 other = shfl_xor_f2(acc[i], o);
+      acc[i] = (lane & o) ? f2_add(other, acc[i]) : f2_add(acc[i], other);
+    }
+  if (lane == 0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (use[i]) S[w + 8 * i] = make_float2(acc[i].h, acc[i].l);
+  }
+}
+
+// beta_j = sqrt(b2) and its reciprocal (one rsqrt in place of a square root and a division).
+__device__ __forceinline__ void lanczos_beta(double b2, double& beta, double& inv) {
+  inv = rsqrt(b2);
+  beta = b2 > 0.0 ? b2 * inv : (b2 <= 0.0 ? 0.0 : b2);  // NaN stays NaN
+}
+// beta_j and 1 / beta_j from the summed dots S (one warp; lane 0 writes): beta^2 =
+// ||w'||^2 - ||h||^2, the difference in double-float.
+__device__ __forceinline__ void beta_of_sums(const float2* S, int j, double* out) {
+  const int lane = threadIdx.x & 31;
+  F2 q{0.f, 0.f};
+  if (lane <= j) {
+    const F2 s = f2_norm(F2{S[lane].x, S[lane].y});
+    q = f2_mul(s, s);
+  }
+  q = warp_sum_f2(q);
+  if (lane == 0) {
+    const F2 d = f2_add(F2{S[31].x, S[31].y}, F2{-q.h, -q.l});
+    double b, inv;
+    lanczos_beta(f2_to_d(d), b, inv);
+    out[0] = b;
+    out[1] = inv;
+  }
+}
+
+// The dot products of a chunk's element w' (lane = element) with the Lanczos
+// vectors q_k, k <= j (q[k]: double-float), and ||w'||^2 in slot 31: lane l returns
+// slot l's sum over the chunk.
+template <class LoadQ>
+__device__ __forceinline__ float2 chunk_dots(F2 w, int j, const LoadQ& q) {
+  F2 v[32];
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    v[k] = F2{0.f, 0.f};
+    if (k < kMaxSteps && k <= j) v[k] = f2_mul(q(k), w);
+  }
+  v[31] = f2_mul(w, w);
+  const F2 s = warp_multi_sum(v, threadIdx.x & 31);
+  return make_float2(s.h, s.l);
 }
 
 // Vector elements of a Lanczos step (one lane = one element).
@@ -320,18 +407,15 @@ __device__ __forceinline__ double lanczos_recur(double w, double alpha, double q
   return fma(-beta, qp, fma(-alpha, qj, w));
 }
 // w'' = w' - sum_{k <= j} h_k q_k in four independent chains (an FP64
-// operation's latency is 64 cycles).
-__device__ __forceinline__ double lanczos_orth(double w, const double* hk, const double (&qk)[kMaxSteps], int j) {
+// operation's latency is 64 cycles).  h: h_k in lane k (one conversion to FP64
+// per warp; done by the warps that sum the slots it was 32 of them, on a unit
+// that issues one every ~19 cycles).
+__device__ __forceinline__ double lanczos_orth(double w, double h, const double (&qk)[kMaxSteps], int j) {
   double a[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
   for (int k = 0; k < kMaxSteps; ++k)
-    if (k <= j) a[k & 3] = fma(hk[k], qk[k], a[k & 3]);
+    if (k <= j) a[k & 3] = fma(__shfl_sync(0xffffffffu, h, k), qk[k], a[k & 3]);
   return w - ((a[0] + a[1]) + (a[2] + a[3]));
-}
-// beta_j = sqrt(b2) and its reciprocal (one rsqrt in place of a square root and a division).
-__device__ __forceinline__ void lanczos_beta(double b2, double& beta, double& inv) {
-  inv = rsqrt(b2);
-  beta = b2 > 0.0 ? b2 * inv : (b2 <= 0.0 ? 0.0 : b2);  // NaN stays NaN
 }
 // sum_k y_k q_k, k < m.
 __device__ __forceinline__ double lanczos_ritz(const double (&yk)[kMaxSteps], const double (&qk)[kMaxSteps], int m) {

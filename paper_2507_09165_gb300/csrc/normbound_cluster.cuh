@@ -34,11 +34,14 @@ __host__ __device__ constexpr int cluster_round16(int b) { return (b + 15) / 16 
 // Shared memory of a CTA, carved in this order.
 struct ClusterSmem {
   float4* xs;        // extra x 64 KB
-  float2 (*red)[8][kSymvTile];  // 2 buffers
+  float2 (*red)[8][kRedStride];  // 2 buffers
   double* Q;         // own x kMaxSteps x 32
+  float2* Qf;        // the same as double-float pairs
   double* w;         // own x 32
   double* fro;       // per tile (every CTA has all of them)
-  double *h, *alpha, *beta, *y;
+  double *alpha, *beta, *y;
+  float2* hs;        // the summed dots as pairs
+  int2* geo;         // (bi, bj) of the CTA's tiles
   double* norms;     // per 256-element block (start vector)
   double* bs;        // block_sum64
   double* scalar;    // 4
@@ -61,11 +64,13 @@ __host__ __device__ inline int cluster_carve(ClusterSmem* s, uint8_t* base, int 
   const int nch = 4 * nbmax, ntl = nbmax * (nbmax + 1) / 2, ds = nch | 1;
   ClusterSmem t;
   t.xs = reinterpret_cast<float4*>(take(extra * 4 * kSymvTile * kSymvTile));
-  t.red = reinterpret_cast<float2(*)[8][kSymvTile]>(take(2 * 8 * kSymvTile * 8));
+  t.red = reinterpret_cast<float2(*)[8][kRedStride]>(take(2 * 8 * kRedStride * 8));
   t.Q = reinterpret_cast<double*>(take(own * kMaxSteps * 32 * 8));
+  t.Qf = reinterpret_cast<float2*>(take(own * kMaxSteps * 32 * 8));
   t.w = reinterpret_cast<double*>(take(own * 32 * 8));
   t.fro = reinterpret_cast<double*>(take(ntl * 8));
-  t.h = reinterpret_cast<double*>(take(32 * 8));
+  t.hs = reinterpret_cast<float2*>(take(32 * 8));
+  t.geo = reinterpret_cast<int2*>(take((kClusterMaxExtra + 1) * 8));
   t.alpha = reinterpret_cast<double*>(take(kMaxSteps * 8));
   t.beta = reinterpret_cast<double*>(take(kMaxSteps * 8));
   t.y = reinterpret_cast<double*>(take(kMaxSteps * 8));
@@ -85,16 +90,15 @@ __host__ __device__ inline int cluster_carve(ClusterSmem* s, uint8_t* base, int 
   return off;
 }
 
-// Stores to the same place in CTA `rank` of the cluster.
-__device__ __forceinline__ void st_remote(float* p, uint32_t rank, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(mapa_shared(smem_u32(p), rank)), "f"(v) : "memory");
+// Stores to the same place (shared address `a` of this CTA) in CTA `rank` of the cluster.
+__device__ __forceinline__ void st_remote(uint32_t a, uint32_t rank, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(mapa_shared(a, rank)), "f"(v) : "memory");
 }
-__device__ __forceinline__ void st_remote(float2* p, uint32_t rank, float2 v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(mapa_shared(smem_u32(p), rank)), "f"(v.x), "f"(v.y)
-               : "memory");
+__device__ __forceinline__ void st_remote(uint32_t a, uint32_t rank, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(mapa_shared(a, rank)), "f"(v.x), "f"(v.y) : "memory");
 }
-__device__ __forceinline__ void st_remote(double* p, uint32_t rank, double v) {
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(mapa_shared(smem_u32(p), rank)), "d"(v) : "memory");
+__device__ __forceinline__ void st_remote(uint32_t a, uint32_t rank, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(mapa_shared(a, rank)), "d"(v) : "memory");
 }
 __device__ __forceinline__ unsigned ld_remote(const unsigned* p, uint32_t rank) {
   unsigned v;
@@ -107,16 +111,16 @@ __device__ __forceinline__ unsigned ld_remote(const unsigned* p, uint32_t rank) 
 struct ClusterSink {
   const ClusterSmem& s;
   const TileGeom& g;
-  int tile, csize, nbmax;
+  int tile, csize, clog, nbmax;  // csize = 2^clog
   __device__ __forceinline__ void put(int i, int slot, float2 v) const {
     const int ch = i >> 5;
-    st_remote(s.part + (ch / csize * (nbmax + 1) + slot) * 32 + (i & 31), ch % csize, v);
+    st_remote(smem_u32(s.part + ((ch >> clog) * (nbmax + 1) + slot) * 32 + (i & 31)), ch & (csize - 1), v);
   }
   __device__ __forceinline__ void row(int i, float2 v) const { put(i, g.bj + 1, v); }
   __device__ __forceinline__ void col(int j, float2 v) const { put(j, g.bi, v); }
   __device__ __forceinline__ void diag(unsigned m) const { atomicMax(s.mdiag, m); }
   __device__ __forceinline__ void fro(double f) const {
-    for (int r = 0; r < csize; ++r) st_remote(s.fro + tile, r, f);
+    for (int r = 0; r < csize; ++r) st_remote(smem_u32(s.fro + tile), r, f);
   }
 };
 
@@ -127,7 +131,7 @@ __device__ __forceinline__ void cl_product(const ClusterSmem& s, int n, int ntil
                                            const float (&x)[8][8]) {
   int buf = 0;
   for (int t = rank, i = 0; t < ntiles; t += csize, ++i, buf ^= 1) {
-    const TileGeom g = tile_geom(t);
+    const TileGeom g = tile_geom_at(s.geo[i].x, s.geo[i].y);
     float vi[8], vj[8], rsum[8], csum[8], fro;
     unsigned mdiag;
 #pragma unroll
@@ -146,19 +150,16 @@ __device__ __forceinline__ void cl_product(const ClusterSmem& s, int n, int ntil
         o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
         o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
       };
-      if (g.diag)
-        tile_fma<STATS, true>(n, g, vi, vj, col, rsum, csum, fro, mdiag);
-      else
-        tile_fma<STATS, false>(n, g, vi, vj, col, rsum, csum, fro, mdiag);
+      tile_fma<STATS>(n, g, vi, vj, col, rsum, csum, fro, mdiag);
     }
-    tile_reduce<STATS>(n, g, rsum, csum, fro, mdiag, s.red[buf], s.bs, ClusterSink{s, g, t, csize, nbmax}, false);
+    tile_reduce<STATS>(n, g, rsum, csum, fro, mdiag, s.red[buf], s.bs, ClusterSink{s, g, t, csize, 31 - __clz(csize), nbmax}, false);
   }
 }
 
 // y of own chunk `o` (global chunk o C + rank) by the four warps of this half
 // of the CTA, in reduce_partials' order; the half's first warp receives it.
 // Both halves call it together (CTA barriers).
-__device__ __forceinline__ double cl_reduce(const ClusterSmem& s, int n, int nb, int o, int nown, int e, int nbmax) {
+__device__ __forceinline__ F2 cl_reduce(const ClusterSmem& s, int n, int nb, int o, int nown, int e, int nbmax) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, hw = w & 3;
   F2 a{0.f, 0.f}, d{0.f, 0.f};
   if (o < nown && e < n) {
@@ -170,12 +171,12 @@ __device__ __forceinline__ double cl_reduce(const ClusterSmem& s, int n, int nb,
   const F2 t = f2_add(a, d);
   s.stg[w * 32 + lane] = make_float2(t.h, t.l);
   __syncthreads();
-  double y = 0.0;
+  F2 y{0.f, 0.f};
   if (hw == 0) {
     F2 acc{s.stg[w * 32 + lane].x, s.stg[w * 32 + lane].y};
 #pragma unroll
     for (int q = 1; q < 4; ++q) acc = f2_add(acc, F2{s.stg[(w + q) * 32 + lane].x, s.stg[(w + q) * 32 + lane].y});
-    y = f2_to_d(acc);
+    y = f2_norm(acc);
   }
   __syncthreads();
   return y;
@@ -199,10 +200,17 @@ __global__ void __launch_bounds__(kNT, 2) nb_cluster_kernel(const ClusterJob jb)
   const bool lead = half_lead_warp();
   auto elem_of = [&](int o) { return (o * C + rank) * 32 + lane; };
 
+  auto put_q = [&](int o, int k, double q) {
+    s.Q[(o * kMaxSteps + k) * 32 + lane] = q;
+    s.Qf[(o * kMaxSteps + k) * 32 + lane] = d_to_f2(q);
+  };
+
   // tiles: the extra ones into shared memory, the first into registers
   float x[8][8];
   for (int t = rank + C, i = 0; t < ntiles; t += C, ++i) {
-    tile_load_x(X, ld, n, tile_geom(t), x);
+    const TileGeom g = tile_geom(t);
+    if (tid == 0) s.geo[i + 1] = make_int2(g.bi, g.bj);
+    tile_load_x(X, ld, n, g, x);
     float4* xt = s.xs + i * 16 * kNT;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -210,7 +218,11 @@ __global__ void __launch_bounds__(kNT, 2) nb_cluster_kernel(const ClusterJob jb)
       xt[kNT * (2 * k + 1) + tid] = make_float4(x[k][4], x[k][5], x[k][6], x[k][7]);
     }
   }
-  if (rank < ntiles) tile_load_x(X, ld, n, tile_geom(rank), x);
+  if (rank < ntiles) {
+    const TileGeom g = tile_geom(rank);
+    if (tid == 0) s.geo[0] = make_int2(g.bi, g.bj);
+    tile_load_x(X, ld, n, g, x);
+  }
 
   // start vector: every CTA forms all of it (no communication)
   for (int vb = 0; vb < nv; ++vb) {
@@ -235,30 +247,32 @@ __global__ void __launch_bounds__(kNT, 2) nb_cluster_kernel(const ClusterJob jb)
     for (int o = wp; o < nown; o += kNT / 32) {
       const int e = elem_of(o);
       const double q = e < n ? lanczos_start(e) * inv : 0.0;
-      s.Q[o * kMaxSteps * 32 + lane] = q;
+      put_q(o, 0, q);
       if (jb.zsave && e < n) jb.Qv[e] = q;
     }
   }
   cluster_sync_all();  // every CTA of the cluster runs before any remote store
 
-  // stores an element of the mat-vec input of own chunk o to every CTA
-  auto put_vh = [&](int e, double v) {
-    const float h = e < n ? __double2float_rn(v) : 0.f;
-    for (int r = 0; r < C; ++r) st_remote(s.vh + e, r, h);
+  // an element of the mat-vec input (0 past n) to every CTA
+  auto put_vh = [&](int e, float h) {
+    const uint32_t a = smem_u32(s.vh + e);
+    if (e >= n) h = 0.f;
+#pragma unroll 4
+    for (int r = 0; r < C; ++r) st_remote(a, r, h);
   };
   // a double-float partial of chunk ch to every CTA
   auto put_norm2 = [&](int ch, const F2& t) {
-    if (lane < C) st_remote(s.norms2 + ch, lane, make_float2(t.h, t.l));
+    if (lane < C) st_remote(smem_u32(s.norms2 + ch), lane, make_float2(t.h, t.l));
   };
   // u = X v: split for the second product, the chunks' shares of ||u||^2
   auto reduce_split = [&](double* u) {
     for (int it = 0; it < nit; ++it) {
       const int o = 2 * it + half, e = elem_of(o);
-      const double y = cl_reduce(s, n, nb, o, nown, e, nbmax);
+      const F2 y = cl_reduce(s, n, nb, o, nown, e, nbmax);
       if (lead && o < nown) {
-        put_vh(e, y);
-        if (u && e < n) u[e] = y;
-        put_norm2(o * C + rank, warp_sum_f2(e < n ? y * y : 0.0));
+        put_vh(e, y.h);
+        if (u && e < n) u[e] = f2_to_d(y);
+        put_norm2(o * C + rank, warp_sum_f2(f2_mul(y, y)));
       }
     }
   };
@@ -282,58 +296,44 @@ __global__ void __launch_bounds__(kNT, 2) nb_cluster_kernel(const ClusterJob jb)
     cluster_sync_all();
     cl_product<false>(s, n, ntiles, rank, C, nbmax, x);
     cluster_sync_all();
-    // w = X u, w' and its dots (ph_reduce_dots)
+    // w = X u, w' and its dots (ph_reduce_dots); alpha_j by a warp that only helps to reduce
+    if (wp == 1) {
+      const double a = warp_sum_chunks(s.norms2, nch, LoadPlain());
+      if (lane == 0) s.scalar[3] = a;
+    }
+    if (nit == 0) __syncthreads();
     for (int it = 0; it < nit; ++it) {
       const int o = 2 * it + half, e = elem_of(o);
-      double y = cl_reduce(s, n, nb, o, nown, e, nbmax);
+      const F2 y = cl_reduce(s, n, nb, o, nown, e, nbmax);
       if (!(lead && o < nown)) continue;
-      const double alpha = warp_sum_chunks(s.norms2, nch, LoadPlain());
+      const double alpha = s.scalar[3];  // published by cl_reduce's barriers
       const double* Qo = s.Q + o * kMaxSteps * 32 + lane;
-      const double qj = Qo[j * 32], qp = j > 0 ? Qo[(j - 1) * 32] : 0.0;
-      y = lanczos_recur(y, alpha, qj, j > 0 ? s.beta[j - 1] : 0.0, qp);
-      s.w[o * 32 + lane] = y;
-      double v[32];
-#pragma unroll
-      for (int k = 0; k < 32; ++k) v[k] = k < kMaxSteps && k <= j ? Qo[(k < kMaxSteps ? k : 0) * 32] * y : 0.0;
-      v[31] = e < n ? y * y : 0.0;
-      const float2 d = d_to_f2(warp_multi_sum(v, lane));
-      for (int r = 0; r < C; ++r) st_remote(s.dots + lane * s.dstride + o * C + rank, r, d);
+      const float2* Qfo = s.Qf + o * kMaxSteps * 32 + lane;
+      const double w = lanczos_recur(f2_to_d(y), alpha, Qo[j * 32], j > 0 ? s.beta[j - 1] : 0.0,
+                                     j > 0 ? Qo[(j - 1) * 32] : 0.0);
+      s.w[o * 32 + lane] = w;
+      const float2 d = chunk_dots(f2_of(e < n ? w : 0.0), j, [&](int k) { return F2{Qfo[k * 32].x, Qfo[k * 32].y}; });
+      const uint32_t a = smem_u32(s.dots + lane * s.dstride + o * C + rank);
+#pragma unroll 4
+      for (int r = 0; r < C; ++r) st_remote(a, r, d);
     }
     cluster_sync_all();
     // Gram-Schmidt pass and q_{j+1} (ph_orth_next)
-    for (int k = wp; k < 32; k += kNT / 32) {
-      if (k > j && k != 31) continue;
-      const float2* p = s.dots + k * s.dstride;
-      F2 acc{0.f, 0.f};
-      for (int ch = lane; ch < nch; ch += 32) acc = f2_add(acc, F2{p[ch].x, p[ch].y});
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const F2 other = shfl_xor_f2(acc, o);
-        acc = (lane & o) ? f2_add(other, acc) : f2_add(acc, other);
-      }
-      if (lane == 0) s.h[k] = f2_to_d(acc);
-    }
+    chunk_sums(s.dots, nch, s.dstride, j, s.hs, LoadPlain());
     __syncthreads();
     if (wp == 7) {
-      double h2 = lane <= j ? s.h[lane] * s.h[lane] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) h2 += __shfl_xor_sync(0xffffffffu, h2, o);
-      if (lane == 0) {
-        double bt, inv;
-        lanczos_beta(s.h[31] - h2, bt, inv);
-        s.scalar[0] = bt;
-        s.scalar[1] = inv;
-      }
+      beta_of_sums(s.hs, j, s.scalar);
     } else if (wp == 6) {
-      const double alpha = warp_sum_chunks(s.norms2, nch, LoadPlain());
-      if (lane == 0) s.alpha[j] = alpha + s.h[j];
+      const double alpha = s.scalar[3];
+      if (lane == 0) s.alpha[j] = alpha + f2_to_d(F2{s.hs[j].x, s.hs[j].y});
     }
+    const double h = wp < nown && lane <= j ? f2_to_d(F2{s.hs[lane].x, s.hs[lane].y}) : 0.0;
     double wo[2] = {0.0, 0.0};  // own chunks wp, wp + 8 (at most 16 chunks a CTA)
     auto next = [&](int o) {
       double qk[kMaxSteps];
 #pragma unroll
       for (int k = 0; k < kMaxSteps; ++k) qk[k] = k <= j ? s.Q[(o * kMaxSteps + k) * 32 + lane] : 0.0;
-      return lanczos_orth(s.w[o * 32 + lane], s.h, qk, j);
+      return lanczos_orth(s.w[o * 32 + lane], h, qk, j);
     };
     if (wp < nown) wo[0] = next(wp);
     if (wp + 8 < nown) wo[1] = next(wp + 8);
@@ -349,9 +349,9 @@ __global__ void __launch_bounds__(kNT, 2) nb_cluster_kernel(const ClusterJob jb)
       if (o < nown) {
         const int e = elem_of(o);
         const double q = wo[i] * inv;
-        s.Q[(o * kMaxSteps + j + 1) * 32 + lane] = q;
+        put_q(o, j + 1, q);
         if (jb.zsave && e < n) jb.Qv[static_cast<int64_t>(j + 1) * jb.npad + e] = q;
-        put_vh(e, q);
+        put_vh(e, __double2float_rn(q));
       }
     }
     cluster_sync_all();
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(kNT, 2) nb_cluster_kernel(const ClusterJob jb)
         yk[k] = k < m ? s.y[k] : 0.0;
       }
       ro[i] = e < n ? lanczos_ritz(yk, qk, m) : 0.0;
-      put_norm2(o * C + rank, warp_sum_f2(ro[i] * ro[i]));
+      put_norm2(o * C + rank, warp_sum_f2(f2_of(ro[i] * ro[i])));
     }
   }
   cluster_sync_all();
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(kNT, 2) nb_cluster_kernel(const ClusterJob jb)
       if (o < nown) {
         const double q = ro[i] * inv;
         s.w[o * 32 + lane] = q;
-        put_vh(elem_of(o), q);
+        put_vh(elem_of(o), __double2float_rn(q));
       }
     }
   }
@@ -403,10 +403,10 @@ __global__ void __launch_bounds__(kNT, 2) nb_cluster_kernel(const ClusterJob jb)
   cluster_sync_all();
   for (int it = 0; it < nit; ++it) {
     const int o = 2 * it + half, e = elem_of(o);
-    const double y = cl_reduce(s, n, nb, o, nown, e, nbmax);
+    const F2 y = cl_reduce(s, n, nb, o, nown, e, nbmax);
     if (!(lead && o < nown)) continue;
-    const double r = e < n ? y - sigma * s.w[o * 32 + lane] : 0.0;
-    put_norm2(o * C + rank, warp_sum_f2(r * r));
+    const double r = e < n ? fma(-sigma, s.w[o * 32 + lane], f2_to_d(y)) : 0.0;
+    put_norm2(o * C + rank, warp_sum_f2(f2_of(r * r)));
   }
   cluster_sync_all();
   if (rank == 0 && wp == 0) {

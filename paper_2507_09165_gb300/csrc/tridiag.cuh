@@ -24,11 +24,14 @@ namespace psd {
 
 // Number of eigenvalues of the unit-scaled T below x: sign changes of the
 // leading minors p_k = (a_k - x) p_{k-1} - b_{k-1}^2 p_{k-2} (no divisions;
-// rescaled when they grow).
+// rescaled when they grow).  M > 0: the order, known at compile time.
+template <int M>
 __device__ __forceinline__ int sturm_count32(const float* a, const float* b, int m, float x) {
+  const int mm = M > 0 ? M : m;
   float pm = 1.f, p = a[0] - x;
   int cnt = (p < 0.f) ? 1 : 0;
-  for (int k = 1; k < m; ++k) {
+#pragma unroll
+  for (int k = 1; k < mm; ++k) {
     const float pn = (a[k] - x) * p - b[k - 1] * b[k - 1] * pm;
     const bool change = (pn == 0.f) ? (p > 0.f) : ((pn < 0.f) != (p < 0.f));
     if (p != 0.f || pn != 0.f) cnt += change ? 1 : 0;
@@ -40,6 +43,84 @@ __device__ __forceinline__ int sturm_count32(const float* a, const float* b, int
     }
   }
   return cnt;
+}
+
+// Inverse iteration on (T - s I) by one thread: Gaussian elimination with
+// partial pivoting on the tridiagonal (a row swap adds a second super-diagonal),
+// three solves.  M > 0: the order, known at compile time -- every array then
+// stays in registers (with run-time bounds they live in local memory, which made
+// the whole eigenpair 25 us instead of ~10).
+template <int M>
+__device__ __forceinline__ void inverse_iterate(const float* a32, const float* b32, int m, float s, double* y) {
+  const int mm = M > 0 ? M : m;
+  const float tiny = 1e-30f;
+  float d[kMaxSteps], du[kMaxSteps], du2[kMaxSteps], l[kMaxSteps], rd[kMaxSteps], v[kMaxSteps];
+  bool piv[kMaxSteps];
+#pragma unroll
+  for (int k = 0; k < mm; ++k) {
+    d[k] = a32[k] - s;
+    du[k] = k < mm - 1 ? b32[k] : 0.f;
+    du2[k] = 0.f;
+    piv[k] = false;
+  }
+#pragma unroll
+  for (int k = 0; k < mm - 1; ++k) {
+    const float dl = b32[k];
+    if (fabsf(d[k]) >= fabsf(dl)) {
+      if (d[k] == 0.f) d[k] = tiny;
+      l[k] = dl / d[k];
+      d[k + 1] -= l[k] * du[k];
+    } else {
+      piv[k] = true;
+      l[k] = d[k] / dl;
+      d[k] = dl;
+      const float t = d[k + 1];
+      d[k + 1] = du[k] - l[k] * t;
+      du[k] = t;
+      if (k < mm - 2) {
+        du2[k] = du[k + 1];
+        du[k + 1] = -l[k] * du[k + 1];
+      }
+    }
+  }
+  if (mm > 0 && d[mm - 1] == 0.f) d[mm - 1] = tiny;
+#pragma unroll
+  for (int k = 0; k < mm; ++k) rd[k] = 1.f / d[k];
+#pragma unroll
+  for (int k = 0; k < mm; ++k) v[k] = 1.f;
+#pragma unroll 1
+  for (int it = 0; it < 3; ++it) {
+#pragma unroll
+    for (int k = 0; k < mm - 1; ++k) {
+      if (piv[k]) {
+        const float t = v[k];
+        v[k] = v[k + 1];
+        v[k + 1] = t - l[k] * v[k];
+      } else {
+        v[k + 1] -= l[k] * v[k];
+      }
+    }
+#pragma unroll
+    for (int k = mm - 1; k >= 0; --k) {
+      float acc = v[k];
+      if (k + 1 < mm) acc -= du[k] * v[k + 1];
+      if (k + 2 < mm) acc -= du2[k] * v[k + 2];
+      v[k] = acc * rd[k];
+    }
+    float mx = 0.f;
+#pragma unroll
+    for (int k = 0; k < mm; ++k) mx = fmaxf(mx, fabsf(v[k]));
+    if (!(mx > 0.f) || !isfinite(mx)) {
+#pragma unroll
+      for (int k = 0; k < mm; ++k) v[k] = k == 0 ? 1.f : 0.f;
+      break;
+    }
+    const float r = 1.f / mx;  // max-norm scaling keeps the iterate in range
+#pragma unroll
+    for (int k = 0; k < mm; ++k) v[k] *= r;
+  }
+#pragma unroll
+  for (int k = 0; k < kMaxSteps; ++k) y[k] = k < mm ? static_cast<double>(v[k]) : 0.0;
 }
 
 // Call with the 32 lanes of one warp.  a32, b32: shared scratch of kMaxSteps
@@ -86,7 +167,8 @@ __device__ __forceinline__ double tridiag_top_eig(const double* alpha, const dou
     if (!(hi - lo > 4.f * 1.2e-7f * fmaxf(fabsf(lo), fabsf(hi)))) break;
     const float w = (hi - lo) * (1.f / 33.f);
     const float x = lo + w * static_cast<float>(lane + 1);
-    const unsigned mask = __ballot_sync(0xffffffffu, sturm_count32(a32, b32, m, x) >= m);
+    const int below = m == kMaxSteps ? sturm_count32<kMaxSteps>(a32, b32, m, x) : sturm_count32<0>(a32, b32, m, x);
+    const unsigned mask = __ballot_sync(0xffffffffu, below >= m);
     const int first = mask ? __ffs(mask) - 1 : 32;
     const float nlo = first == 0 ? lo : lo + w * static_cast<float>(first);
     const float nhi = first == 32 ? hi : lo + w * static_cast<float>(first + 1);
@@ -94,66 +176,11 @@ __device__ __forceinline__ double tridiag_top_eig(const double* alpha, const dou
     hi = nhi;
   }
   if (lane == 0) {
-    // inverse iteration on (T - s I): Gaussian elimination with partial
-    // pivoting on the tridiagonal (a row swap adds a second super-diagonal)
     const float s = 0.5f * (lo + hi);
-    const float tiny = 1e-30f;
-    float d[kMaxSteps], du[kMaxSteps], du2[kMaxSteps], l[kMaxSteps], rd[kMaxSteps], v[kMaxSteps];
-    bool piv[kMaxSteps];
-    for (int k = 0; k < m; ++k) {
-      d[k] = a32[k] - s;
-      du[k] = k < m - 1 ? b32[k] : 0.f;
-      du2[k] = 0.f;
-      piv[k] = false;
-    }
-    for (int k = 0; k < m - 1; ++k) {
-      const float dl = b32[k];
-      if (fabsf(d[k]) >= fabsf(dl)) {
-        if (d[k] == 0.f) d[k] = tiny;
-        l[k] = dl / d[k];
-        d[k + 1] -= l[k] * du[k];
-      } else {
-        piv[k] = true;
-        l[k] = d[k] / dl;
-        d[k] = dl;
-        const float t = d[k + 1];
-        d[k + 1] = du[k] - l[k] * t;
-        du[k] = t;
-        if (k < m - 2) {
-          du2[k] = du[k + 1];
-          du[k + 1] = -l[k] * du[k + 1];
-        }
-      }
-    }
-    if (m > 0 && d[m - 1] == 0.f) d[m - 1] = tiny;
-    for (int k = 0; k < m; ++k) rd[k] = 1.f / d[k];
-    for (int k = 0; k < m; ++k) v[k] = 1.f;
-    for (int it = 0; it < 3; ++it) {
-      for (int k = 0; k < m - 1; ++k) {
-        if (piv[k]) {
-          const float t = v[k];
-          v[k] = v[k + 1];
-          v[k + 1] = t - l[k] * v[k];
-        } else {
-          v[k + 1] -= l[k] * v[k];
-        }
-      }
-      for (int k = m - 1; k >= 0; --k) {
-        float acc = v[k];
-        if (k + 1 < m) acc -= du[k] * v[k + 1];
-        if (k + 2 < m) acc -= du2[k] * v[k + 2];
-        v[k] = acc * rd[k];
-      }
-      float mx = 0.f;
-      for (int k = 0; k < m; ++k) mx = fmaxf(mx, fabsf(v[k]));
-      if (!(mx > 0.f) || !isfinite(mx)) {
-        for (int k = 0; k < m; ++k) v[k] = k == 0 ? 1.f : 0.f;
-        break;
-      }
-      const float r = 1.f / mx;  // max-norm scaling keeps the iterate in range
-      for (int k = 0; k < m; ++k) v[k] *= r;
-    }
-    for (int k = 0; k < kMaxSteps; ++k) y[k] = k < m ? static_cast<double>(v[k]) : 0.0;
+    if (m == kMaxSteps)
+      inverse_iterate<kMaxSteps>(a32, b32, m, s, y);
+    else
+      inverse_iterate<0>(a32, b32, m, s, y);
   }
   __syncwarp();
   // FP64 Rayleigh quotient and normalisation (lane-parallel, fixed order)
