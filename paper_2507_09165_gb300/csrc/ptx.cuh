@@ -68,6 +68,21 @@ __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, vola
   }
 }
 
+// ------------------------------------- programmatic dependent launch
+// A kernel launched with pdl_attr() may be set up (barriers, tensor memory,
+// clusters) while its predecessor in the stream drains.  pdl_wait() returns once
+// the predecessor has completed and its writes are visible: it stands in front
+// of every global access.  pdl_launch() lets the successor be set up in turn.
+// Both do nothing in an ordinary launch.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+inline cudaLaunchAttribute pdl_attr() {
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
+
 // ------------------------------------------------- counters between CTAs
 // A counter that other CTAs increment after writing data this CTA's TMA
 // loads will read: the writer orders its stores before the increment (fence,

@@ -617,6 +617,8 @@ __global__ void __launch_bounds__(threads16(EW), 1)
   cluster_sync_all();  // both CTAs' barriers initialised before any arrival crosses the pair
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
+  pdl_launch();
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1341,13 +1343,14 @@ cudaError_t launch_symgemm_pair(int dtype, int epi, const CUtensorMap& tmA, cons
   cfg.blockDim = dim3(threads16(ew));
   cfg.dynamicSmemBytes = smem_bytes_pair(ew);
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1] = pdl_attr();
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k, tmA, tmB, p, out_dtype == DT_BF16 ? 1 : 0);
 }
 
