@@ -494,7 +494,7 @@ cudaError_t bgemm(BatchPlan* p, int epi, const Mat& A, const Mat& B, const Mat* 
     const Mat* ops[2] = {&A, &B};
     CUtensorMap tm[4];
     for (int i = 0; i < 4; ++i)
-      if (!encode_tmap_rows(&tm[i], DT_F16X2, bpart(p, *ops[i >> 1], i & 1), cols, rows, p->ldm, 128, 64))
+      if (!encode_tmap_rows(&tm[i], DT_F16X2, bpart(p, *ops[i >> 1], i & 1), cols, rows, p->ldm, 128, kRowBytesF32))
         return cudaErrorInvalidValue;
     g.num_tiles = p->ntiles_pair;
     g.tiles = p->d_tiles_pair;

@@ -234,6 +234,7 @@ bool get_schedule(psd_precision_t prec, Schedule& s);
 // single B, kRowBytesX3Single.
 constexpr int kRowBytes16 = 128;
 constexpr int kRowBytesX3Single = 128;
+constexpr int kRowBytesF32 = 128;
 inline int x3_row_bytes(bool b_single) { return b_single ? kRowBytesX3Single : 64; }
 // row_bytes: bytes of K per box row, 128 (128-byte swizzle) or 64 (64-byte swizzle).
 bool encode_tmap(CUtensorMap* map, int dtype, const void* base, int64_t n, int64_t ld, int box_rows,
@@ -300,7 +301,7 @@ cudaError_t launch_symgemm_x3(int et, bool b_single, int epi, int out, const CUt
                               int grid, cudaStream_t stream, bool pair = false);
 // The FP32 path's product (symgemm_f32.cu): scaled FP16 pairs on SM pairs,
 // promoted accumulation; tm = {A_hi, A_lo, B_hi, B_lo}, each with 128-row
-// boxes of 64 bytes; tiles from make_tile_list_pair; ep.in_scale / y_scale /
+// boxes of kRowBytesF32 bytes; tiles from make_tile_list_pair; ep.in_scale / y_scale /
 // out_scale carry the operands' scales; EPI_FINAL writes 16 shares per tile.
 cudaError_t launch_symgemm_f32(int epi, const CUtensorMap* tm, const GemmParams& p, int grid, cudaStream_t stream);
 int num_sms();

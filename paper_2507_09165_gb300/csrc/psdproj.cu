@@ -312,7 +312,8 @@ cudaError_t gemm(Plan* p, int epi, const Mat& A, const Mat& B, const Mat* out, c
     CUtensorMap tm[4];
     use_balanced_tiles(p, g);
     for (int i = 0; i < 4; ++i)
-      if (!encode_tmap(&tm[i], DT_F16X2, part_ptr(p, *ops[i >> 1], i & 1), n, ldm, i < 2 ? 128 : g.b_rows(), 64))
+      if (!encode_tmap(&tm[i], DT_F16X2, part_ptr(p, *ops[i >> 1], i & 1), n, ldm, i < 2 ? 128 : g.b_rows(),
+                       kRowBytesF32))
         return cudaErrorInvalidValue;
     if (epi == EPI_FINAL) p->ncompl = 16 * p->ntiles_bal;
     return launch_symgemm_f32(epi, tm, g, grid, s);

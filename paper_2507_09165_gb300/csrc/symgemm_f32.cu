@@ -36,17 +36,17 @@ constexpr int kEW = 8;                    // epilogue warps: two per 32-lane qua
 constexpr int kThreadsF = 128 + 32 * kEW;
 constexpr int kRegsIo = 40, kRegsEpi = 232;
 static_assert(128 * kRegsIo + 256 * kRegsEpi <= kThreadsF * 168, "register shares within the launch's registers");
-// 6 stages of 32 KB: 128 rows of A_hi, A_lo, B_hi, B_lo (B: this CTA's half),
-// 32 K elements (64-byte rows, 64-byte swizzle).
-constexpr int kRowBytesF = 64;
+// 3 stages of 64 KB: 128 rows of A_hi, A_lo, B_hi, B_lo (B: this CTA's half),
+// 64 K elements (128-byte rows, 128-byte swizzle).  6 stages of 64-byte rows in
+// the same space measured 4-8% slower (n = 3001: 4.07 against 3.76 ms).
+constexpr int kRowBytesF = kRowBytesF32;
 constexpr int kKElems = kRowBytesF / 2;
-constexpr int kOpBytes = kBM * kRowBytesF;  // 8 KB
+constexpr int kOpBytes = kBM * kRowBytesF;  // 16 KB
 constexpr int kStageBytesF = 4 * kOpBytes;
-constexpr int kStagesF = 6;
+constexpr int kStagesF = 3;
 constexpr int kChunkK = 128;
 constexpr int kChunkBlocks = kChunkK / kKElems;
-constexpr int kSW = kStgWords;
-constexpr int kEpiBytesF = 32 * kSW * 4;  // one 32 x 32 square of words per warp
+constexpr int kEpiBytesF = 32 * kStgWords * 4;  // per warp: 32 x 32 words (stage outputs) or 32 x 33 (final)
 constexpr int kTmemCols = 512;
 __host__ __device__ constexpr int smem_bytes_f32() {
   return 1024 + kStagesF * kStageBytesF + kEW * kEpiBytesF + 8 * (2 * kStagesF + 5) + 16;
@@ -56,31 +56,44 @@ static_assert(smem_bytes_f32() <= 232448, "shared memory per CTA");
 // the leader's barrier: they are given this long to land before the CTA exits.
 constexpr unsigned long long kDrainNs = 200000ull;
 
-__device__ __forceinline__ float2 half2_sum(uint32_t hi, uint32_t lo) {
-  const float2 h = __half22float2(*reinterpret_cast<__half2*>(&hi));
-  const float2 l = __half22float2(*reinterpret_cast<__half2*>(&lo));
-  return make_float2(h.x + l.x, h.y + l.y);
+__device__ __forceinline__ uint32_t pack_h2(float a, float b) {
+  const __half2 h = __floats2half2_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ float2 unpack_h2(uint32_t w) { return __half22float2(*reinterpret_cast<const __half2*>(&w)); }
+
+// 8 consecutive pair elements (w[e] = hi | lo << 16) to memory, clipped at `valid`.
+__device__ __forceinline__ void store_pair8(uint16_t* dh, uint16_t* dl, const uint32_t (&w)[8], int valid) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    h[e] = __byte_perm(w[2 * e], w[2 * e + 1], 0x5410);
+    l[e] = __byte_perm(w[2 * e], w[2 * e + 1], 0x7632);
+  }
+  if (valid >= 8) {
+    *reinterpret_cast<uint4*>(dh) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(dl) = make_uint4(l[0], l[1], l[2], l[3]);
+  } else {
+    for (int e = 0; e < valid; ++e) {
+      dh[e] = static_cast<uint16_t>(w[e]);
+      dl[e] = static_cast<uint16_t>(w[e] >> 16);
+    }
+  }
 }
 
-// 8 consecutive pair elements (w[e] = hi | lo << 16) to hi[0..7] and lo[0..7], clipped at `valid`.
-__device__ __forceinline__ void store_pair8(uint16_t* hi, uint16_t* lo, const uint32_t (&w)[8], int valid) {
-  if (valid >= 8) {
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      h[e] = __byte_perm(w[2 * e], w[2 * e + 1], 0x5410);
-      l[e] = __byte_perm(w[2 * e], w[2 * e + 1], 0x7632);
-    }
-    *reinterpret_cast<uint4*>(hi) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(lo) = make_uint4(l[0], l[1], l[2], l[3]);
-  } else {
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-      if (e < valid) {
-        hi[e] = static_cast<uint16_t>(w[e]);
-        lo[e] = static_cast<uint16_t>(w[e] >> 16);
-      }
-  }
+// A warp's staging square: 32 rows of 32 words, the 16-byte group g of row t at
+// g ^ (t & 7).  Word stores down a column of rows, 16-byte stores and loads along
+// a row per lane, and 16-byte loads of 64-byte segments (4 lanes a row) are all
+// free of bank conflicts.
+__device__ __forceinline__ int sq_word(int t, int e) { return 32 * t + ((((e >> 2) ^ (t & 7)) << 2) | (e & 3)); }
+__device__ __forceinline__ uint4* sq_group(uint32_t* S, int t, int g) {
+  return reinterpret_cast<uint4*>(S + 32 * t) + (g ^ (t & 7));
+}
+// Row t of the square: the 8 words from 8 seg on.
+__device__ __forceinline__ void sq_load8(uint32_t* S, int t, int seg, uint32_t (&w)[8]) {
+  const uint4 a = *sq_group(S, t, 2 * seg), b = *sq_group(S, t, 2 * seg + 1);
+  w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+  w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
 }
 
 // Moves the sums of a warp's later chunks one chunk down (a loop over chunks
@@ -92,6 +105,10 @@ __device__ __forceinline__ void next_chunk(float (&sum)[4][32]) {
     for (int j = 0; j < 32; ++j) sum[i][j] = sum[i + 1][j];
 }
 
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
 struct EpiOut {
   uint16_t *hi, *lo;         // the block's output pair
   const uint16_t *yh, *yl;   // EPI_POLY: the block's Y pair
@@ -100,91 +117,105 @@ struct EpiOut {
 };
 
 // One 32 x 32 chunk: lane l holds row r0 + l, v[j] the FP32 sum at column c0 + j.
-// Y is read along its own memory row r0 + l (Y is stored symmetric): 64
-// contiguous bytes per lane and part, all loads issued together.  hi and lo
-// travel as one 32-bit word through the staging square, written at (r, c) and
-// mirrored at (c, r) with 16-byte stores (33-word rows: both directions read
-// without bank conflicts); a diagonal chunk reads its upper part twice.
+// Global memory is read (Y) and written in segments of 64 bytes by 4 lanes
+// (whole sectors), 8 rows an instruction; between that shape and a row per
+// lane everything goes through the staging square as hi | lo words.  The square
+// holds the chunk transposed for the mirrored rows (c, r) and then as it is for
+// (r, c); a diagonal chunk is symmetrised from its upper part and written once.
+// With scalar conversions and staged words read one by one a chunk took
+// 5000-7500 cycles and the tensor cores waited at the end of every tile; with a
+// row per lane in global memory (16-byte pieces of sectors) n = 3001 was 10% slower.
 template <int EPI>
 __device__ __forceinline__ void epilogue_pair(const EpiOut& eo, int n, int64_t ldc, int64_t ldy, int r0, int c0,
                                               const float* v, uint32_t* S, int lane, bool track,
                                               unsigned& amax_bits) {
   const int r = r0 + lane;
   const bool diag = r0 == c0;
-  uint4 yh[4], yl[4];
+  const int seg = lane & 3, sr = lane >> 2;  // segment and row (+ 8 k) of the global accesses
+  uint32_t w[32];                            // the lane's row: hi | lo << 16
   if (EPI == EPI_POLY) {
+    uint4 yh[4], yl[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      yh[q] = yl[q] = make_uint4(0u, 0u, 0u, 0u);
-      const int c = c0 + 8 * q;
+    for (int k = 0; k < 4; ++k) {
+      yh[k] = yl[k] = make_uint4(0u, 0u, 0u, 0u);
+      const int rr = r0 + sr + 8 * k, c = c0 + 8 * seg;
       // rows hold round_up(n, 64) elements: a 16-byte load that starts below n stays inside (what lies past n is not used)
-      if (r < n && c < n) {
-        yh[q] = __ldg(reinterpret_cast<const uint4*>(eo.yh + static_cast<int64_t>(r) * ldy + c));
-        yl[q] = __ldg(reinterpret_cast<const uint4*>(eo.yl + static_cast<int64_t>(r) * ldy + c));
+      if (rr < n && c < n) {
+        yh[k] = __ldg(reinterpret_cast<const uint4*>(eo.yh + static_cast<int64_t>(rr) * ldy + c));
+        yl[k] = __ldg(reinterpret_cast<const uint4*>(eo.yl + static_cast<int64_t>(rr) * ldy + c));
       }
     }
-  }
-  __syncwarp();
+    __syncwarp();  // the previous chunk's reads of S are done
 #pragma unroll
-  for (int j = 0; j < 32; j += 2) {
-    float a = eo.cacc * v[j], b = eo.cacc * v[j + 1];
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t h[4] = {yh[k].x, yh[k].y, yh[k].z, yh[k].w}, l[4] = {yl[k].x, yl[k].y, yl[k].z, yl[k].w};
+#pragma unroll
+      for (int g = 0; g < 2; ++g)
+        *sq_group(S, sr + 8 * k, 2 * seg + g) =
+            make_uint4(__byte_perm(h[2 * g], l[2 * g], 0x5410), __byte_perm(h[2 * g], l[2 * g], 0x7632),
+                       __byte_perm(h[2 * g + 1], l[2 * g + 1], 0x5410), __byte_perm(h[2 * g + 1], l[2 * g + 1], 0x7632));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+      const uint4 a = *sq_group(S, lane, g);
+      w[4 * g] = a.x; w[4 * g + 1] = a.y; w[4 * g + 2] = a.z; w[4 * g + 3] = a.w;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    float a = eo.cacc * v[2 * q], b = eo.cacc * v[2 * q + 1];
     if (EPI == EPI_POLY) {
-      const uint4& h4 = yh[j >> 3];
-      const uint4& l4 = yl[j >> 3];
-      const int m = (j >> 1) & 3;
-      const uint32_t hw = m == 0 ? h4.x : m == 1 ? h4.y : m == 2 ? h4.z : h4.w;
-      const uint32_t lw = m == 0 ? l4.x : m == 1 ? l4.y : m == 2 ? l4.z : l4.w;
-      const float2 y = half2_sum(hw, lw);
-      a = fmaf(eo.cacc, v[j], eo.cy * y.x);
-      b = fmaf(eo.cacc, v[j + 1], eo.cy * y.y);
-      if (diag && j == lane) a += eo.cdiag;
-      if (diag && j + 1 == lane) b += eo.cdiag;
+      const float2 ya = unpack_h2(w[2 * q]), yb = unpack_h2(w[2 * q + 1]);  // (hi, lo)
+      a = fmaf(eo.cacc, v[2 * q], eo.cy * (ya.x + ya.y));
+      b = fmaf(eo.cacc, v[2 * q + 1], eo.cy * (yb.x + yb.y));
+      if (diag && 2 * q == lane) a += eo.cdiag;
+      if (diag && 2 * q + 1 == lane) b += eo.cdiag;
     }
-    const __half ah = __float2half_rn(a), bh = __float2half_rn(b);
-    const __half al = __float2half_rn(a - __half2float(ah)), bl = __float2half_rn(b - __half2float(bh));
-    S[lane * kSW + j] = __half_as_ushort(ah) | (static_cast<uint32_t>(__half_as_ushort(al)) << 16);
-    S[lane * kSW + j + 1] = __half_as_ushort(bh) | (static_cast<uint32_t>(__half_as_ushort(bl)) << 16);
-    if (track && r < n) {
-      if (c0 + j < n) {
-        const float t = (__half2float(ah) + __half2float(al)) * eo.unscale;
-        amax_bits = max(amax_bits, __float_as_uint(fabsf(t)));
-      }
-      if (c0 + j + 1 < n) {
-        const float t = (__half2float(bh) + __half2float(bl)) * eo.unscale;
-        amax_bits = max(amax_bits, __float_as_uint(fabsf(t)));
-      }
+    const uint32_t hi = pack_h2(a, b);
+    const float2 h = unpack_h2(hi);
+    const uint32_t lo = pack_h2(a - h.x, b - h.y);
+    w[2 * q] = __byte_perm(hi, lo, 0x5410);
+    w[2 * q + 1] = __byte_perm(hi, lo, 0x7632);
+  }
+  if (track && r < n) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      const float2 t = unpack_h2(w[j]);
+      if (c0 + j < n) amax_bits = max(amax_bits, __float_as_uint(fabsf((t.x + t.y) * eo.unscale)));
     }
   }
   __syncwarp();
-  const int seg = 8 * (lane & 3);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int jj = (lane >> 2) + 8 * k;
-    const int c = c0 + jj;
-    if (c < n && r0 + seg < n) {  // memory row c, elements r0 + seg ..
-      uint32_t w[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int t = seg + e;
-        w[e] = diag ? S[min(t, jj) * kSW + max(t, jj)] : S[t * kSW + jj];
-      }
-      const int64_t at = static_cast<int64_t>(c) * ldc + r0 + seg;
-      store_pair8(eo.hi + at, eo.lo + at, w, n - (r0 + seg));
-    }
-  }
+  for (int j = 0; j < 32; ++j) S[sq_word(j, lane)] = w[j];  // row j = column c0 + j
+  __syncwarp();
   if (!diag) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int tt = (lane >> 2) + 8 * k;
-      const int rr = r0 + tt;
-      if (rr < n && c0 + seg < n) {  // memory row r0 + tt, elements c0 + seg ..
-        uint32_t w[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) w[e] = S[tt * kSW + seg + e];
-        const int64_t at = static_cast<int64_t>(rr) * ldc + c0 + seg;
-        store_pair8(eo.hi + at, eo.lo + at, w, n - (c0 + seg));
-      }
+      const int jj = sr + 8 * k, c = c0 + jj, e0 = r0 + 8 * seg;
+      uint32_t u[8];
+      sq_load8(S, jj, seg, u);
+      const int64_t at = static_cast<int64_t>(c) * ldc + e0;
+      if (c < n && e0 < n) store_pair8(eo.hi + at, eo.lo + at, u, n - e0);
     }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      const uint32_t up = S[sq_word(lane, j)];  // element (j, lane) of the upper part
+      if (j < lane) w[j] = up;
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int g = 0; g < 8; ++g) *sq_group(S, lane, g) = make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int tt = sr + 8 * k, rr = r0 + tt, e0 = c0 + 8 * seg;
+    uint32_t u[8];
+    sq_load8(S, tt, seg, u);
+    const int64_t at = static_cast<int64_t>(rr) * ldc + e0;
+    if (rr < n && e0 < n) store_pair8(eo.hi + at, eo.lo + at, u, n - e0);
   }
 }
 
@@ -310,9 +341,9 @@ __global__ void __launch_bounds__(kThreadsF, 1)
                 for (int k = 0; k < kRowBytesF / 32; ++k) {
                   const uint32_t off = 32 * k;
                   const uint32_t more = ((kb - kc) | k) == 0 ? 0u : 1u;
-                  mma_f16_pair(d_tmem, sw64_kmajor_desc(ah + off), sw64_kmajor_desc(bl + off), idesc, more);
-                  mma_f16_pair(d_tmem, sw64_kmajor_desc(al + off), sw64_kmajor_desc(bh + off), idesc, 1u);
-                  mma_f16_pair(d_tmem, sw64_kmajor_desc(ah + off), sw64_kmajor_desc(bh + off), idesc, 1u);
+                  mma_f16_pair(d_tmem, sw128_kmajor_desc(ah + off), sw128_kmajor_desc(bl + off), idesc, more);
+                  mma_f16_pair(d_tmem, sw128_kmajor_desc(al + off), sw128_kmajor_desc(bh + off), idesc, 1u);
+                  mma_f16_pair(d_tmem, sw128_kmajor_desc(ah + off), sw128_kmajor_desc(bh + off), idesc, 1u);
                 }
                 mma_commit_pair(empty_bar(s), 3);  // frees the stage in both CTAs
               }
@@ -372,6 +403,13 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       const int ch_end = r0 < n ? min((tc.w + 31) >> 5, (n - tc.y + 31) >> 5) : ch_begin;
       const uint32_t lanes = static_cast<uint32_t>(32 * ew) << 16;
       const int kbn = (n + kKElems - 1) / kKElems;
+      if (EPI == EPI_POLY && r0 + lane < n) {  // this tile's Y towards L2 while the products run
+        const int64_t at = (br.off + br.dy + r0 + lane) * p.ep.ldy + tc.y;
+        for (int ch = max(half, ch_begin + ((ch_begin ^ half) & 1)); ch < ch_end; ch += 2) {
+          prefetch_l2(static_cast<const uint16_t*>(p.ep.Y) + at + 32 * ch);
+          prefetch_l2(static_cast<const uint16_t*>(p.ep.Y_lo) + at + 32 * ch);
+        }
+      }
       float sum[4][32] = {};
       bool ok = true;
       for (int kc = 0; kc < kbn; kc += kChunkBlocks) {
