@@ -78,7 +78,8 @@ struct BlockRec {
   // EPI_FINAL with EpiParams::cres unset: if set, the shares of <out, X - out>
   // of the tile at launch position t go to cres at the tile's position in the
   // request's own tile list, t + cres_shift (a served request; 4 per 128-row
-  // tile, 8 per tile on SM pairs: 4 (2 (t + cres_shift) + rank) + warp).
+  // tile; on SM pairs 2 EW per tile, EW epilogue warps: EW (2 (t + cres_shift) +
+  // rank) + warp).
   double* cres;
   int64_t cres_shift;
 };

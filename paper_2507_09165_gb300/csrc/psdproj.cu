@@ -127,12 +127,10 @@ struct Plan {
   BlockRec* d_block = nullptr;   // the one block of a single projection
   int4* d_tiles = nullptr;
   int ntiles = 0;
-  int4* d_tiles_pair = nullptr;  // 256 x 256 tiles of the final product of the 16-bit chains on CTA pairs
-  int ntiles_pair = 0;
-  int4* d_tiles_bal = nullptr;  // 256 x tile_w tiles of every other product on CTA pairs (pair_tile_width)
+  int4* d_tiles_bal = nullptr;  // 256 x tile_w tiles of the products on CTA pairs (pair_tile_width)
   int ntiles_bal = 0;
   int tile_w = 0;
-  int ncompl = 0;  // complementarity shares the final product writes (4 per one-SM tile, 8 per pair tile, 16 on the FP32 path)
+  int ncompl = 0;  // complementarity shares the final product writes (4 per one-SM tile, 16 per pair tile)
   double* d_compl = nullptr;  // 4 per tile: shares of <out, X - out> from the final product
   cudaGraphExec_t exec = nullptr;
   bool graph_tried = false;
@@ -185,15 +183,12 @@ psd_status_t build_plan(Plan* p, void* user_ws, size_t user_bytes) {
   const size_t o_info = o_state + round_up(sizeof(DevState), 256);
   const size_t o_block = o_info + round_up(sizeof(psd_info_t), 256);
   const size_t o_tiles = o_block + round_up(sizeof(BlockRec), 256);
-  std::vector<int4> tiles_pair = make_tile_list_pair(n);
-  p->ntiles_pair = static_cast<int>(tiles_pair.size());
   p->tile_w = pair_tile_width(n);
   std::vector<int4> tiles_bal = make_tile_list_pair(n, 0, 8, p->tile_w);
   p->ntiles_bal = static_cast<int>(tiles_bal.size());
   const size_t o_compl = o_tiles + round_up(sizeof(int4) * std::max<size_t>(tiles.size(), 1), 256);
-  const size_t ncompl_max = std::max({4 * tiles.size(), 8 * tiles_pair.size(), 16 * tiles_bal.size(), size_t{1}});
-  const size_t o_pair = o_compl + round_up(sizeof(double) * ncompl_max, 256);
-  const size_t o_bal = o_pair + round_up(sizeof(int4) * std::max<size_t>(tiles_pair.size(), 1), 256);
+  const size_t ncompl_max = std::max({4 * tiles.size(), 16 * tiles_bal.size(), size_t{1}});
+  const size_t o_bal = o_compl + round_up(sizeof(double) * ncompl_max, 256);
   const size_t small = o_bal + sizeof(int4) * std::max<size_t>(tiles_bal.size(), 1);
   uint8_t* sm = nullptr;
   if (cudaMalloc(&sm, small) != cudaSuccess) {
@@ -207,13 +202,9 @@ psd_status_t build_plan(Plan* p, void* user_ws, size_t user_bytes) {
   p->d_block = reinterpret_cast<BlockRec*>(sm + o_block);
   p->d_tiles = reinterpret_cast<int4*>(sm + o_tiles);
   p->d_compl = reinterpret_cast<double*>(sm + o_compl);
-  p->d_tiles_pair = reinterpret_cast<int4*>(sm + o_pair);
   p->d_tiles_bal = reinterpret_cast<int4*>(sm + o_bal);
   if (!tiles.empty() &&
       cudaMemcpy(p->d_tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-    return PSD_ERR_CUDA;
-  if (!tiles_pair.empty() && cudaMemcpy(p->d_tiles_pair, tiles_pair.data(), sizeof(int4) * tiles_pair.size(),
-                                        cudaMemcpyHostToDevice) != cudaSuccess)
     return PSD_ERR_CUDA;
   if (!tiles_bal.empty() && cudaMemcpy(p->d_tiles_bal, tiles_bal.data(), sizeof(int4) * tiles_bal.size(),
                                        cudaMemcpyHostToDevice) != cudaSuccess)
@@ -282,21 +273,16 @@ cudaError_t gemm(Plan* p, int epi, const Mat& A, const Mat& B, const Mat* out, c
         (epi == EPI_FINAL || odt == dt || (odt == DT_F16X2 && dt == DT_F16))) {
       // 16-bit products on CTA pairs: M = 256, half of B in each CTA (128-row boxes)
       CUtensorMap ta, tb;
-      if (epi == EPI_FINAL) {
-        // 256-wide tiles at any order: the shares of <out, X - out> are per tile,
-        // and a served request's list is the same
-        g.num_tiles = p->ntiles_pair;
-        g.tiles = p->d_tiles_pair;
-      } else {
-        use_balanced_tiles(p, g);
-      }
+      use_balanced_tiles(p, g);
       if (!encode_tmap(&ta, dt, part_ptr(p, A, 0), n, ldm, 128) ||
           !encode_tmap(&tb, dt, part_ptr(p, B, 0), n, ldm, g.b_rows()))
         return cudaErrorInvalidValue;
       const uint32_t fmt = dt == DT_BF16 ? 1u : 0u;
       g.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | (16u << 24);  // M = 256; N per tile
-      if (epi == EPI_FINAL) p->ncompl = 8 * p->ntiles_pair;
-      return launch_symgemm_pair(dt, epi, ta, tb, g, grid, s, epi == EPI_FINAL ? -1 : odt);
+      if (epi != EPI_FINAL) return launch_symgemm_pair(dt, epi, ta, tb, g, grid, s, odt);
+      // 8 epilogue warps: the final product reads X and writes both triangles in FP32
+      p->ncompl = 16 * p->ntiles_bal;
+      return launch_symgemm_pair(dt, epi, ta, tb, g, grid, s, -1, /*many_small=*/true);
     }
     CUtensorMap ta, tb;
     if (!encode_tmap(&ta, dt, part_ptr(p, A, 0), n, ldm, 128) || !encode_tmap(&tb, dt, part_ptr(p, B, 0), n, ldm, 256))

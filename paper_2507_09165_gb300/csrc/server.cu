@@ -76,9 +76,9 @@ struct Request {
   int g = 0;         // product of the stage in progress: 0 Y, 1 P, 2 X_t, 3 final
   int k = 0;         // tiles of that product done
   int ntiles = 0;    // bound on the tile count (admission)
-  std::vector<int4> tl;  // tile list of order n: 256 x 256 tiles on SM pairs (make_tile_list_pair)
-  double* cres = nullptr;  // shares of <out, X - out>, 8 per tile of tl in the one-SM order (arena rows
-                           // after the matrices)
+  std::vector<int4> tl;   // tile list of order n: 256 x 256 tiles on SM pairs (make_tile_list_pair)
+  std::vector<int4> tlf;  // the final product's: the single projection's tiles (pair_tile_width), in its order
+  double* cres = nullptr;  // shares of <out, X - out>, 16 per tile of tlf (arena rows after the matrices)
   Clock::time_point t_submit;
   double latency_ms = 0.0;
   psd_info_t info{};
@@ -122,17 +122,28 @@ struct RowAllocator {
   }
 };
 
-// Tiles of one request of order n (two 128-row tiles per upper 256 x 256 block).
+// The tiles of a request's product g (3: the final product).
+const std::vector<int4>& list_of(const Request* r, int g) { return g == 3 ? r->tlf : r->tl; }
+
+// Tiles of the final product of a request of order n.
+int64_t final_tiles_of(int64_t n) {
+  const int64_t w = pair_tile_width(n);
+  int64_t tiles = 0;
+  for (int64_t m0 = 0; m0 < n; m0 += 256) tiles += (n - m0 + w - 1) / w;
+  return tiles;
+}
+
+// Bound on the tiles of any product of a request of order n.
 int64_t tiles_of(int64_t n) {
   const int64_t nb = (n + 255) / 256;
-  return nb * (nb + 1);
+  return std::max(nb * (nb + 1), final_tiles_of(n));
 }
 
 // Arena rows of a request of order n: its four matrices, then its shares of
-// <out, X - out> (8 doubles per 256 x 256 tile, 4 per 128-row half: tiles_of(n)
-// halves) in whole rows of ldm 16-bit elements.
+// <out, X - out> (16 doubles per tile of the final product) in whole rows of ldm
+// 16-bit elements.
 int64_t rows_of(int64_t ldm, int64_t n) {
-  const int64_t share_bytes = 4 * static_cast<int64_t>(sizeof(double)) * tiles_of(n);
+  const int64_t share_bytes = 16 * static_cast<int64_t>(sizeof(double)) * final_tiles_of(n);
   return 4 * n + (share_bytes + 2 * ldm - 1) / (2 * ldm);
 }
 
@@ -204,7 +215,7 @@ __global__ void adopt_kernel(DevArgs* dst_args, DevState* dst_st, const DevArgs*
 }
 
 // A request that finishes in a step: its record slot and its shares of
-// <out, X - out> (ncompl = 4 per tile).
+// <out, X - out> (ncompl = 16 per tile of the final product).
 struct FinRec {
   int slot;
   int ncompl;
@@ -371,8 +382,10 @@ cudaError_t step_gemm(psd_server* s, int dti, int epi, const BlockRec* d_blocks,
   g.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | (16u << 24);  // M = 256: tiles on SM pairs
   ++launches;
   // SM pairs with 4 epilogue warps per CTA: served steps mix large requests,
-  // whose long main loops want the 6-stage ring
-  return launch_symgemm_pair(dti == 1 ? DT_BF16 : DT_F16, epi, s->tmA[dti], s->tmB[dti], g, num_sms(), s->main);
+  // whose long main loops want the 6-stage ring; the final product has 8, as in
+  // the single projection (its shares are per warp)
+  return launch_symgemm_pair(dti == 1 ? DT_BF16 : DT_F16, epi, s->tmA[dti], s->tmB[dti], g, num_sms(), s->main, -1,
+                             epi == EPI_FINAL);
 }
 
 // Builds and enqueues one scheduler step over `run`.  A step is one grouped
@@ -461,11 +474,11 @@ bool enqueue_step(psd_server* s, const std::vector<Request*>& run, int& launches
   int64_t budget = kStepBudget;
   for (int i : order) {
     Request* r = run[i];
-    const int nt = static_cast<int>(r->tl.size());
     const int64_t cost = 2 * ((r->n + 63) / 64);  // K-blocks of 64 per 256-row tile (two 128-row tiles)
     Cursor c{r->stage, r->g, r->k, false};
     bool any = false;
     for (;;) {
+      const int nt = static_cast<int>(list_of(r, c.g).size());
       const int rem = nt - c.k;
       int64_t m = std::min<int64_t>(rem, std::max<int64_t>(budget, 0) / cost);
       if (m <= 0 && !any) m = std::min<int64_t>(rem, std::max<int64_t>(1, kStepBudget / kQuantumDiv / cost));
@@ -506,7 +519,7 @@ bool enqueue_step(psd_server* s, const std::vector<Request*>& run, int& launches
         // final product: tile q of the request sits at launch position q - cres_shift
         if (g == 3) hb[3 * mb + it->req].cres_shift = it->begin - (nt_all - start);
         for (int q = it->begin; q < it->end; ++q) {
-          int4 tc = r->tl[q];
+          int4 tc = list_of(r, g)[q];
           tc.z = it->req;
           ht[nt_all++] = tc;
         }
@@ -518,7 +531,7 @@ bool enqueue_step(psd_server* s, const std::vector<Request*>& run, int& launches
   int nf = 0;
   for (int i = 0; i < nrun; ++i)
     if (next[i].done) {
-      hfin[nf++] = FinRec{run[i]->slot, 8 * static_cast<int>(run[i]->tl.size()), run[i]->cres};
+      hfin[nf++] = FinRec{run[i]->slot, 16 * static_cast<int>(run[i]->tlf.size()), run[i]->cres};
       fin_ids.push_back(run[i]->id);
     }
   {
@@ -756,17 +769,18 @@ extern "C" psd_status_t psd_server_create(size_t hbm_budget_bytes, int32_t devic
   const size_t row_bytes = static_cast<size_t>(s->ldm) * 2;
   const size_t lane_bytes = round_up(kLaneHead + lanczos_bytes(max_order), 1024);
   const size_t recs_bytes = round_up(kRecBytes * max_batch, 1024);
-  // tile capacity: sum over requests of tiles_of(n) <= (max_order/256 + 3) rows/1024 + 2 max_batch
+  // tile capacity: sum over requests of tiles_of(n) <= (max_order/256 + 3) rows/1024 + 80 max_batch (small
+  // orders' final products have up to one tile per SM pair)
   auto fixed_for = [&](int64_t tile_cap) {
     return 1024 + recs_bytes + kLanes * lane_bytes + kRing * round_up(stage_layout(max_batch, tile_cap).total, 1024);
   };
   int64_t rows = 0;
-  int64_t tile_cap = 2 * max_batch;
+  int64_t tile_cap = 80 * max_batch;
   for (int it = 0; it < 3; ++it) {  // rows and tile capacity depend on each other; settle them
     const size_t fixed = fixed_for(tile_cap);
     rows = hbm_budget_bytes > fixed ? static_cast<int64_t>((hbm_budget_bytes - fixed) / row_bytes) : 0;
     rows = std::min(rows, kMaxArenaRows);
-    tile_cap = 2 * static_cast<int64_t>(max_batch) + (max_order / 256 + 3) * (rows / 1024 + 1);
+    tile_cap = 80 * static_cast<int64_t>(max_batch) + (max_order / 256 + 3) * (rows / 1024 + 1);
   }
   while (rows > 0 && fixed_for(tile_cap) + static_cast<size_t>(rows) * row_bytes > hbm_budget_bytes) --rows;
   if (rows < rows_of(s->ldm, max_order)) {
@@ -843,7 +857,10 @@ extern "C" psd_status_t psd_server_submit(psd_server_t* s, int64_t n, const floa
   r->dt = precision == PSD_PREC_BF16 ? DT_BF16 : DT_F16;
   r->ready = reinterpret_cast<cudaEvent_t>(ready);
   r->ntiles = static_cast<int>(tiles_of(n));
-  if (n > 0) r->tl = make_tile_list_pair(n, 0);
+  if (n > 0) {
+    r->tl = make_tile_list_pair(n, 0);
+    r->tlf = make_tile_list_pair(n, 0, 8, pair_tile_width(n));
+  }
   r->t_submit = Clock::now();
   {
     std::lock_guard<std::mutex> lk(s->mu);
