@@ -43,7 +43,7 @@ struct DevState {
   double maxdiag;
   double inv_lambda;     // 1 / lam~ (0 when lam~ == 0)
   int m;                 // Lanczos steps taken
-  int done;              // breakdown reached
+  int done;              // nonzero once the Lanczos run has stopped (the multi-launch form: after which step)
   int status;            // first psd_status_t raised on the device
   unsigned maxdiag_bits; // max |X_ii| as float bits (atomicMax)
   unsigned absmax_bits;  // max |X_T(i,j)| as float bits (atomicMax)

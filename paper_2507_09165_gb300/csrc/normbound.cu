@@ -458,7 +458,7 @@ __device__ __forceinline__ bool ph_orth_next(const NBCtx& c, int cta, int ncta, 
     c.st->alpha[j] = __ldcg(&c.st->alpha[j]) + f2_to_d(F2{sh.u.orth.s[j].x, sh.u.orth.s[j].y});
     c.st->beta[j] = beta;
     c.st->m = j + 1;
-    if (stop) c.st->done = 1;
+    if (stop) c.st->done = j + 1;
   }
   if (!stop) {
     const double inv = sh.scalar[1];
@@ -623,7 +623,11 @@ __global__ void __launch_bounds__(kNT) nb_reduce_dots_kernel(NBCtx c, int j) {
   ph_reduce_dots(c, blockIdx.x, j, sh);
 }
 __global__ void __launch_bounds__(kNT) nb_orth_kernel(NBCtx c, int j) {
-  if (c.st->done) return;
+  // `done` is j + 1 once step j stopped: set by this very launch in the last step,
+  // while CTAs of it may still be starting -- they must not take it for an earlier
+  // step's, some warps before and some after it is set
+  const int done = c.st->done;
+  if (done != 0 && done <= j) return;
   __shared__ NBShared sh;
   ph_orth_next(c, blockIdx.x, gridDim.x, j, sh);
 }

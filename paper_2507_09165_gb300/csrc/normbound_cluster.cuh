@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(kNT, 2) nb_cluster_kernel(const ClusterJob jb)
       st->sigma = sigma;
       st->fro = fro;
       st->m = m;
-      st->done = 1;
+      st->done = m;
       st->status = 0;
       st->maxdiag_bits = md;
       st->absmax_bits = 0;
