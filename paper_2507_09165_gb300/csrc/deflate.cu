@@ -92,46 +92,45 @@ __global__ void gram_kernel(int n, int64_t npad, const double* __restrict__ Q, c
 
 // Symmetric 2 x 2 Schur rotation (Golub & Van Loan, Sec. 8.5): (c, s) with
 // [c s; -s c]^T [app apq; apq aqq] [c s; -s c] diagonal.
-__device__ void sym_schur2(double app, double apq, double aqq, double& c, double& s) {
-  if (apq == 0.0) {
-    c = 1.0;
-    s = 0.0;
+template <class T>
+__device__ void sym_schur2(T app, T apq, T aqq, T& c, T& s) {
+  if (apq == T(0)) {
+    c = T(1);
+    s = T(0);
     return;
   }
-  const double tau = (aqq - app) / (2.0 * apq);
-  const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-  c = 1.0 / sqrt(1.0 + t * t);
+  const T tau = (aqq - app) / (T(2) * apq);
+  const T t = (tau >= T(0) ? T(1) : T(-1)) / (fabs(tau) + sqrt(T(1) + tau * tau));
+  c = T(1) / sqrt(T(1) + t * t);
   s = t * c;
 }
 
-// Eigen-decomposition of the m x m Rayleigh quotient: parallel cyclic Jacobi
-// with the round-robin ordering (Golub & Van Loan, Sec. 8.5.5): each of the
-// M - 1 rounds of a sweep (M = m rounded up to even) rotates M / 2 disjoint
-// index pairs at once.  Disjoint rotations leave each other's 2 x 2 blocks
-// alone, so a round equals the same rotations applied one by one.  Thread
-// (k, i) = (t % 32, t / 32) applies rotation i to row k (the column rotations,
-// of A and of V), then to column k (the row rotations).  Eigenpairs sorted by
-// |mu| descending.
-constexpr int kRrThreads = 32 * (kM / 2);
-__global__ void __launch_bounds__(kRrThreads) rr_kernel(const DevState* st, const double* H, double* W, double* mu) {
-  __shared__ double A[kM][kM], V[kM][kM];
-  __shared__ double cs[kM / 2][2];
-  __shared__ int pq[kM / 2][2];
-  __shared__ int converged;
-  const int m = st->m, t = threadIdx.x, k = t & 31, i = t >> 5;
+// Shared scratch of the Jacobi sweeps.
+template <class T>
+struct JacobiScratch {
+  T cs[kM / 2][2];
+  int pq[kM / 2][2];
+  int converged;
+};
+
+// Parallel cyclic Jacobi with the round-robin ordering (Golub & Van Loan, Sec.
+// 8.5.5): each of the M - 1 rounds of a sweep (M = m rounded up to even)
+// rotates M / 2 disjoint index pairs at once.  Disjoint rotations leave each
+// other's 2 x 2 blocks alone, so a round equals the same rotations applied one
+// by one.  Thread (k, i) = (t % 32, t / 32) applies rotation i to row k (the
+// column rotations, of A and of V), then to column k (the row rotations).
+// Sweeps until the off-diagonal's share of ||A||_F^2 is at most `tol`, or
+// `max_sweeps`.
+template <class T>
+__device__ void jacobi_sweeps(T (*A)[kM], T (*V)[kM], int m, T tol, int max_sweeps, JacobiScratch<T>& sh) {
+  const int t = threadIdx.x, k = t & 31, i = t >> 5;
   const int M = m + (m & 1);
-  for (int e = t; e < m * m; e += blockDim.x) {
-    const int r = e / m, c = e % m;
-    A[r][c] = 0.5 * (H[r * kM + c] + H[c * kM + r]);
-    V[r][c] = r == c ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  for (int sweep = 0; sweep < 40 && m > 1; ++sweep) {
+  for (int sweep = 0; sweep < max_sweeps && m > 1; ++sweep) {
     if (i == 0) {
-      double off = 0.0, tot = 0.0;
+      T off = T(0), tot = T(0);
       if (k < m)
         for (int j = 0; j < m; ++j) {
-          const double v = A[k][j] * A[k][j];
+          const T v = A[k][j] * A[k][j];
           tot += v;
           if (j != k) off += v;
         }
@@ -139,10 +138,10 @@ __global__ void __launch_bounds__(kRrThreads) rr_kernel(const DevState* st, cons
         off += __shfl_xor_sync(0xffffffffu, off, o);
         tot += __shfl_xor_sync(0xffffffffu, tot, o);
       }
-      if (k == 0) converged = !(off > 1e-30 * tot);  // also on NaN
+      if (k == 0) sh.converged = !(off > tol * tot);  // also on NaN
     }
     __syncthreads();
-    if (converged) break;
+    if (sh.converged) break;
     for (int r = 0; r < M - 1; ++r) {
       if (t < M / 2) {  // pair t of round r (circle method, player M - 1 fixed)
         int p = t == 0 ? r : (r + t) % (M - 1);
@@ -152,34 +151,111 @@ __global__ void __launch_bounds__(kRrThreads) rr_kernel(const DevState* st, cons
           p = q;
           q = x;
         }
-        double c = 1.0, sn = 0.0;
+        T c = T(1), sn = T(0);
         if (q < m) sym_schur2(A[p][p], A[p][q], A[q][q], c, sn);
-        pq[t][0] = p;
-        pq[t][1] = q < m ? q : -1;  // the dummy player of an odd m
-        cs[t][0] = c;
-        cs[t][1] = sn;
+        sh.pq[t][0] = p;
+        sh.pq[t][1] = q < m ? q : -1;  // the dummy player of an odd m
+        sh.cs[t][0] = c;
+        sh.cs[t][1] = sn;
       }
       __syncthreads();
-      const bool act = k < m && i < M / 2 && pq[i][1] >= 0;
-      const int p = act ? pq[i][0] : 0, q = act ? pq[i][1] : 0;
-      const double c = act ? cs[i][0] : 1.0, sn = act ? cs[i][1] : 0.0;
+      const bool act = k < m && i < M / 2 && sh.pq[i][1] >= 0;
+      const int p = act ? sh.pq[i][0] : 0, q = act ? sh.pq[i][1] : 0;
+      const T c = act ? sh.cs[i][0] : T(1), sn = act ? sh.cs[i][1] : T(0);
       if (act) {  // columns p, q of row k
-        const double akp = A[k][p], akq = A[k][q];
+        const T akp = A[k][p], akq = A[k][q];
         A[k][p] = c * akp - sn * akq;
         A[k][q] = sn * akp + c * akq;
-        const double vkp = V[k][p], vkq = V[k][q];
+        const T vkp = V[k][p], vkq = V[k][q];
         V[k][p] = c * vkp - sn * vkq;
         V[k][q] = sn * vkp + c * vkq;
       }
       __syncthreads();
       if (act) {  // rows p, q of column k; the annihilated pair set to 0 exactly
-        const double apk = A[p][k], aqk = A[q][k];
-        A[p][k] = k == q ? 0.0 : c * apk - sn * aqk;
-        A[q][k] = k == p ? 0.0 : sn * apk + c * aqk;
+        const T apk = A[p][k], aqk = A[q][k];
+        A[p][k] = k == q ? T(0) : c * apk - sn * aqk;
+        A[q][k] = k == p ? T(0) : sn * apk + c * aqk;
       }
       __syncthreads();
     }
   }
+  __syncthreads();
+}
+
+// C = op(A) B of m x m matrices (ta: A transposed), FP64, one element per thread and step.
+__device__ void mat_mul(const double (*A)[kM], const double (*B)[kM], double (*C)[kM], int m, bool ta) {
+  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+    const int r = e / m, c = e % m;
+    double s0 = 0.0, s1 = 0.0;
+    for (int j = 0; j + 1 < m; j += 2) {
+      s0 = fma(ta ? A[j][r] : A[r][j], B[j][c], s0);
+      s1 = fma(ta ? A[j + 1][r] : A[r][j + 1], B[j + 1][c], s1);
+    }
+    if (m & 1) s0 = fma(ta ? A[m - 1][r] : A[r][m - 1], B[m - 1][c], s0);
+    C[r][c] = s0 + s1;
+  }
+  __syncthreads();
+}
+
+// Eigen-decomposition of the m x m Rayleigh quotient, eigenpairs sorted by
+// |mu| descending.  A round of FP64 rotations costs ~5000 cycles (this GPU
+// issues an FP64 instruction every ~19 cycles per SM), so the sweeps run in
+// FP32 first, on H scaled to unit norm; their V, made orthogonal to FP64 by two
+// Newton-Schulz steps V <- V (3 I - V^T V) / 2 (its error, ~1e-6, is squared by
+// each), takes H to V^T H V, whose off-diagonal is ~1e-7, and two or three FP64
+// sweeps finish to the same criterion as sweeps from the start did.
+constexpr int kRrThreads = 32 * (kM / 2);
+__global__ void __launch_bounds__(kRrThreads) rr_kernel(const DevState* st, const double* H, double* W, double* mu) {
+  __shared__ double A[kM][kM], V[kM][kM], B[kM][kM], C[kM][kM];
+  __shared__ float Af[kM][kM], Vf[kM][kM];
+  __shared__ JacobiScratch<float> shf;
+  __shared__ JacobiScratch<double> sh;
+  __shared__ double scale;
+  const int m = st->m, t = threadIdx.x;
+  for (int e = t; e < m * m; e += blockDim.x) {
+    const int r = e / m, c = e % m;
+    A[r][c] = 0.5 * (H[r * kM + c] + H[c * kM + r]);
+    V[r][c] = r == c ? 1.0 : 0.0;
+  }
+  __syncthreads();
+  if (t < 32) {
+    double tot = 0.0;
+    if (t < m)
+      for (int j = 0; j < m; ++j) tot = fma(A[t][j], A[t][j], tot);
+    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    if (t == 0) scale = tot > 0.0 && isfinite(tot) ? 1.0 / sqrt(tot) : 0.0;
+  }
+  __syncthreads();
+  if (m > 2 && scale > 0.0 && isfinite(scale)) {
+    for (int e = t; e < m * m; e += blockDim.x) {
+      const int r = e / m, c = e % m;
+      Af[r][c] = static_cast<float>(A[r][c] * scale);
+      Vf[r][c] = r == c ? 1.f : 0.f;
+    }
+    __syncthreads();
+    jacobi_sweeps<float>(Af, Vf, m, 1e-11f, 8, shf);
+    for (int e = t; e < m * m; e += blockDim.x) V[e / m][e % m] = static_cast<double>(Vf[e / m][e % m]);
+    __syncthreads();
+    for (int it = 0; it < 2; ++it) {
+      mat_mul(V, V, B, m, true);
+      for (int e = t; e < m * m; e += blockDim.x) {
+        const int r = e / m, c = e % m;
+        B[r][c] = (r == c ? 1.5 : 0.0) - 0.5 * B[r][c];
+      }
+      __syncthreads();
+      mat_mul(V, B, C, m, false);
+      for (int e = t; e < m * m; e += blockDim.x) V[e / m][e % m] = C[e / m][e % m];
+      __syncthreads();
+    }
+    mat_mul(A, V, B, m, false);
+    mat_mul(V, B, C, m, true);
+    for (int e = t; e < m * m; e += blockDim.x) {
+      const int r = e / m, c = e % m;
+      A[r][c] = 0.5 * (C[r][c] + C[c][r]);
+    }
+    __syncthreads();
+  }
+  jacobi_sweeps<double>(A, V, m, 1e-30, 40, sh);
   if (t == 0) {
     int order[kM];
     for (int j = 0; j < m; ++j) order[j] = j;
