@@ -262,13 +262,13 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     tma_prefetch_desc(&tmBh);
     tma_prefetch_desc(&tmBl);
   }
-  if (warp == 1) {
-    tmem_alloc_pair(smem_u32(tmem_holder), kTmemCols);
-    tmem_relinquish_pair();
-  }
+  if (warp == 1) tmem_alloc_pair(smem_u32(tmem_holder), kTmemCols);
   tc_fence_before();
-  cluster_sync_all();  // both CTAs' barriers initialised before any arrival crosses the pair
+  cluster_sync_all();  // both CTAs' barriers initialised and both allocations made
   tc_fence_after();
+  // The permit is the pair's: given up by one CTA before the other has allocated (its
+  // warps may start late beside other work), it left that allocation waiting for good.
+  if (warp == 1) tmem_relinquish_pair();
   const uint32_t tmem_base = *tmem_holder;
 
   if (warp < 4) {

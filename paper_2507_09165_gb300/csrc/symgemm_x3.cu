@@ -388,7 +388,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 1) {
     if (PAIR) {
       tmem_alloc_pair(smem_u32(tmem_holder), kTmemCols);
-      tmem_relinquish_pair();
     } else {
       tmem_alloc(smem_u32(tmem_holder), kTmemCols);
       tmem_relinquish();
@@ -396,10 +395,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   tc_fence_before();
   if (PAIR)
-    cluster_sync_all();  // both CTAs' barriers initialised before any arrival crosses the pair
+    cluster_sync_all();  // both CTAs' barriers initialised and both allocations made
   else
     __syncthreads();
   tc_fence_after();
+  // The permit is the pair's: given up by one CTA before the other has allocated (its
+  // warps may start late beside other work), it left that allocation waiting for good.
+  if (PAIR && warp == 1) tmem_relinquish_pair();
   const uint32_t tmem_base = *tmem_holder;
   constexpr bool TF32 = ET == DT_TF32X3;
   constexpr int kKElems = X3Cfg<B1>::kRowBytes / (TF32 ? 4 : 2);  // K elements per stage
