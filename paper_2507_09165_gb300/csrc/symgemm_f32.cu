@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(kThreadsF, 1)
   tc_fence_before();
   cluster_sync_all();  // both CTAs' barriers initialised and both allocations made
   tc_fence_after();
-  // The permit is the pair's: given up by one CTA before the other has allocated (its
-  // warps may start late beside other work), it left that allocation waiting for good.
+  // only now: nothing before the barrier orders one CTA giving up the permit against
+  // the other CTA's allocation
   if (warp == 1) tmem_relinquish_pair();
   const uint32_t tmem_base = *tmem_holder;
 

@@ -2,7 +2,8 @@
 // (hi, lo), hi = RN(v), lo = RN(v - hi), and the product formed on the tensor
 // cores as A_hi B_hi + A_hi B_lo + A_lo B_hi accumulated in one FP32 tensor
 // memory accumulator (the lo * lo term is below the accumulation error).
-//   TF32 pairs (kind::tf32): the FP32 path; three-term TF32 splitting as in
+//   TF32 pairs (kind::tf32; the product entry point only -- the FP32 path runs on
+//     scaled FP16 pairs, symgemm_f32.cu): three-term TF32 splitting as in
 //     Ootomo & Yokota, "Recovering single precision accuracy from Tensor Cores
 //     while surpassing the FP32 theoretical peak performance" (IJHPCA 2022).
 //   FP16 pairs (kind::f16): about 22 significant bits (fewer where the lo part
@@ -399,8 +400,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   else
     __syncthreads();
   tc_fence_after();
-  // The permit is the pair's: given up by one CTA before the other has allocated (its
-  // warps may start late beside other work), it left that allocation waiting for good.
+  // only now: nothing before the barrier orders one CTA giving up the permit against
+  // the other CTA's allocation
   if (PAIR && warp == 1) tmem_relinquish_pair();
   const uint32_t tmem_base = *tmem_holder;
   constexpr bool TF32 = ET == DT_TF32X3;
@@ -724,7 +725,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 using KernelX3 = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                           const GemmParams);
 
-// Instances: TF32 pairs (the FP32 path: pair outputs, the FP32 final output);
+// Instances: TF32 pairs (the product entry point: pair outputs, the FP32 final output);
 // FP16 pairs (pair or FP16 outputs); FP16 pair A with a single FP16 B (P X of
 // the mixed precision's pair stages, FP16 output).
 KernelX3 pick_pair(bool b1, int epi, int out) {
