@@ -2,8 +2,9 @@
 // cast X_0 = X / lam~ (Algorithm 2 step 3).
 //
 // Lanczos on A = X^2 (Parlett, The Symmetric Eigenvalue Problem, Ch. 13):
-// 20 steps, A q = X (X q), Lanczos vectors and all recurrences in FP64 with
-// full re-orthogonalisation (classical Gram-Schmidt, two passes), then the
+// 20 steps, A q = X (X q), Lanczos vectors and all recurrences in FP64: the
+// three-term recurrence, then full re-orthogonalisation (one classical
+// Gram-Schmidt pass), then the
 // largest Ritz pair (sigma, q) of the tridiagonal T_m and
 //     lam~ = sqrt(sigma + ||X (X q) - sigma q||_2),
 // raised to max(lam~, ||X||_F / sqrt(n), max_i |X_ii|) (both lower bounds of
@@ -19,8 +20,9 @@
 // TwoSum error-free transformation (Knuth; Ogita, Rump & Oishi, "Accurate sum
 // and dot product", SIAM J. Sci. Comput. 2005), converted to FP64 per vector
 // element.  A mat-vec is thus accurate to a few FP32 roundings of the 8-term
-// runs (~1e-7 relative); every operation on vectors -- the recurrences, dot
-// products, re-orthogonalisation and norms -- is FP64 in a fixed order.
+// runs (~1e-7 relative); the recurrences and the re-orthogonalisation are FP64,
+// the dot products and norms that feed them double-float (FP32 pairs, ~48
+// bits), all in a fixed order.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -53,7 +55,7 @@ __device__ unsigned long long g_debug_barrier_limit_ns = kWaitLimitNs;
 //
 // Every phase of the norm bound is a device function over virtual blocks of
 // kNT = 256 threads.  It runs either as the body of its own kernel (one CTA
-// per virtual block: the multi-launch path, 151 launches per bound) or inside
+// per virtual block: the multi-launch path, kNormBoundLaunches per bound) or inside
 // one persistent cooperative kernel whose CTAs take virtual blocks
 // blockIdx.x, blockIdx.x + gridDim.x, ... between grid-wide barriers.  Both
 // execute the same arithmetic in the same order and give the same bits.
@@ -332,16 +334,28 @@ __device__ __forceinline__ F2 reduce_partials(const NBCtx& c, int ch, NBShared& 
   const int e = ch * 32 + lane;
   F2 a{0.f, 0.f}, d{0.f, 0.f};
   if (e < c.n) {
+    // P1 of bj = b + hw, + 4, ... then P2 of bi = hw, + 4, ... <= b: about (nb + 1) / 4
+    // entries, ten loads in flight (a loop unrolled over a few entries waits for
+    // the loads of its remainder one by one): the bound at n = 2000 417 -> 389 us,
+    // 4096 578 -> 546, 10000 2042 -> 1981, and unchanged where one cluster runs it
     const int b = e / kSymvTile;
-#pragma unroll 8
-    for (int bj = b + hw; bj < c.nb; bj += 4) {
-      const float2 t = __ldcg(c.P1 + static_cast<int64_t>(bj) * c.npad + e);
-      a = f2_add(a, F2{t.x, t.y});
-    }
-#pragma unroll 8
-    for (int bi = hw; bi <= b; bi += 4) {
-      const float2 t = __ldcg(c.P2 + static_cast<int64_t>(bi) * c.npad + e);
-      d = f2_add(d, F2{t.x, t.y});
+    const int c1 = (c.nb - b - hw + 3) / 4, c2 = (b - hw + 4) / 4, cnt = c1 + c2;
+    for (int i0 = 0; i0 < cnt; i0 += 10) {
+      float2 p[10];
+#pragma unroll
+      for (int k = 0; k < 10; ++k) {
+        const int i = i0 + k;
+        const float2* at = i < c1 ? c.P1 + static_cast<int64_t>(b + hw + 4 * i) * c.npad
+                                  : c.P2 + static_cast<int64_t>(hw + 4 * (i - c1)) * c.npad;
+        p[k] = i < cnt ? __ldcg(at + e) : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int k = 0; k < 10; ++k) {
+        if (i0 + k < c1)
+          a = f2_add(a, F2{p[k].x, p[k].y});
+        else if (i0 + k < cnt)
+          d = f2_add(d, F2{p[k].x, p[k].y});
+      }
     }
   }
   const F2 t = f2_add(a, d);
