@@ -72,9 +72,9 @@ def tensor_pipe(prec, n):
 # Tensor-core products of one projection per precision (each symmetric product does
 # n^3 (1 + 256/n) flops): fp16/bf16 22 (3T + 1, T = 7); mixed 30 (stages 2-3: Y with a pair
 # output 1, Y^2 of pairs 3, P X 2; stages 1 and 4: Y 1, P with a pair output 1, P X 2; stages
-# 5-7 three each; final 1); fp32 93 TF32 products
-# (31 split products of 3), whose peak is half the bf16 rate.
-CHAIN_PRODUCTS = {"fp16": (22, 1.0), "bf16": (22, 1.0), "mixed": (30, 1.0), "fp32": (93, 0.5)}
+# 5-7 three each; final 1); fp32 93 FP16 products
+# (31 split products of 3).
+CHAIN_PRODUCTS = {"fp16": (22, 1.0), "bf16": (22, 1.0), "mixed": (30, 1.0), "fp32": (93, 1.0)}
 
 
 def step_roofline(prec, n, ms_step, peak_bf16):
@@ -102,7 +102,7 @@ def roofline_traffic(prec, n):
     return t["bytes"] if h.hexdigest() == t["sha256"] else None
 
 
-DTYPE = {"fp16": "f16", "bf16": "bf16", "fp32": "f32 (tf32x3)", "mixed": "f16 + f16 hi/lo pairs", "fp8_late": "f16 + e4m3"}
+DTYPE = {"fp16": "f16", "bf16": "bf16", "fp32": "f32 (f16x3)", "mixed": "f16 + f16 hi/lo pairs", "fp8_late": "f16 + e4m3"}
 
 
 def parse():
@@ -645,17 +645,17 @@ def run_ours(args):
 
     # dominant kernel: the symmetric tensor-core product of the chain, same kernel, shape and
     # form as in the projection (mixed: the FP16-pair split product of stages 2-3; fp16/bf16:
-    # the 16-bit product; both on SM pairs; fp32: the TF32x3 split product on one SM), timed
-    # alone with CUDA events on the launching stream
+    # the 16-bit product; both on SM pairs; fp32: the same FP16-pair split product, which the
+    # chain runs with scaled operands and promoted accumulation), timed alone with CUDA events on the launching stream
     ld = (n + 63) // 64 * 64
-    kprec = {"mixed": "mixed", "fp32": "fp32", "bf16": "bf16"}.get(prec, "fp16")
-    parts, et = {"mixed": (2, torch.float16), "fp32": (2, torch.float32),
+    kprec = {"mixed": "mixed", "fp32": "mixed", "bf16": "bf16"}.get(prec, "fp16")
+    parts, et = {"mixed": (2, torch.float16), "fp32": (2, torch.float16),
                  "bf16": (1, torch.bfloat16)}.get(prec, (1, torch.float16))
     A = (torch.randn(parts, n, ld, device=dev) / math.sqrt(n)).to(et)
     if parts == 2:
         A[1].mul_(1.0 / 2048)  # lo part of a hi/lo pair
     C = torch.empty_like(A)
-    form = 0 if prec == "fp32" else b.EPI_CTA_PAIR
+    form = b.EPI_CTA_PAIR
     for _ in range(3):
         b.psd_symm_product(n, A, A, ld, C, 0, kprec, form, stream=s)
     reps = 20 if parts == 1 else 8
@@ -670,8 +670,7 @@ def run_ours(args):
     products = 3 if parts == 2 else 1  # the split product runs three tensor-core products
     alg_flops = products * n ** 3 * (1 + 256 / n)  # symmetric product, 256-wide tiles: n^3 (1 + b/n)
     achieved = alg_flops / (gemm_ms * 1e-3) / 1e12
-    # dense peaks: bf16/fp16 measured; tf32 nominally half of that rate
-    peak = peaks["bf16_tflops"] * (0.5 if prec == "fp32" else 1.0)
+    peak = peaks["bf16_tflops"]
 
     # the comparator of the metric: the same library's FP32 path on the same matrix
     fp32_ms = None
@@ -720,9 +719,8 @@ def run_ours(args):
                          "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
                          "kernel": "%s symmetric product (%d tensor-core product%s per launch%s), timed alone: "
                                    "%.4f ms" % (kprec, products, "s" if products > 1 else "",
-                                                "" if prec == "fp32" else ", SM pairs", gemm_ms),
-                         "peak_source": "%s bf16 burst (MEASURED_PEAKS.json)%s"
-                                        % (peak_src, ", x0.5 nominal tf32/bf16 ratio" if prec == "fp32" else ""),
+                                                ", SM pairs", gemm_ms),
+                         "peak_source": "%s bf16 burst (MEASURED_PEAKS.json)" % peak_src,
                          "algorithmic_flops_per_launch": alg_flops},
             "step_roofline": step_roofline(prec, n, ms_step, peaks["bf16_tflops"]),
             "tensor_pipe": tensor_pipe(prec, n),
@@ -736,7 +734,7 @@ def run_ours(args):
                               "std": statistics.pstdev(per_step), "min": min(per_step), "max": max(per_step)},
             "fp32_path": None if fp32_ms is None else {
                 "ms": fp32_ms, "speedup": fp32_ms / ms_step,
-                "what": "same library, precision fp32 (TF32x3 products, f~*_single, 31 products), same matrix"},
+                "what": "same library, precision fp32 (split FP16 products, f~*_single, 31 products), same matrix"},
             "clocks": clocks,
             "cpu_baseline": cpu,
             "accuracy": acc,

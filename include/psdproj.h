@@ -64,8 +64,10 @@ typedef enum {
 
 typedef enum {
   PSD_PREC_FP32 = 0,  /* f~*_single (Table 1), T = 10, 31 products; each product
-                         is three TF32 tensor-core products of the hi/lo split
-                         operands (Ootomo & Yokota 2022), FP32 accumulation */
+                         is three FP16 tensor-core products of hi/lo split
+                         operands (about 22 bits: FP16 pairs of the values times
+                         a power of two; the splitting of Ootomo & Yokota 2022),
+                         FP32 sums rounded to nearest every 128 terms */
   PSD_PREC_FP16 = 1,  /* f~*_half (Table 2), T = 7, 22 products, FP16 operands,
                          FP32 accumulation in tensor memory */
   PSD_PREC_BF16 = 2,  /* as FP16 with BF16 operands */
