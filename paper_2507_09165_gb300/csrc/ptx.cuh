@@ -1,7 +1,9 @@
 // Inline-PTX wrappers for the sm_103a tensor-core path: mbarriers, TMA tile
 // loads, tensor memory (tcgen05.alloc / mma / commit / ld) and the shared
 // memory matrix descriptor.  Written from the PTX ISA description of these
-// instructions; every wait is bounded (see wait_bounded).
+// instructions.  Waits on mbarriers are bounded (see wait_bounded); tensor-memory
+// allocation and cluster barriers have no bounded form, so what they wait for
+// is ordered by the code around them (see tmem_pair_setup).
 #pragma once
 #include <cuda.h>
 #include <cstdint>
@@ -265,6 +267,7 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Tensor memory of a CTA pair: one warp of each CTA performs these together.
+// Kernels call tmem_pair_setup / tmem_pair_teardown below, which order the two CTAs.
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
                : "memory");
@@ -274,6 +277,39 @@ __device__ __forceinline__ void tmem_relinquish_pair() {
 }
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+// Tensor memory of a CTA pair from start to end: every thread of both CTAs calls
+// both functions, warp 1 of each CTA allocates and frees.  An allocation is one
+// operation of two CTAs that blocks without a limit, so each step of one CTA that
+// the other's may depend on has a cluster barrier between them:
+//   before the allocation: both CTAs run (and have initialised their mbarriers);
+//     without it the leader's allocation can begin while the peer has not been
+//     started on its SM;
+//   before the permit is given up: both allocations are made;
+//   before the release: both CTAs have finished with tensor memory;
+//   after it: neither CTA leaves its SM while the other's release is under way.
+// Returns the address of the allocation (the same in both CTAs).
+__device__ __forceinline__ uint32_t tmem_pair_setup(volatile uint32_t* holder, uint32_t ncols) {
+  const bool alloc_warp = (threadIdx.x >> 5) == 1;
+  __syncwarp();
+  cluster_sync_all();
+  if (alloc_warp) tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(holder)), ncols);
+  tc_fence_before();
+  cluster_sync_all();
+  tc_fence_after();
+  if (alloc_warp) tmem_relinquish_pair();
+  return *holder;
+}
+__device__ __forceinline__ void tmem_pair_teardown(uint32_t tmem_base, uint32_t ncols) {
+  __syncwarp();
+  tc_fence_before();
+  cluster_sync_all();
+  if ((threadIdx.x >> 5) == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem_base, ncols);
+  }
+  __syncwarp();
+  cluster_sync_all();
 }
 // D[tmem of both SMs] (+)= A * B^T for the pair, issued by one thread of the leader.
 __device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,

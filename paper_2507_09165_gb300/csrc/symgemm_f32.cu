@@ -262,14 +262,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     tma_prefetch_desc(&tmBh);
     tma_prefetch_desc(&tmBl);
   }
-  if (warp == 1) tmem_alloc_pair(smem_u32(tmem_holder), kTmemCols);
-  tc_fence_before();
-  cluster_sync_all();  // both CTAs' barriers initialised and both allocations made
-  tc_fence_after();
-  // only now: nothing before the barrier orders one CTA giving up the permit against
-  // the other CTA's allocation
-  if (warp == 1) tmem_relinquish_pair();
-  const uint32_t tmem_base = *tmem_holder;
+  const uint32_t tmem_base = tmem_pair_setup(tmem_holder, kTmemCols);
 
   if (warp < 4) {
     reg_dec<kRegsIo>();
@@ -303,6 +296,14 @@ __global__ void __launch_bounds__(kThreadsF, 1)
               s = 0;
               ph ^= 1u;
             }
+          }
+        }
+        // the ring's last commits have arrived: none is on its way to a CTA that has left
+        for (int q = 0; ok && q < kStagesF; ++q) {
+          ok = wait_bounded(empty_bar(s), ph ^ 1u, abort_flag);
+          if (++s == kStagesF) {
+            s = 0;
+            ph ^= 1u;
           }
         }
         if (!ok && issued) {
@@ -485,12 +486,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
 
   // every operand read, remote arrival and copy of the pair is complete
   // before either CTA releases tensor memory or exits
-  tc_fence_before();
-  cluster_sync_all();
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc_pair(tmem_base, kTmemCols);
-  }
+  tmem_pair_teardown(tmem_base, kTmemCols);
   if (threadIdx.x == 0 && *abort_flag) raise_status(p.ep.status, PSD_ERR_TIMEOUT);
 }
 

@@ -386,24 +386,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     tma_prefetch_desc(&tmBh);
     if (!B1) tma_prefetch_desc(&tmBl);
   }
-  if (warp == 1) {
-    if (PAIR) {
-      tmem_alloc_pair(smem_u32(tmem_holder), kTmemCols);
-    } else {
+  uint32_t tmem_base;
+  if constexpr (PAIR) {
+    tmem_base = tmem_pair_setup(tmem_holder, kTmemCols);
+  } else {
+    if (warp == 1) {
       tmem_alloc(smem_u32(tmem_holder), kTmemCols);
       tmem_relinquish();
     }
-  }
-  tc_fence_before();
-  if (PAIR)
-    cluster_sync_all();  // both CTAs' barriers initialised and both allocations made
-  else
+    tc_fence_before();
     __syncthreads();
-  tc_fence_after();
-  // only now: nothing before the barrier orders one CTA giving up the permit against
-  // the other CTA's allocation
-  if (PAIR && warp == 1) tmem_relinquish_pair();
-  const uint32_t tmem_base = *tmem_holder;
+    tc_fence_after();
+    tmem_base = *tmem_holder;
+  }
   constexpr bool TF32 = ET == DT_TF32X3;
   constexpr int kKElems = X3Cfg<B1>::kRowBytes / (TF32 ? 4 : 2);  // K elements per stage
   constexpr int kKStep = TF32 ? 8 : 16;    // K per MMA instruction (32 bytes)
@@ -445,6 +440,16 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!B1) tma_load_2d(base + 2 * kABytes + kBBytes, &tmBl, kb * kKElems, yb, full_bar(s));
           }
           last_parity[s] = static_cast<int>(ph);
+          if (++s == kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      if constexpr (PAIR) {
+        // the ring's last commits have arrived: none is on its way to a CTA that has left
+        for (int q = 0; ok && q < kStages; ++q) {
+          ok = wait_bounded(empty_bar(s), ph ^ 1u, abort_flag);
           if (++s == kStages) {
             s = 0;
             ph ^= 1u;
@@ -707,17 +712,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   // pair form: every operand read, remote arrival and copy of the pair is
   // complete before either CTA releases tensor memory or exits
-  tc_fence_before();
-  if (PAIR)
-    cluster_sync_all();
-  else
+  if constexpr (PAIR) {
+    tmem_pair_teardown(tmem_base, kTmemCols);
+  } else {
+    tc_fence_before();
     __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    if (PAIR)
-      tmem_dealloc_pair(tmem_base, kTmemCols);
-    else
+    if (warp == 1) {
+      tc_fence_after();
       tmem_dealloc(tmem_base, kTmemCols);
+    }
   }
   if (threadIdx.x == 0 && *abort_flag && p.ep.status) atomicCAS(p.ep.status, 0, PSD_ERR_TIMEOUT);
 }
