@@ -229,8 +229,8 @@ psd_status_t psd_symm_product(int64_t n, const void *A, const void *B, int64_t l
  *   - an arena of 16-bit rows (row length ldm = max_order rounded up to 64):
  *     a request of order n holds 4 n contiguous rows for X_0, two rotating
  *     iterates and the stage polynomial, the four matrices of one stage, and
- *     ceil(32 T / (2 ldm)) more for the shares of <out, X - out> of its T
- *     final-product tiles (T = nb (nb + 1), nb = ceil(n / 256), an upper bound);
+ *     ceil(64 T / (2 ldm)) more for the shares of <out, X - out> of its T
+ *     final-product tiles;
  *   - per-request records (argument block, device state, report), max_batch
  *     of them;
  *   - the Lanczos scratch of two preparation streams (norm bound of order up
@@ -246,6 +246,9 @@ psd_status_t psd_symm_product(int64_t n, const void *A, const void *B, int64_t l
  * in the same step, so a small request runs a whole stage per step while a
  * large one's products are spread over several steps (it always receives a
  * minimum share).  Requests that finish get their report in the same step.
+ * Served products run on single SMs, not on SM pairs as a direct call's do: beside
+ * the preparation streams the pair form has stalled for good (rarely), inside a
+ * tensor-memory allocation of two SMs that blocks without a limit.
  *
  * Results: each request's arithmetic (norm bound kernels, tile partition,
  * summation order, coefficients and roundings) is that of psd_project with the

@@ -77,9 +77,9 @@ struct BlockRec {
   int64_t db, dc, dy;
   // EPI_FINAL with EpiParams::cres unset: if set, the shares of <out, X - out>
   // of the tile at launch position t go to cres at the tile's position in the
-  // request's own tile list, t + cres_shift (a served request; 4 per 128-row
-  // tile; on SM pairs 2 EW per tile, EW epilogue warps: EW (2 (t + cres_shift) +
-  // rank) + warp).
+  // request's own tile list, t + cres_shift (a served request), EW per 128-row
+  // tile (EW epilogue warps); on SM pairs 2 EW per tile: EW (2 (t + cres_shift) +
+  // rank) + warp.
   double* cres;
   int64_t cres_shift;
 };
@@ -245,10 +245,11 @@ bool encode_tmap(CUtensorMap* map, int dtype, const void* base, int64_t n, int64
 // pair written to ep.C / ep.C_lo; -1: the operand type).
 // many_small: a launch over many small matrices (the blocks of a block-diagonal
 // cone, orders <= 1024), run with 8 epilogue warps and a 3-stage ring where an
-// instance exists.
+// instance exists.  final_warps: epilogue warps of EPI_FINAL, 4 or 8 (its shares
+// of <out, X - out> are one per warp of each tile).
 cudaError_t launch_symgemm(int dtype, int epi, const CUtensorMap& tmA, const CUtensorMap& tmB,
                            const GemmParams& p, int grid, cudaStream_t stream, int out_dtype = -1,
-                           bool many_small = false);
+                           bool many_small = false, int final_warps = 4);
 // The same product on CTA pairs (tcgen05.mma.cta_group::2, M = 256): tiles
 // from make_tile_list_pair, tmB with 128-row boxes (each CTA loads half of
 // B), p.idesc with M = 256; 16-bit operands; EPI_COPY / EPI_POLY / EPI_SCALE

@@ -9,8 +9,8 @@
 //   arena: rows of ldm 16-bit elements; a request of order n holds the 4 n
 //          rows [row, row + 4n): X_0, R1, P, R3 (X_0, the two rotating
 //          iterates, the stage polynomial), then the rows that hold the
-//          per-warp shares of <out, X - out> of its final product (4 doubles
-//          per tile, at the tile's position in the request's tile list).
+//          per-warp shares of <out, X - out> of its final product (8 doubles
+//          per 128-row tile, at the tile's position in the request's tile list).
 //
 // Stage t of a request (cur: X_{t-1}; R1/R3 alternate):
 //   cur = X_0 (t = 0), R1 (t odd), R3 (t even > 0);  Y = R1 (t even), R3 (t odd)
@@ -19,7 +19,11 @@
 // 16-bit symmetric tensor-core kernels of symgemm.cu over a block table with
 // per-block row offsets and coefficients, so one launch covers every running
 // request whatever its stage; a step spreads large products over several
-// launches under a work budget (enqueue_step).  The norm bound runs on a preparation stream
+// launches under a work budget (enqueue_step).  They run in the one-SM form:
+// on SM pairs (the single projection's form) served steps beside the preparation
+// streams stalled for good a few times in thousands of bursts, in one recorded case inside the
+// pair's tensor-memory allocation, which blocks without a limit; the one-SM
+// allocation involves no other CTA.  Elements have the same bits in both forms.  The norm bound runs on a preparation stream
 // ("lane") with the single-projection kernels, replayed from a CUDA graph per
 // (lane, n); its result is copied into the request's record.
 #include <algorithm>
@@ -76,9 +80,9 @@ struct Request {
   int g = 0;         // product of the stage in progress: 0 Y, 1 P, 2 X_t, 3 final
   int k = 0;         // tiles of that product done
   int ntiles = 0;    // bound on the tile count (admission)
-  std::vector<int4> tl;   // tile list of order n: 256 x 256 tiles on SM pairs (make_tile_list_pair)
-  std::vector<int4> tlf;  // the final product's: the single projection's tiles (pair_tile_width), in its order
-  double* cres = nullptr;  // shares of <out, X - out>, 16 per tile of tlf (arena rows after the matrices)
+  std::vector<int4> tl;   // tile list of order n (make_tile_list)
+  std::vector<int4> tlf;  // the final product's (final_tile_list)
+  double* cres = nullptr;  // shares of <out, X - out>, 8 per tile of tlf (arena rows after the matrices)
   Clock::time_point t_submit;
   double latency_ms = 0.0;
   psd_info_t info{};
@@ -125,11 +129,21 @@ struct RowAllocator {
 // The tiles of a request's product g (3: the final product).
 const std::vector<int4>& list_of(const Request* r, int g) { return g == 3 ? r->tlf : r->tl; }
 
-// Tiles of the final product of a request of order n.
+// Tiles of the final product of a request of order n: the single projection's
+// 256-row tiles (pair_tile_width) in its order, each as its two 128-row halves, so
+// that with 8 epilogue warps a tile's per-warp shares of <out, X - out> are those
+// of one CTA of the single projection's SM pair, at the same positions.  A half
+// that lies below the order or the diagonal keeps its place and writes zeros.
+std::vector<int4> final_tile_list(int64_t n) {
+  std::vector<int4> tiles;
+  for (const int4& t : make_tile_list_pair(n, 0, 8, pair_tile_width(n)))
+    for (int h = 0; h < 2; ++h) tiles.push_back(make_int4(t.x + 128 * h, t.y, t.z, t.w));
+  return tiles;
+}
 int64_t final_tiles_of(int64_t n) {
   const int64_t w = pair_tile_width(n);
   int64_t tiles = 0;
-  for (int64_t m0 = 0; m0 < n; m0 += 256) tiles += (n - m0 + w - 1) / w;
+  for (int64_t m0 = 0; m0 < n; m0 += 256) tiles += 2 * ((n - m0 + w - 1) / w);
   return tiles;
 }
 
@@ -140,10 +154,10 @@ int64_t tiles_of(int64_t n) {
 }
 
 // Arena rows of a request of order n: its four matrices, then its shares of
-// <out, X - out> (16 doubles per tile of the final product) in whole rows of ldm
+// <out, X - out> (8 doubles per tile of the final product) in whole rows of ldm
 // 16-bit elements.
 int64_t rows_of(int64_t ldm, int64_t n) {
-  const int64_t share_bytes = 16 * static_cast<int64_t>(sizeof(double)) * final_tiles_of(n);
+  const int64_t share_bytes = 8 * static_cast<int64_t>(sizeof(double)) * final_tiles_of(n);
   return 4 * n + (share_bytes + 2 * ldm - 1) / (2 * ldm);
 }
 
@@ -167,7 +181,7 @@ struct psd_server {
   uint8_t* h_stage[psd::kRing] = {};
   size_t stage_bytes = 0;
   uint16_t* arena = nullptr;
-  CUtensorMap tmA[2], tmB[2];  // [0] FP16, [1] BF16 views of the arena (128-row boxes: the pair form)
+  CUtensorMap tmA[2], tmB[2];  // [0] FP16, [1] BF16 views of the arena (128- and 256-row boxes)
   // streams and events
   cudaStream_t main = nullptr;
   cudaStream_t lane[psd::kLanes] = {};
@@ -215,7 +229,7 @@ __global__ void adopt_kernel(DevArgs* dst_args, DevState* dst_st, const DevArgs*
 }
 
 // A request that finishes in a step: its record slot and its shares of
-// <out, X - out> (ncompl = 16 per tile of the final product).
+// <out, X - out> (ncompl = 8 per tile of the final product).
 struct FinRec {
   int slot;
   int ncompl;
@@ -379,13 +393,13 @@ cudaError_t step_gemm(psd_server* s, int dti, int epi, const BlockRec* d_blocks,
   g.ep.per_block_coef = 1;
   g.ep.absmax_blocks = epi == EPI_SCALE ? 2 : 0;
   const uint32_t fmt = dti == 1 ? 1u : 0u;
-  g.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | (16u << 24);  // M = 256: tiles on SM pairs
+  g.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | (8u << 24);  // M = 128; N per tile
   ++launches;
-  // SM pairs with 4 epilogue warps per CTA: served steps mix large requests,
-  // whose long main loops want the 6-stage ring; the final product has 8, as in
-  // the single projection (its shares are per warp)
-  return launch_symgemm_pair(dti == 1 ? DT_BF16 : DT_F16, epi, s->tmA[dti], s->tmB[dti], g, num_sms(), s->main, -1,
-                             epi == EPI_FINAL);
+  // 4 epilogue warps: served steps mix large requests, whose main loops want the
+  // 4-stage ring; the final product has 8, as in the single projection (its shares
+  // are per warp)
+  return launch_symgemm(dti == 1 ? DT_BF16 : DT_F16, epi, s->tmA[dti], s->tmB[dti], g, num_sms(), s->main, -1,
+                        /*many_small=*/false, /*final_warps=*/8);
 }
 
 // Builds and enqueues one scheduler step over `run`.  A step is one grouped
@@ -474,7 +488,7 @@ bool enqueue_step(psd_server* s, const std::vector<Request*>& run, int& launches
   int64_t budget = kStepBudget;
   for (int i : order) {
     Request* r = run[i];
-    const int64_t cost = 2 * ((r->n + 63) / 64);  // K-blocks of 64 per 256-row tile (two 128-row tiles)
+    const int64_t cost = (r->n + 63) / 64;  // K-blocks of 64 per tile
     Cursor c{r->stage, r->g, r->k, false};
     bool any = false;
     for (;;) {
@@ -531,7 +545,7 @@ bool enqueue_step(psd_server* s, const std::vector<Request*>& run, int& launches
   int nf = 0;
   for (int i = 0; i < nrun; ++i)
     if (next[i].done) {
-      hfin[nf++] = FinRec{run[i]->slot, 16 * static_cast<int>(run[i]->tlf.size()), run[i]->cres};
+      hfin[nf++] = FinRec{run[i]->slot, 8 * static_cast<int>(run[i]->tlf.size()), run[i]->cres};
       fin_ids.push_back(run[i]->id);
     }
   {
@@ -769,18 +783,18 @@ extern "C" psd_status_t psd_server_create(size_t hbm_budget_bytes, int32_t devic
   const size_t row_bytes = static_cast<size_t>(s->ldm) * 2;
   const size_t lane_bytes = round_up(kLaneHead + lanczos_bytes(max_order), 1024);
   const size_t recs_bytes = round_up(kRecBytes * max_batch, 1024);
-  // tile capacity: sum over requests of tiles_of(n) <= (max_order/256 + 3) rows/1024 + 80 max_batch (small
-  // orders' final products have up to one tile per SM pair)
+  // tile capacity: sum over requests of tiles_of(n) <= (max_order/256 + 3) rows/1024 + 160 max_batch (small
+  // orders' final products have up to one tile per SM)
   auto fixed_for = [&](int64_t tile_cap) {
     return 1024 + recs_bytes + kLanes * lane_bytes + kRing * round_up(stage_layout(max_batch, tile_cap).total, 1024);
   };
   int64_t rows = 0;
-  int64_t tile_cap = 80 * max_batch;
+  int64_t tile_cap = 160 * max_batch;
   for (int it = 0; it < 3; ++it) {  // rows and tile capacity depend on each other; settle them
     const size_t fixed = fixed_for(tile_cap);
     rows = hbm_budget_bytes > fixed ? static_cast<int64_t>((hbm_budget_bytes - fixed) / row_bytes) : 0;
     rows = std::min(rows, kMaxArenaRows);
-    tile_cap = 80 * static_cast<int64_t>(max_batch) + (max_order / 256 + 3) * (rows / 1024 + 1);
+    tile_cap = 160 * static_cast<int64_t>(max_batch) + (max_order / 256 + 3) * (rows / 1024 + 1);
   }
   while (rows > 0 && fixed_for(tile_cap) + static_cast<size_t>(rows) * row_bytes > hbm_budget_bytes) --rows;
   if (rows < rows_of(s->ldm, max_order)) {
@@ -820,7 +834,7 @@ extern "C" psd_status_t psd_server_create(size_t hbm_budget_bytes, int32_t devic
     ok = cudaEventCreateWithFlags(&s->prep_ev[k], cudaEventDisableTiming) == cudaSuccess;
   for (int d = 0; ok && d < 2; ++d)
     ok = encode_tmap_rows(&s->tmA[d], d ? DT_BF16 : DT_F16, s->arena, s->ldm, rows, s->ldm, 128) &&
-         encode_tmap_rows(&s->tmB[d], d ? DT_BF16 : DT_F16, s->arena, s->ldm, rows, s->ldm, 128);
+         encode_tmap_rows(&s->tmB[d], d ? DT_BF16 : DT_F16, s->arena, s->ldm, rows, s->ldm, 256);
   ok = ok && cudaDeviceSynchronize() == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -858,8 +872,8 @@ extern "C" psd_status_t psd_server_submit(psd_server_t* s, int64_t n, const floa
   r->ready = reinterpret_cast<cudaEvent_t>(ready);
   r->ntiles = static_cast<int>(tiles_of(n));
   if (n > 0) {
-    r->tl = make_tile_list_pair(n, 0);
-    r->tlf = make_tile_list_pair(n, 0, 8, pair_tile_width(n));
+    r->tl = make_tile_list(n);
+    r->tlf = final_tile_list(n);
   }
   r->t_submit = Clock::now();
   {

@@ -302,7 +302,7 @@ template <int EPI, bool IN8, int OUTK, int EW = 4>
 __global__ void __launch_bounds__(threads16(EW), 1)
     symgemm16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const GemmParams p, const int bf16_flag) {
-  static_assert(EW == 4 || (EW == 8 && EPI != EPI_FINAL), "8 epilogue warps: stage products only");
+  static_assert(EW == 4 || EW == 8, "4 or 8 epilogue warps");
   constexpr int kStages16 = stages16(EW);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -491,7 +491,9 @@ __global__ void __launch_bounds__(threads16(EW), 1)
       // position in the block's own list (served requests)
       double* cdst = nullptr;
       if (EPI == EPI_FINAL)
-        cdst = p.ep.cres ? p.ep.cres + 4 * t : br.cres ? br.cres + 4 * (t + br.cres_shift) : nullptr;
+        cdst = p.ep.cres ? p.ep.cres + EW * static_cast<int64_t>(t)
+               : br.cres ? br.cres + EW * (static_cast<int64_t>(t) + br.cres_shift)
+                         : nullptr;
       ComplAcc cacc;
       ComplAcc* cap = cdst ? &cacc : nullptr;
 #pragma unroll 1
@@ -511,7 +513,7 @@ __global__ void __launch_bounds__(threads16(EW), 1)
       }
       if (EPI == EPI_FINAL && cdst) {
         const double cs = compl_warp_sum(cacc);
-        if (lane == 0) cdst[ew] = cs;
+        if (lane == 0) cdst[EW == 4 ? ew : ewi] = cs;
       }
       tc_fence_before();
       __syncwarp();
@@ -1095,7 +1097,7 @@ Kernel16 kernel16_for8(int epi, int outk) {
     return epi == EPI_COPY    ? symgemm16_kernel<EPI_COPY, false, 0, 8>
            : epi == EPI_POLY  ? symgemm16_kernel<EPI_POLY, false, 0, 8>
            : epi == EPI_SCALE ? symgemm16_kernel<EPI_SCALE, false, 0, 8>
-                              : nullptr;
+                              : symgemm16_kernel<EPI_FINAL, false, 0, 8>;
   if (outk == 2)
     return epi == EPI_COPY ? symgemm16_kernel<EPI_COPY, false, 2, 8>
            : epi == EPI_POLY ? symgemm16_kernel<EPI_POLY, false, 2, 8>
@@ -1378,7 +1380,8 @@ cudaError_t launch_symgemm_chain(int dtype, const ChainMaps& maps, const ChainPr
 }
 
 cudaError_t launch_symgemm(int dtype, int epi, const CUtensorMap& tmA, const CUtensorMap& tmB,
-                           const GemmParams& p, int grid, cudaStream_t stream, int out_dtype, bool many_small) {
+                           const GemmParams& p, int grid, cudaStream_t stream, int out_dtype, bool many_small,
+                           int final_warps) {
   if (p.num_tiles == 0) return cudaSuccess;
   if (dtype != DT_F16 && dtype != DT_BF16 && dtype != DT_E4M3) return cudaErrorNotSupported;
   if (out_dtype < 0) out_dtype = dtype;
@@ -1386,9 +1389,10 @@ cudaError_t launch_symgemm(int dtype, int epi, const CUtensorMap& tmA, const CUt
   const bool in8 = dtype == DT_E4M3;
   const int outk = epi == EPI_FINAL ? 0 : out_dtype == DT_E4M3 ? 1 : out_dtype == DT_F16X2 ? 2 : 0;
   if (outk == 2 && dtype != DT_F16) return cudaErrorNotSupported;
-  // 8 epilogue warps where the launch has one (the final product keeps 4: its
-  // per-warp shares of <out, X - out> are four per tile)
-  Kernel16 k8 = many_small && !in8 ? kernel16_for8(epi, outk) : nullptr;
+  // 8 epilogue warps where the launch has an instance; the final product's number is
+  // the caller's, who sums the per-warp shares of <out, X - out>
+  const bool want8 = epi == EPI_FINAL ? final_warps == 8 : many_small;
+  Kernel16 k8 = want8 && !in8 ? kernel16_for8(epi, outk) : nullptr;
   const int ew = k8 ? 8 : 4;
   Kernel16 k = k8 ? k8 : kernel16_for(epi, in8, outk);
   if (!k) return cudaErrorNotSupported;

@@ -67,3 +67,11 @@ def test_kernels_on_pairs_use_nothing_else():
                           r"ok = wait_bounded\(empty_bar\(s\), ph \^ 1u, abort_flag\);", tail)
             assert m and m.start() < tail.index("tmem_pair_teardown("), name
     assert kernels == 3
+
+
+def test_served_steps_run_on_single_sms():
+    # beside the server's other streams no pair's allocation is made at all
+    code = _sources()["server.cu"]
+    for launch in ("launch_symgemm_pair(", "launch_symgemm_x3(", "launch_symgemm_f32("):
+        assert launch not in code
+    assert "launch_symgemm(" in code
