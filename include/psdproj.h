@@ -228,13 +228,11 @@ psd_status_t psd_symm_product(int64_t n, const void *A, const void *B, int64_t l
  * creation into
  *   - an arena of 16-bit rows (row length ldm = max_order rounded up to 64):
  *     a request of order n holds 4 n contiguous rows for X_0, two rotating
- *     iterates and the stage polynomial, the four matrices of one stage, and
- *     ceil(64 T / (2 ldm)) more for the shares of <out, X - out> of its T
- *     final-product tiles;
+ *     iterates and the stage polynomial, the four matrices of one stage;
  *   - per-request records (argument block, device state, report), max_batch
  *     of them;
  *   - the Lanczos scratch of two preparation streams (norm bound of order up
- *     to max_order each).
+ *     to max_order each), or of one where two leave too few rows.
  * A host thread admits queued requests in arrival order while their rows and
  * a record fit, runs their norm bound and X_0 = X / lam~ on a preparation
  * stream, and lets each join the running set at the next step.  A scheduler

@@ -2,15 +2,17 @@
 // layer around Algorithm 2; the paper itself projects one matrix at a time).
 //
 // Device memory (one allocation of the caller's HBM budget):
-//   [launch status | records | lane scratch x kLanes | staging x kRing | arena]
+//   [launch status | records | lane scratch x lanes | staging x kRing | arena]
 //   record (per admitted request): DevArgs | DevState | psd_info_t
 //   lane scratch: DevArgs | DevState | Lanczos buffers of order max_order
 //   staging: the block tables and tile lists of one scheduler step
 //   arena: rows of ldm 16-bit elements; a request of order n holds the 4 n
 //          rows [row, row + 4n): X_0, R1, P, R3 (X_0, the two rotating
-//          iterates, the stage polynomial), then the rows that hold the
-//          per-warp shares of <out, X - out> of its final product (8 doubles
-//          per 128-row tile, at the tile's position in the request's tile list).
+//          iterates, the stage polynomial).  The final product reads X_0 and the
+//          last iterate only; P's rows then take its per-warp shares of
+//          <out, X - out> (8 doubles per 128-row tile, at the tile's position in
+//          the request's tile list: at most 2 ceil(n/256) ceil(n/32) tiles of 64
+//          bytes, in 2 n ldm >= 128 n bytes).
 //
 // Stage t of a request (cur: X_{t-1}; R1/R3 alternate):
 //   cur = X_0 (t = 0), R1 (t odd), R3 (t even > 0);  Y = R1 (t even), R3 (t odd)
@@ -42,7 +44,7 @@
 namespace psd {
 namespace {
 
-constexpr int kLanes = 2;            // preparation streams
+constexpr int kLanes = 2;            // preparation streams (one where the budget has no room for two)
 constexpr int kRing = 2;             // scheduler steps in flight
 constexpr size_t kRecBytes = 1280;   // DevArgs (256) | DevState (768) | psd_info_t (256)
 constexpr size_t kLaneHead = 1024;   // DevArgs (256) | DevState (768)
@@ -82,7 +84,7 @@ struct Request {
   int ntiles = 0;    // bound on the tile count (admission)
   std::vector<int4> tl;   // tile list of order n (make_tile_list)
   std::vector<int4> tlf;  // the final product's (final_tile_list)
-  double* cres = nullptr;  // shares of <out, X - out>, 8 per tile of tlf (arena rows after the matrices)
+  double* cres = nullptr;  // shares of <out, X - out>, 8 per tile of tlf (in P's rows)
   Clock::time_point t_submit;
   double latency_ms = 0.0;
   psd_info_t info{};
@@ -140,26 +142,17 @@ std::vector<int4> final_tile_list(int64_t n) {
     for (int h = 0; h < 2; ++h) tiles.push_back(make_int4(t.x + 128 * h, t.y, t.z, t.w));
   return tiles;
 }
-int64_t final_tiles_of(int64_t n) {
-  const int64_t w = pair_tile_width(n);
-  int64_t tiles = 0;
-  for (int64_t m0 = 0; m0 < n; m0 += 256) tiles += 2 * ((n - m0 + w - 1) / w);
-  return tiles;
-}
 
-// Bound on the tiles of any product of a request of order n.
+// Bound on the tiles of a stage product of a request of order n (two 128-row tiles
+// per upper 256 x 256 block); a small order's final product can have more
+// (enqueue_step keeps a step's tiles within its staging).
 int64_t tiles_of(int64_t n) {
   const int64_t nb = (n + 255) / 256;
-  return std::max(nb * (nb + 1), final_tiles_of(n));
+  return nb * (nb + 1);
 }
 
-// Arena rows of a request of order n: its four matrices, then its shares of
-// <out, X - out> (8 doubles per tile of the final product) in whole rows of ldm
-// 16-bit elements.
-int64_t rows_of(int64_t ldm, int64_t n) {
-  const int64_t share_bytes = 8 * static_cast<int64_t>(sizeof(double)) * final_tiles_of(n);
-  return 4 * n + (share_bytes + 2 * ldm - 1) / (2 * ldm);
-}
+// Arena rows of a request of order n: its four matrices.
+int64_t rows_of(int64_t n) { return 4 * n; }
 
 struct StepDone;
 
@@ -176,6 +169,7 @@ struct psd_server {
   uint8_t* mem = nullptr;
   int* d_launch_status = nullptr;
   uint8_t* recs = nullptr;
+  int lanes = psd::kLanes;
   uint8_t* lane_mem[psd::kLanes] = {};
   uint8_t* d_stage[psd::kRing] = {};
   uint8_t* h_stage[psd::kRing] = {};
@@ -297,7 +291,7 @@ void CUDART_CB on_step_done(void* arg) {
       r->info = d->infos[k];
       r->latency_ms = std::chrono::duration<double, std::milli>(now - r->t_submit).count();
       r->state = RQ_DONE;
-      s->rows_alloc.release(r->row, rows_of(s->ldm, r->n));
+      s->rows_alloc.release(r->row, rows_of(r->n));
       s->tiles_held -= r->ntiles;
       s->free_slots.push_back(r->slot);
       s->lat.push_back(r->latency_ms);
@@ -410,7 +404,8 @@ cudaError_t step_gemm(psd_server* s, int dti, int epi, const BlockRec* d_blocks,
 // small request runs a whole stage per step.  Requests are visited smallest
 // first against a work budget of kStepBudget tile-K-blocks, which bounds the
 // step's duration; a request the budget does not reach still gets
-// kStepBudget / kQuantumDiv worth of tiles, so large requests always progress.
+// kStepBudget / kQuantumDiv worth of tiles, so large requests always progress
+// (as far as the step's staging goes, which always has a tile for each).
 // Every tile's arithmetic is the same whichever launch computes it.
 // Between building the step and enqueueing its GPU work the running set moves
 // on, so that the completion callback never sees a request that is still
@@ -486,8 +481,10 @@ bool enqueue_step(psd_server* s, const std::vector<Request*>& run, int& launches
   for (int i = 0; i < nrun; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return run[a]->n < run[b]->n; });
   int64_t budget = kStepBudget;
+  int64_t room = 4 * s->tile_cap - nrun;  // staging, less a tile for each request
   for (int i : order) {
     Request* r = run[i];
+    ++room;
     const int64_t cost = (r->n + 63) / 64;  // K-blocks of 64 per tile
     Cursor c{r->stage, r->g, r->k, false};
     bool any = false;
@@ -496,7 +493,9 @@ bool enqueue_step(psd_server* s, const std::vector<Request*>& run, int& launches
       const int rem = nt - c.k;
       int64_t m = std::min<int64_t>(rem, std::max<int64_t>(budget, 0) / cost);
       if (m <= 0 && !any) m = std::min<int64_t>(rem, std::max<int64_t>(1, kStepBudget / kQuantumDiv / cost));
+      m = std::min(m, room);
       if (m <= 0) break;
+      room -= m;
       parts[c.g].push_back({i, c.k, c.k + static_cast<int>(m)});
       any = true;
       budget -= m * cost;
@@ -599,13 +598,13 @@ bool enqueue_step(psd_server* s, const std::vector<Request*>& run, int& launches
 // stops the scheduler; the GPU work already enqueued is drained first.
 void fail_all(psd_server* s) {
   cudaStreamSynchronize(s->main);
-  for (int l = 0; l < kLanes; ++l) cudaStreamSynchronize(s->lane[l]);
+  for (int l = 0; l < s->lanes; ++l) cudaStreamSynchronize(s->lane[l]);
   std::lock_guard<std::mutex> lk(s->mu);
   for (auto* v : {&s->prep, &s->run})
     for (Request* r : *v) {
       r->info.status = PSD_ERR_CUDA;
       r->state = RQ_DONE;
-      s->rows_alloc.release(r->row, rows_of(s->ldm, r->n));
+      s->rows_alloc.release(r->row, rows_of(r->n));
       s->tiles_held -= r->ntiles;
       s->free_slots.push_back(r->slot);
     }
@@ -632,16 +631,16 @@ void scheduler(psd_server* s) {
         while (!s->queue.empty()) {
           Request* r = s->queue.front();
           if (s->free_slots.empty() || s->tiles_held + r->ntiles > s->tile_cap) break;
-          const int64_t row = s->rows_alloc.alloc(rows_of(s->ldm, r->n));
+          const int64_t row = s->rows_alloc.alloc(rows_of(r->n));
           if (row < 0) break;
           s->peak_rows = std::max(s->peak_rows, s->rows_alloc.used);
           r->row = row;
-          r->cres = reinterpret_cast<double*>(s->arena + (row + 4 * r->n) * s->ldm);
+          r->cres = reinterpret_cast<double*>(s->arena + (row + 2 * r->n) * s->ldm);  // P's rows
           r->slot = s->free_slots.back();
           s->free_slots.pop_back();
           s->tiles_held += r->ntiles;
           r->lane = s->lane_next;
-          s->lane_next = (s->lane_next + 1) % kLanes;
+          s->lane_next = (s->lane_next + 1) % s->lanes;
           r->state = RQ_PREP;
           s->queue.pop_front();
           admitted.push_back(r);
@@ -783,21 +782,23 @@ extern "C" psd_status_t psd_server_create(size_t hbm_budget_bytes, int32_t devic
   const size_t row_bytes = static_cast<size_t>(s->ldm) * 2;
   const size_t lane_bytes = round_up(kLaneHead + lanczos_bytes(max_order), 1024);
   const size_t recs_bytes = round_up(kRecBytes * max_batch, 1024);
-  // tile capacity: sum over requests of tiles_of(n) <= (max_order/256 + 3) rows/1024 + 160 max_batch (small
-  // orders' final products have up to one tile per SM)
+  // tile capacity: sum over requests of tiles_of(n) <= (max_order/256 + 3) rows/1024 + 2 max_batch
   auto fixed_for = [&](int64_t tile_cap) {
-    return 1024 + recs_bytes + kLanes * lane_bytes + kRing * round_up(stage_layout(max_batch, tile_cap).total, 1024);
+    return 1024 + recs_bytes + s->lanes * lane_bytes + kRing * round_up(stage_layout(max_batch, tile_cap).total, 1024);
   };
-  int64_t rows = 0;
-  int64_t tile_cap = 160 * max_batch;
-  for (int it = 0; it < 3; ++it) {  // rows and tile capacity depend on each other; settle them
-    const size_t fixed = fixed_for(tile_cap);
-    rows = hbm_budget_bytes > fixed ? static_cast<int64_t>((hbm_budget_bytes - fixed) / row_bytes) : 0;
-    rows = std::min(rows, kMaxArenaRows);
-    tile_cap = 160 * static_cast<int64_t>(max_batch) + (max_order / 256 + 3) * (rows / 1024 + 1);
+  int64_t rows = 0, tile_cap = 0;
+  for (s->lanes = kLanes; s->lanes >= 1; --s->lanes) {
+    tile_cap = 2 * max_batch;
+    for (int it = 0; it < 3; ++it) {  // rows and tile capacity depend on each other; settle them
+      const size_t fixed = fixed_for(tile_cap);
+      rows = hbm_budget_bytes > fixed ? static_cast<int64_t>((hbm_budget_bytes - fixed) / row_bytes) : 0;
+      rows = std::min(rows, kMaxArenaRows);
+      tile_cap = 2 * static_cast<int64_t>(max_batch) + (max_order / 256 + 3) * (rows / 1024 + 1);
+    }
+    while (rows > 0 && fixed_for(tile_cap) + static_cast<size_t>(rows) * row_bytes > hbm_budget_bytes) --rows;
+    if (rows >= rows_of(max_order)) break;
   }
-  while (rows > 0 && fixed_for(tile_cap) + static_cast<size_t>(rows) * row_bytes > hbm_budget_bytes) --rows;
-  if (rows < rows_of(s->ldm, max_order)) {
+  if (s->lanes == 0) {
     delete s;
     cudaSetDevice(prev);
     return PSD_ERR_NO_MEMORY;
@@ -818,14 +819,14 @@ extern "C" psd_status_t psd_server_create(size_t hbm_budget_bytes, int32_t devic
   p += 1024;
   s->recs = p;
   p += recs_bytes;
-  for (int l = 0; l < kLanes; ++l, p += lane_bytes) s->lane_mem[l] = p;
+  for (int l = 0; l < s->lanes; ++l, p += lane_bytes) s->lane_mem[l] = p;
   for (int k = 0; k < kRing; ++k, p += s->stage_bytes) s->d_stage[k] = p;
   s->arena = reinterpret_cast<uint16_t*>(p);
   for (int k = 0; ok && k < kRing; ++k) ok = cudaMallocHost(&s->h_stage[k], s->stage_bytes) == cudaSuccess;
   int lo = 0, hi = 0;
   cudaDeviceGetStreamPriorityRange(&lo, &hi);
   ok = ok && cudaStreamCreateWithPriority(&s->main, cudaStreamNonBlocking, lo) == cudaSuccess;
-  for (int l = 0; ok && l < kLanes; ++l)
+  for (int l = 0; ok && l < s->lanes; ++l)
     ok = cudaStreamCreateWithPriority(&s->lane[l], cudaStreamNonBlocking, hi) == cudaSuccess;
   for (int k = 0; ok && k < kRing; ++k)
     ok = cudaEventCreateWithFlags(&s->step_ev[k], cudaEventDisableTiming) == cudaSuccess;
@@ -995,7 +996,7 @@ extern "C" psd_status_t psd_server_destroy(psd_server_t* s) {
   cudaGetDevice(&prev);
   cudaSetDevice(s->device);
   cudaStreamSynchronize(s->main);  // host callbacks of the last steps have run after this
-  for (int l = 0; l < kLanes; ++l) cudaStreamSynchronize(s->lane[l]);
+  for (int l = 0; l < s->lanes; ++l) cudaStreamSynchronize(s->lane[l]);
   destroy_resources(s);
   cudaSetDevice(prev);
   return PSD_OK;
