@@ -65,14 +65,47 @@ constexpr int kFp8Stages = 2;
 constexpr float kFp8ScaleX = 256.f;
 constexpr float kFp8ScaleY = 256.f;
 
-// FP32 path: scales of the FP16 pairs.  |X_t(i,j)|, |Y(i,j)| <= their spectral
-// norms (~1.03 in the composite's basin) and |P(i,j)| <= a_1 = 8.3; entries of
-// a spread iterate are ~1/sqrt(n).  2^13 and 2^12 leave a factor 8 and 2 below
-// FP16's 65504, and put the lo parts' smallest step at 2^-37 and 2^-36 in place
-// of an unscaled pair's 2^-24 (which at n = 10,000 is coarser than the pair's
-// own 2^-23 relative step for every entry).
-constexpr float kF32ScaleX = 8192.f;
-constexpr float kF32ScaleP = 4096.f;
+// FP32 path: scales of the FP16 pairs.  A symmetric matrix's entries are at most
+// its spectral norm, and the norms follow from the coefficients: with the spectrum
+// of X_{t-1} in [-x, x], Y has norm x^2, P max |a + b y + c y^2| over y <= x^2 and
+// X_t max |z (a + b z^2 + c z^4)| / post over z <= x (Table 1: X_t up to 2.02, Y
+// 4.08, P 8.31).  Each matrix gets the largest power of two that keeps its norm a
+// factor kF32Headroom below FP16's 65504: 2^15 for X_0 and the last stages' X_t, 2^12
+// for the first P.  The lo parts' smallest step is then 2^-39 of X_0's bound
+// (2^-24 for an unscaled pair, which at n = 10,000 is coarser than the pair's own
+// 2^-23 relative step for every entry), so an entry keeps its 22 bits down to
+// 2^-17 of the bound; TF32 pairs keep theirs at every magnitude.  Relative error of
+// the smallest row of D A D, n = 1000, D from 1 to 1e-6: TF32 pairs 8.1e-5, these
+// 9.6e-5 (2^13 for every X_t and Y: 2.3e-4); of the whole matrix 5.8e-6 and 3.7e-6.
+constexpr double kF32Headroom = 1.8;
+
+struct F32Range {
+  double x = 1.0;      // norm of the stage's input iterate
+  double y, p, out;    // of Y, P and X_t
+  void stage(const double (&c)[3], double post) {
+    y = x * x;
+    p = out = 0.0;
+    auto poly = [&](double t) { return std::fabs(c[0] + c[1] * t + c[2] * t * t); };
+    auto at = [&](double t) {  // t = z^2 in [0, y]
+      if (!(t >= 0.0 && t <= y)) return;
+      p = std::max(p, poly(t));
+      out = std::max(out, std::sqrt(t) * poly(t) / post);
+    };
+    at(0.0);
+    at(y);
+    if (c[2] != 0.0) {
+      at(-c[1] / (2.0 * c[2]));  // P' = 0
+      const double d = 9.0 * c[1] * c[1] - 20.0 * c[0] * c[2];  // (z P)' = a + 3 b t + 5 c t^2 = 0
+      if (d >= 0.0)
+        for (double sgn : {-1.0, 1.0}) at((-3.0 * c[1] + sgn * std::sqrt(d)) / (10.0 * c[2]));
+    }
+  }
+};
+inline float f32_scale(double norm) {
+  double sc = 1.0;
+  while (2.0 * sc * norm * kF32Headroom <= 65504.0) sc *= 2.0;
+  return static_cast<float>(sc);
+}
 
 inline float fp8_poly_scale(const double (&c)[3]) {
   double m = 0.0;
@@ -148,23 +181,26 @@ cudaError_t run_chain(psd_precision_t prec, const Schedule& sched, int nslots, i
     m.slot = pool.alloc(kind_slots(kind));
     return m;
   };
-  Mat X0 = make(stage_kinds(prec, 0, T).x, kFp8ScaleX, kF32ScaleX);
+  F32Range range;
+  Mat X0 = make(stage_kinds(prec, 0, T).x, kFp8ScaleX, f32_scale(range.x));
   if (X0.slot < 0) return cudaErrorMemoryAllocation;
   if ((e = ops.cast(X0)) != cudaSuccess) return e;
   Mat cur = X0;
   for (int t = 0; t < T; ++t) {
     const StageKinds k = stage_kinds(prec, t, T);
-    Mat Y = make(k.y, kFp8ScaleY, kF32ScaleX);
+    range.stage(sched.coef[t], sched.post[t]);
+    Mat Y = make(k.y, kFp8ScaleY, f32_scale(range.y));
     if (Y.slot < 0) return cudaErrorMemoryAllocation;
     if ((e = ops.gemm(EPI_COPY, cur, cur, &Y, nullptr, 0.f, 0.f, 0.f, 1.f, false)) != cudaSuccess) return e;
-    Mat P = make(k.p, fp8_poly_scale(sched.coef[t]), kF32ScaleP);
+    Mat P = make(k.p, fp8_poly_scale(sched.coef[t]), f32_scale(range.p));
     if (P.slot < 0) return cudaErrorMemoryAllocation;
     if ((e = ops.gemm(EPI_POLY, Y, Y, &P, &Y, static_cast<float>(sched.coef[t][0]),
                       static_cast<float>(sched.coef[t][1]), static_cast<float>(sched.coef[t][2]), 1.f, false)) !=
         cudaSuccess)
       return e;
     pool.release(Y);
-    Mat Xn = make(k.out, kFp8ScaleX, kF32ScaleX);
+    Mat Xn = make(k.out, kFp8ScaleX, f32_scale(range.out));
+    range.x = range.out;
     if (Xn.slot < 0) return cudaErrorMemoryAllocation;
     if ((e = ops.gemm(EPI_SCALE, cur, P, &Xn, nullptr, 0.f, 0.f, 0.f, static_cast<float>(1.0 / sched.post[t]),
                       t == T - 1)) != cudaSuccess)

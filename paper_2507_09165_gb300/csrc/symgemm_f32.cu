@@ -4,7 +4,7 @@
 // A matrix M of the FP32 chain is stored as hi = RN16(2^s M), lo = RN16(2^s M -
 // hi): about 22 significant bits.  The power of two 2^s lifts the lo parts of
 // the iterates' entries (~1/sqrt(n)) out of FP16's subnormals, which otherwise
-// cap an unscaled pair at an absolute 2^-25 (chain.h kF32Scale*).  The products
+// cap an unscaled pair at an absolute 2^-25 (chain.h F32Range).  The products
 // run on SM pairs (tcgen05.mma.cta_group::2, M = 256) as in symgemm.cu and
 // symgemm_x3.cu, at the FP16 rate: twice that of the TF32 split.
 //
