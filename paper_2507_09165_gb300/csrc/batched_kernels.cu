@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "epilogue.cuh"
 #include "internal.h"
 #include "ptx.cuh"
 #include "tridiag.cuh"
@@ -917,10 +918,7 @@ __device__ __forceinline__ void bstore4(const BatchCast& c, int64_t pos, const f
     uint16_t l[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const float x = v[k] * c.scale;
-      const __half h = __float2half_rn(x);
-      u[k] = __half_as_ushort(h);
-      l[k] = __half_as_ushort(__float2half_rn(x - __half2float(h)));
+      split_h2_sat(v[k] * c.scale, u[k], l[k]);
     }
     put4_16(static_cast<uint16_t*>(c.M_lo) + pos, l, valid);
   } else {

@@ -1,12 +1,27 @@
 // Epilogue pieces shared by the product kernels (symgemm.cu, symgemm_f32.cu).
 #pragma once
 
+#include <cuda_fp16.h>
+
 #include "internal.h"
 
 namespace psd {
 
 __device__ __forceinline__ void raise_status(int* status, int code) {
   if (status) atomicCAS(status, 0, code);
+}
+
+// Two values as FP16, a in the low half: rounded to nearest, to +-65504 beyond
+// FP16's range (a NaN stays a NaN).
+__device__ __forceinline__ uint32_t pack_h2_sat(float a, float b) {
+  uint32_t r;
+  asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  return r;
+}
+// x as an FP16 pair hi + lo (bits), both saturating.
+__device__ __forceinline__ void split_h2_sat(float x, uint16_t& hi, uint16_t& lo) {
+  hi = static_cast<uint16_t>(pack_h2_sat(x, 0.f));
+  lo = static_cast<uint16_t>(pack_h2_sat(x - __half2float(__ushort_as_half(hi)), 0.f));
 }
 
 // Row stride (words) of a warp's 32 x 32 FP32 staging square.

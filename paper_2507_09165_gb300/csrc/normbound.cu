@@ -33,6 +33,7 @@
 #include <tuple>
 #include <type_traits>
 
+#include "epilogue.cuh"
 #include "internal.h"
 #include "normbound.cuh"
 #include "ptx.cuh"
@@ -833,10 +834,7 @@ __device__ __forceinline__ void store4(void* M, void* M_lo, int64_t pos, const f
     uint16_t l[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const float x = v[k] * scale;
-      const __half h = __float2half_rn(x);
-      u[k] = __half_as_ushort(h);
-      l[k] = __half_as_ushort(__float2half_rn(x - __half2float(h)));
+      split_h2_sat(v[k] * scale, u[k], l[k]);
     }
     put16(static_cast<uint16_t*>(M_lo) + pos, l, valid);
   } else {

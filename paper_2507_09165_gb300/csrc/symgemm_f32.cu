@@ -56,10 +56,7 @@ static_assert(smem_bytes_f32() <= 232448, "shared memory per CTA");
 // the leader's barrier: they are given this long to land before the CTA exits.
 constexpr unsigned long long kDrainNs = 200000ull;
 
-__device__ __forceinline__ uint32_t pack_h2(float a, float b) {
-  const __half2 h = __floats2half2_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
+__device__ __forceinline__ __half2 as_h2(uint32_t w) { return *reinterpret_cast<const __half2*>(&w); }
 __device__ __forceinline__ float2 unpack_h2(uint32_t w) { return __half22float2(*reinterpret_cast<const __half2*>(&w)); }
 
 // 8 consecutive pair elements (w[e] = hi | lo << 16) to memory, clipped at `valid`.
@@ -113,7 +110,7 @@ struct EpiOut {
   uint16_t *hi, *lo;         // the block's output pair
   const uint16_t *yh, *yl;   // EPI_POLY: the block's Y pair
   float cacc, cy, cdiag;     // stored value = cacc * acc + cy * (y_hi + y_lo) (+ cdiag on the diagonal)
-  float unscale;             // stored value -> value (max |X_T|)
+  float unscale;             // stored value -> value (the report's largest)
 };
 
 // One 32 x 32 chunk: lane l holds row r0 + l, v[j] the FP32 sum at column c0 + j.
@@ -132,6 +129,8 @@ __device__ __forceinline__ void epilogue_pair(const EpiOut& eo, int n, int64_t l
   const int r = r0 + lane;
   const bool diag = r0 == c0;
   const int seg = lane & 3, sr = lane >> 2;  // segment and row (+ 8 k) of the global accesses
+  const int nc = n - c0;                     // columns below the order, for the range check
+  __half2 big = __float2half2_rn(0.f);
   uint32_t w[32];                            // the lane's row: hi | lo << 16
   if (EPI == EPI_POLY) {
     uint4 yh[4], yl[4];
@@ -172,17 +171,23 @@ __device__ __forceinline__ void epilogue_pair(const EpiOut& eo, int n, int64_t l
       if (diag && 2 * q == lane) a += eo.cdiag;
       if (diag && 2 * q + 1 == lane) b += eo.cdiag;
     }
-    const uint32_t hi = pack_h2(a, b);
+    const uint32_t hi = pack_h2_sat(a, b);
+    if (2 * q < nc) big = __hmax2(big, __habs2(as_h2(2 * q + 1 < nc ? hi : hi & 0xFFFFu)));
     const float2 h = unpack_h2(hi);
-    const uint32_t lo = pack_h2(a - h.x, b - h.y);
+    const uint32_t lo = pack_h2_sat(a - h.x, b - h.y);
     w[2 * q] = __byte_perm(hi, lo, 0x5410);
     w[2 * q + 1] = __byte_perm(hi, lo, 0x7632);
   }
-  if (track && r < n) {
+  // a value beyond FP16 is stored as +-65504 (+ up to as much in lo): the iterates stay
+  // finite, and whatever the stage the report gives the size that did not fit
+  const float2 bg = __half22float2(big);
+  if (r < n && (track || fmaxf(bg.x, bg.y) == 65504.f)) {
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
       const float2 t = unpack_h2(w[j]);
-      if (c0 + j < n) amax_bits = max(amax_bits, __float_as_uint(fabsf((t.x + t.y) * eo.unscale)));
+      float m = fabsf(t.x + t.y);
+      if (EPI != EPI_POLY && fabsf(eo.cacc * v[j]) > 65504.f) m = fabsf(eo.cacc * v[j]);
+      if (c0 + j < n && (track || m >= 65504.f)) amax_bits = max(amax_bits, __float_as_uint(m * eo.unscale));
     }
   }
   __syncwarp();
@@ -394,7 +399,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       const int4 tc = p.tiles[t];
       const BlockRec& br = p.blocks[tc.z];
       const int n = br.n;
-      if (EPI != EPI_FINAL && track_launch && amax_block != tc.z) {
+      if (EPI != EPI_FINAL && amax_block != tc.z) {
         if (amax_block >= 0) flush_amax(amax_block);
         amax_block = tc.z;
       }
@@ -481,7 +486,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       }
       __syncwarp();
     }
-    if (EPI != EPI_FINAL && track_launch && amax_block >= 0) flush_amax(amax_block);
+    if (EPI != EPI_FINAL && amax_block >= 0) flush_amax(amax_block);
   }
 
   // every operand read, remote arrival and copy of the pair is complete
