@@ -40,8 +40,8 @@ struct BatchPlan {
   int* d_status = nullptr;
   int4* d_tiles = nullptr;
   int ntiles = 0;
-  // 256 x 256 tiles on SM pairs (FP16 / BF16 plans), chosen by the autotuner
-  // when faster than every schedule of the 128-row tiles
+  // 256 x 256 tiles on SM pairs: FP16 / BF16 plans, chosen by the autotuner when
+  // faster than every schedule of the 128-row tiles; FP32 plans, in the chosen order
   int4* d_tiles_pair = nullptr;
   int ntiles_pair = 0;
   bool pair = false;
@@ -111,11 +111,14 @@ void free_bplan(BatchPlan* p) {
 //   order 0: blocks largest first, each block's tiles in its grouped raster;
 //   order 1: all tiles by estimated cost (K-steps x width, plus a fixed
 //            epilogue share), dealt in boustrophedon rounds of `grid` tiles.
-// Index = 3 order + g, raster group kTileGroups[g].
+// Index = 3 order + g, raster group kTileGroups[g].  The FP32 path's products run
+// over 256 x 256 tiles on SM pairs (`pair`): the same orders, dealt in rounds of the
+// pairs; a block has at most 4 tile rows, so the raster groups are all alike there.
 constexpr int kTileGroups[3] = {4, 8, 16};
 constexpr int kNumSchedules = 6;
+static_assert(kMaxBatchOrder <= kTileGroups[0] * 256, "pair tiles: one raster group");
 
-std::vector<int4> schedule_tiles(const std::vector<int>& sizes, int cand, int grid) {
+std::vector<int4> schedule_tiles(const std::vector<int>& sizes, int cand, int grid, bool pair = false) {
   const int count = static_cast<int>(sizes.size());
   const int order = cand / 3, group = kTileGroups[cand % 3];
   std::vector<int> blocks(count);
@@ -123,7 +126,7 @@ std::vector<int4> schedule_tiles(const std::vector<int>& sizes, int cand, int gr
   std::stable_sort(blocks.begin(), blocks.end(), [&](int x, int y) { return sizes[x] > sizes[y]; });
   std::vector<int4> tiles;
   for (int b : blocks) {
-    std::vector<int4> tl = make_tile_list(sizes[b], b, group);
+    std::vector<int4> tl = pair ? make_tile_list_pair(sizes[b], b, group) : make_tile_list(sizes[b], b, group);
     tiles.insert(tiles.end(), tl.begin(), tl.end());
   }
   if (order == 0 || grid <= 1) return tiles;
@@ -141,19 +144,9 @@ std::vector<int4> schedule_tiles(const std::vector<int>& sizes, int cand, int gr
   return out;
 }
 
-// Pair-form tiles: blocks largest first, each block's 256 x 256 tiles in its
-// grouped raster (make_tile_list_pair).
-std::vector<int4> pair_tiles(const std::vector<int>& sizes) {
-  std::vector<int> blocks(sizes.size());
-  for (size_t b = 0; b < sizes.size(); ++b) blocks[b] = static_cast<int>(b);
-  std::stable_sort(blocks.begin(), blocks.end(), [&](int x, int y) { return sizes[x] > sizes[y]; });
-  std::vector<int4> tiles;
-  for (int b : blocks) {
-    std::vector<int4> tl = make_tile_list_pair(sizes[b], b, 8);
-    tiles.insert(tiles.end(), tl.begin(), tl.end());
-  }
-  return tiles;
-}
+// Pair-form tiles of the 16-bit plans: blocks largest first, each block's 256 x 256
+// tiles in its grouped raster.
+std::vector<int4> pair_tiles(const std::vector<int>& sizes) { return schedule_tiles(sizes, 0, 1, true); }
 constexpr int kPairCandidate = kNumSchedules;  // autotune candidate index of the pair form
 
 struct TuneReport {
@@ -568,7 +561,11 @@ cudaError_t enqueue_batch(BatchPlan* p, cudaStream_t s) {
 // product of the chain's first stage (median of 3 after a warm-up, on a
 // private stream; the slots hold zeros, which leaves the timing unchanged).
 psd_status_t tune_bplan(BatchPlan* p) {
-  const int grid = std::max(1, std::min(num_sms(), p->ntiles));
+  // FP32: the pair tiles in the candidates' orders; others: the 128-row tiles
+  const bool f32 = p->prec == PSD_PREC_FP32;
+  const int grid = f32 ? std::max(1, std::min(num_sms() / 2, p->ntiles_pair))
+                       : std::max(1, std::min(num_sms(), p->ntiles));
+  int4* d_sched = f32 ? p->d_tiles_pair : p->d_tiles;
   const auto key = tune_key(p);
   // the pair form: FP16 / BF16 plans (every product a 16-bit product), not with the chain form
   const bool pair_ok = (p->prec == PSD_PREC_FP16 || p->prec == PSD_PREC_BF16) && g_force_form != 1;
@@ -596,11 +593,14 @@ psd_status_t tune_bplan(BatchPlan* p) {
     float best = 0.f;
     bool ok = true;
     for (int c = 0; c < rep.ncand && ok; ++c) {
+      if (f32 && c % 3 != 0) {  // the same list as the order's first raster group
+        rep.ms[c] = rep.ms[c - 1];
+        continue;
+      }
       p->pair = c == kPairCandidate;
       if (!p->pair) {
-        const std::vector<int4> t = schedule_tiles(p->sizes, c, grid);
-        ok = cudaMemcpyAsync(p->d_tiles, t.data(), sizeof(int4) * t.size(), cudaMemcpyHostToDevice, ts) ==
-             cudaSuccess;
+        const std::vector<int4> t = schedule_tiles(p->sizes, c, grid, f32);
+        ok = cudaMemcpyAsync(d_sched, t.data(), sizeof(int4) * t.size(), cudaMemcpyHostToDevice, ts) == cudaSuccess;
       }
       float ms[3] = {};
       for (int r = -1; r < 3 && ok; ++r) {
@@ -624,12 +624,12 @@ psd_status_t tune_bplan(BatchPlan* p) {
     g_tuned[key] = chosen;
   }
   p->pair = chosen == kPairCandidate;
-  const std::vector<int4> t = schedule_tiles(p->sizes, p->pair ? 0 : chosen, grid);
-  if (cudaMemcpy(p->d_tiles, t.data(), sizeof(int4) * t.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+  const std::vector<int4> t = schedule_tiles(p->sizes, p->pair ? 0 : chosen, grid, f32);
+  if (cudaMemcpy(d_sched, t.data(), sizeof(int4) * t.size(), cudaMemcpyHostToDevice) != cudaSuccess)
     return PSD_ERR_CUDA;
   // each block's final-product shares, in the block's own tile order (schedule-independent
   // sums), positions in the tile list the final product runs over
-  const std::vector<int4> tf = p->on_pairs() ? pair_tiles(p->sizes) : t;
+  const std::vector<int4> tf = p->pair ? pair_tiles(p->sizes) : t;
   std::map<std::tuple<int, int, int>, int> pos;
   for (int i = 0; i < static_cast<int>(tf.size()); ++i) pos[std::make_tuple(tf[i].z, tf[i].x, tf[i].y)] = i;
   std::vector<int> cidx;
