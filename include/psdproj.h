@@ -421,6 +421,10 @@ psd_status_t psd_project_deflate(int64_t n, const float *X, int64_t ld, float *o
  *     once, so the bound and a projection built on it report PSD_ERR_TIMEOUT
  *     (every block of a batch; the kernel's CTAs leave at their next wait;
  *     nothing hangs or faults).
+ *     A direct bound of order up to 1152 runs on one thread-block cluster, whose
+ *     barriers are the hardware's and have no limit: there 0 gives up likewise
+ *     (orders above 32, which have more than one CTA's work) and other values
+ *     have no effect.
  * PSD_ERR_INVALID_ARG for an unknown knob or a value out of range,
  * PSD_ERR_CUDA if the copy to the device failed.  Synchronous. */
 #define PSD_DEBUG_BOUND_SCALE 1

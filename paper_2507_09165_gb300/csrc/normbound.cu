@@ -47,7 +47,8 @@ namespace {
 // none; a factor below 1 drives the chain past the composite's basin and
 // exercises the overshoot report) and the limit of the grid barriers' waits
 // (0: every barrier that is not already complete gives up at once and the
-// bound returns PSD_ERR_TIMEOUT).  Read by the kernels at run time, so
+// bound returns PSD_ERR_TIMEOUT; the cluster form, whose barriers are the
+// hardware's, takes up the limit 0 only).  Read by the kernels at run time, so
 // captured graphs see the current values.
 __device__ double g_debug_bound_scale = 1.0;
 __device__ unsigned long long g_debug_barrier_limit_ns = kWaitLimitNs;

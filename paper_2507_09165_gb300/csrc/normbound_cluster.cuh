@@ -255,6 +255,18 @@ __global__ void __launch_bounds__(kNT, 2) nb_cluster_kernel(const ClusterJob jb)
     }
   }
   cluster_sync_all();  // every CTA of the cluster runs before any remote store
+  // The cluster's barriers are the hardware's and have no limit of their own.  A wait
+  // limit of 0 (psd_debug_set) gives up here, where the other forms' first barrier
+  // does: one CTA alone (one chunk of 32 elements) has nobody to wait for.
+  if (g_debug_barrier_limit_ns == 0ull && nch > 1) {  // the same in every CTA
+    if (rank == 0 && tid == 0) {
+      st->m = st->done = 0;
+      st->maxdiag_bits = st->absmax_bits = 0;
+      st->sigma = st->resid = st->lambda = st->fro = st->maxdiag = st->inv_lambda = 0.0;
+      st->status = PSD_ERR_TIMEOUT;
+    }
+    return;
+  }
 
   // an element of the mat-vec input (0 past n) to every CTA
   auto put_vh = [&](int e, float h) {
