@@ -464,11 +464,17 @@ def batched_leg(dev, prec="fp16", reps=5):
             "tflops_22n3": flops / (ms * 1e-3) / 1e12}
 
 
+SERVE_LIMIT_S = 20.0  # a served request that takes longer (they take milliseconds) has stalled
+
+
 def serving_leg(dev, args, prec="fp16"):
     """Interleaved ADMM solves (min <C,X>, diag X = 1, X PSD; C = -L/4 with L the Laplacian of
     G(n, 0.01): the max-cut SDP, n in {500, 2000, 8000}, seeds 8-10) as Poisson-arriving requests
     to one psd_server.  (With C = L itself the optimum is 0 at X = 11^T and the surrogate's
-    relative gap does not converge under ADMM even with FP32 projections.)"""
+    relative gap does not converge under ADMM even with FP32 projections.)
+
+    Every wait has a limit.  When one runs out the leg reports that it is not finished and
+    leaves the server as it is: destroying it would wait for the same work."""
     import numpy as np
     import torch
     from paper_2507_09165_gb300 import admm, binding as b, synth
@@ -483,18 +489,26 @@ def serving_leg(dev, args, prec="fp16"):
                 o = torch.empty_like(C)
                 warm.append((b.psd_server_submit(server, n, C, n, o, n, prec), o))
         for t, _ in warm:
-            b.psd_server_wait(server, t)
+            b.psd_server_wait(server, t, int(1000 * SERVE_LIMIT_S))
         # untimed warm-up phase of the same workload (the first seconds on a fresh
         # process have run at half the throughput)
         admm.run_serving(server, graphs, prec, solve_rate=args.serve_rate, arrival_seconds=1.0,
-                         iters=max(5, args.serve_iters // 5), seed=99)
+                         iters=max(5, args.serve_iters // 5), seed=99, request_limit_s=SERVE_LIMIT_S)
         base = b.psd_server_stats(server)
         with Clocks(dev.index or 0) as clk:
             res = admm.run_serving(server, graphs, prec, solve_rate=args.serve_rate,
-                                   arrival_seconds=args.serve_seconds, iters=args.serve_iters, seed=5)
+                                   arrival_seconds=args.serve_seconds, iters=args.serve_iters, seed=5,
+                                   request_limit_s=SERVE_LIMIT_S)
         st = b.psd_server_stats(server)
-    finally:
+    except (TimeoutError, b.PsdError) as e:
+        if isinstance(e, b.PsdError) and b.STATUS.get(e.status) != "PSD_ERR_TIMEOUT":
+            b.psd_server_destroy(server)
+            raise
+        return {"unfinished": str(e) or "a served request timed out"}
+    except BaseException:
         b.psd_server_destroy(server)
+        raise
+    b.psd_server_destroy(server)
     out = admm.summarize(res)
     out.update(workload="ADMM solves of min <C,X>, diag(X) = 1, X PSD (max-cut: C = -L/4, L the Laplacian of "
                         "G(n, 0.01)), n in {500, 2000, 8000} (seeds 8-10); solves Poisson at %.1f/s for %.1f s, "
@@ -540,6 +554,19 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
+def note(text):
+    print("[bench] " + text, file=sys.stderr, flush=True)
+
+
+def leg(name, fn, *args):
+    """Runs one leg of the bench, named on stderr as it starts and ends."""
+    note(name + " ...")
+    t0 = time.perf_counter()
+    res = fn(*args)
+    note("%s done in %.1f s" % (name, time.perf_counter() - t0))
+    return res
+
+
 def run_ours(args):
     import numpy as np
     import torch
@@ -565,6 +592,7 @@ def run_ours(args):
     Xd = Xh.to(dev)
     out = torch.empty_like(Xd)
     s = torch.cuda.current_stream(dev)
+    note("projection ...")
     for _ in range(max(args.warmup, 3)):
         b.psd_project(n, Xd, n, out, prec, s)
     info = b.psd_last_info(s)
@@ -631,6 +659,7 @@ def run_ours(args):
         s.wait_stream(s_out)
         s.wait_stream(s_in)
 
+    note("projection done, end to end ...")
     if e2e_steps:
         e2e_pass(2)
     torch.cuda.synchronize(dev)
@@ -642,6 +671,7 @@ def run_ours(args):
     torch.cuda.synchronize(dev)
     barrier()
     e2e_ms = reduce_max(ev0.elapsed_time(ev1) / e2e_steps, dev) if e2e_steps else None
+    note("end to end done, product kernel and FP32 path ...")
 
     # dominant kernel: the symmetric tensor-core product of the chain, same kernel, shape and
     # form as in the projection (mixed: the FP16-pair split product of stages 2-3; fp16/bf16:
@@ -685,24 +715,26 @@ def run_ours(args):
         ev1.record(s)
         torch.cuda.synchronize(dev)
         fp32_ms = ev0.elapsed_time(ev1) / k32
+    note("product kernel and FP32 path done")
     batched = None
     if rank == 0 and not args.no_batched:
-        batched = batched_leg(dev)
-    serving = None
-    if rank == 0 and not args.no_serve:
-        serving = serving_leg(dev, args)
+        batched = leg("batched", batched_leg, dev)
     bands = None
     if rank == 0 and not args.no_bands:
-        bands = bands_leg(dev)
+        bands = leg("bands", bands_leg, dev)
     deflate = None
     if rank == 0 and not args.no_deflate:
-        deflate = deflate_leg(dev, n)
+        deflate = leg("deflation", deflate_leg, dev, n)
     acc = None
     if rank == 0 and not args.no_accuracy:
-        acc = accuracy_check(n, prec, dev)
+        acc = leg("accuracy", accuracy_check, n, prec, dev)
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu:
-        cpu = cpu_baseline(n)
+        cpu = leg("cpu baseline", cpu_baseline, n)
+    # last, so that nothing measured above depends on the server finishing
+    serving = None
+    if rank == 0 and not args.no_serve:
+        serving = leg("serving", serving_leg, dev, args)
 
     if rank == 0:
         value = job_ms_per_projection(ms_step, world)
@@ -745,6 +777,9 @@ def run_ours(args):
             "info": {k: info[k] for k in ("lambda_bound", "lanczos_steps", "overshoot_max", "compl_resid")},
         }
         print(json.dumps(line), flush=True)
+    if serving and "unfinished" in serving:
+        sys.stderr.flush()
+        os._exit(0)  # the line is out; the server and the device are not waited for
     if world > 1:
         torch.distributed.destroy_process_group()
 

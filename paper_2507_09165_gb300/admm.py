@@ -93,7 +93,7 @@ class Solve:
 
 
 def run_serving(server, graphs, precision="fp16", solve_rate=8.0, arrival_seconds=2.5, iters=50,
-                think_ms=0.5, seed=0, sigma_range=(0.5, 2.0), max_solves=None):
+                think_ms=0.5, seed=0, sigma_range=(0.5, 2.0), max_solves=None, request_limit_s=None):
     """Interleaved ADMM solves as a request stream against a psd_server.
 
     graphs: {n: C} device float32 tensors (one Laplacian per size class).
@@ -102,6 +102,8 @@ def run_serving(server, graphs, precision="fp16", solve_rate=8.0, arrival_second
     sigma drawn log-uniformly from sigma_range; each runs `iters` iterations,
     issuing the next request an Exp(think_ms) time after the previous one
     completes.  Returns per-request records and per-solve summaries.
+    request_limit_s: raises TimeoutError once a request has not completed that
+    many seconds after its submission (None: no limit).
     """
     import torch
     from . import binding as b
@@ -135,6 +137,7 @@ def run_serving(server, graphs, precision="fp16", solve_rate=8.0, arrival_second
                 V = sv.make_input()
                 a["ticket"] = b.psd_server_submit(server, sv.n, V, sv.n, sv.S, sv.n, precision, ready=sv.ready)
                 a["state"] = "wait"
+                a["t_submit"] = now
             if a["state"] == "wait":
                 done, info, lat = b.psd_server_poll(server, a["ticket"])
                 if done:
@@ -149,6 +152,8 @@ def run_serving(server, graphs, precision="fp16", solve_rate=8.0, arrival_second
                         continue
                     a["state"] = "think"
                     a["t_next"] = now + rng.exponential(think_ms * 1e-3)
+                elif request_limit_s is not None and now - a["t_submit"] > request_limit_s:
+                    raise TimeoutError("a request of order %d has not completed in %g s" % (sv.n, request_limit_s))
             still.append(a)
         active = still
         if active and all(a["state"] == "wait" for a in active) and nxt >= len(arrivals):
