@@ -675,23 +675,23 @@ def run_ours(args):
 
     # dominant kernel: the symmetric tensor-core product of the chain, same kernel, shape and
     # form as in the projection (mixed: the FP16-pair split product of stages 2-3; fp16/bf16:
-    # the 16-bit product; both on SM pairs; fp32: the same FP16-pair split product, which the
-    # chain runs with scaled operands and promoted accumulation), timed alone with CUDA events on the launching stream
+    # the 16-bit product; fp32: the scaled-pair product with promoted accumulation; all on SM
+    # pairs), timed alone with CUDA events on the launching stream
     ld = (n + 63) // 64 * 64
-    kprec = {"mixed": "mixed", "fp32": "mixed", "bf16": "bf16"}.get(prec, "fp16")
+    kprec = {"mixed": "mixed", "fp32": "fp32", "bf16": "bf16"}.get(prec, "fp16")
     parts, et = {"mixed": (2, torch.float16), "fp32": (2, torch.float16),
                  "bf16": (1, torch.bfloat16)}.get(prec, (1, torch.float16))
     A = (torch.randn(parts, n, ld, device=dev) / math.sqrt(n)).to(et)
     if parts == 2:
         A[1].mul_(1.0 / 2048)  # lo part of a hi/lo pair
     C = torch.empty_like(A)
-    form = b.EPI_CTA_PAIR
+    form, scales = (b.EPI_SCALED_PAIR, (1.0, 1.0, 1.0)) if prec == "fp32" else (b.EPI_CTA_PAIR, ())
     for _ in range(3):
-        b.psd_symm_product(n, A, A, ld, C, 0, kprec, form, stream=s)
+        b.psd_symm_product(n, A, A, ld, C, 0, kprec, form, params=scales, stream=s)
     reps = 20 if parts == 1 else 8
     ev0.record(s)
     for _ in range(reps):
-        b.psd_symm_product(n, A, A, ld, C, 0, kprec, form, stream=s)
+        b.psd_symm_product(n, A, A, ld, C, 0, kprec, form, params=scales, stream=s)
     ev1.record(s)
     torch.cuda.synchronize(dev)
     gemm_ms = ev0.elapsed_time(ev1) / reps

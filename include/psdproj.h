@@ -192,6 +192,13 @@ psd_status_t psd_project_batched(int32_t count, const psd_block_desc_t *d_descs,
 #define PSD_EPI_GROUPED 0x100
 #define PSD_EPI_F16_PAIR_OUT 0x200
 #define PSD_EPI_CTA_PAIR 0x400
+/*   PSD_EPI_SCALED_PAIR (FP32, epi 0-3, no other flag): run the FP32 path's kernel.
+ *     Every operand (A, B, C, Y) is an FP16 hi/lo pair of its values times a power
+ *     of two, n*ld elements a part; the epilogue's own params are followed by
+ *     {in_scale, y_scale, out_scale}: the products' sum (rounded to FP32 every 128
+ *     K) is multiplied by in_scale, Y by y_scale, and C is split (saturating) from
+ *     value * out_scale; all three powers of two. */
+#define PSD_EPI_SCALED_PAIR 0x800
 
 /* Symmetric product C = epi(A * B) of two n x n symmetric matrices in the
  * chain's storage (A, B, C share the leading dimension ld, a multiple of 8;
@@ -199,7 +206,7 @@ psd_status_t psd_project_batched(int32_t count, const psd_block_desc_t *d_descs,
  * tensor cores and mirrored, so C is exactly symmetric.
  *   precision FP16 / BF16: single 16-bit matrices;
  *   precision MIXED: FP16 pairs (epi 0-2), precision FP32: TF32 pairs (FP32
- *     containers): every operand (A, B, C, Y) is two matrices stored back to
+ *     containers; the FP32 projection itself runs PSD_EPI_SCALED_PAIR): every operand (A, B, C, Y) is two matrices stored back to
  *     back, hi at M and lo at M + n*ld elements, value = hi + lo; the product
  *     is A_hi B_hi + A_hi B_lo + A_lo B_hi in one FP32 accumulator (TF32:
  *     folded every 128 K into a round-to-nearest running sum).

@@ -221,7 +221,7 @@ def psd_project_batched(count, d_descs, precision="bf16", stream=None):
 
 
 _PRODUCT_BYTES = {"fp16": (1, 2), "bf16": (1, 2), "mixed": (2, 2), "fp32": (2, 4), "fp8_late": (1, 1)}
-_FP8_PARAMS = {0: 3, 1: 6, 2: 4}  # epilogue params followed by (in_scale, y_scale, out_scale)
+_SCALED_PARAMS = {0: 3, 1: 6, 2: 4, 3: 4}  # epilogue params followed by (in_scale, y_scale, out_scale)
 
 
 def _check_extent(t, need, what):
@@ -235,6 +235,7 @@ def _check_extent(t, need, what):
 EPI_GROUPED = 0x100         # PSD_EPI_GROUPED
 EPI_F16_PAIR_OUT = 0x200    # PSD_EPI_F16_PAIR_OUT
 EPI_CTA_PAIR = 0x400        # PSD_EPI_CTA_PAIR
+EPI_SCALED_PAIR = 0x800     # PSD_EPI_SCALED_PAIR
 
 
 def psd_symm_product(n, A, B, ld, C, ld_out=0, precision="fp16", epi=0, params=(), aux=None, ld_aux=0,
@@ -244,6 +245,8 @@ def psd_symm_product(n, A, B, ld, C, ld_out=0, precision="fp16", epi=0, params=(
     if pname in _PRODUCT_BYTES and n > 0:
         parts, esz = _PRODUCT_BYTES[pname]
         need = ((parts - 1) * n * ld + (n - 1) * ld + n) * esz  # pairs: hi, then lo at + n * ld
+        if epi & EPI_SCALED_PAIR:
+            need = 4 * n * ld  # FP16 pairs, whole rows
         _check_extent(A, need, "A")
         _check_extent(B, need, "B")
         if kind == 3:
@@ -253,8 +256,9 @@ def psd_symm_product(n, A, B, ld, C, ld_out=0, precision="fp16", epi=0, params=(
             _check_extent(C, need + (n * ld * esz if epi & EPI_F16_PAIR_OUT else 0), "C")
             if kind == 1:
                 _check_extent(aux, need, "aux (Y)")
-    if pname == "fp8_late" and len(params) < _FP8_PARAMS.get(kind, 0):
-        raise ValueError("fp8_late epilogue %d takes %d params" % (kind, _FP8_PARAMS[kind]))
+    scaled = pname == "fp8_late" or epi & EPI_SCALED_PAIR
+    if scaled and len(params) < _SCALED_PARAMS.get(kind, 0):
+        raise ValueError("epilogue %d with scales takes %d params" % (kind, _SCALED_PARAMS[kind]))
     arr = (ctypes.c_double * max(1, len(params)))(*params) if params else None
     _check(lib().psd_symm_product(n, _ptr(A), _ptr(B), ld, _ptr(C), ld_out, _prec(precision), epi, arr,
                                   _ptr(aux), ld_aux, _ptr(d_absmax), _stream(stream)), "psd_symm_product")

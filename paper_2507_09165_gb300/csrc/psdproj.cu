@@ -527,7 +527,10 @@ psd_status_t psd_symm_product(int64_t n, const void* A, const void* B, int64_t l
   epi &= 0xFF;
   const bool grouped = (flags & PSD_EPI_GROUPED) != 0, pair_out = (flags & PSD_EPI_F16_PAIR_OUT) != 0;
   const bool cta_pair = (flags & PSD_EPI_CTA_PAIR) != 0;
-  if (flags & ~(PSD_EPI_GROUPED | PSD_EPI_F16_PAIR_OUT | PSD_EPI_CTA_PAIR)) return PSD_ERR_INVALID_ARG;
+  const bool scaled = flags == PSD_EPI_SCALED_PAIR;  // the FP32 path's kernel
+  if ((flags & ~(PSD_EPI_GROUPED | PSD_EPI_F16_PAIR_OUT | PSD_EPI_CTA_PAIR)) != 0 && !scaled)
+    return PSD_ERR_INVALID_ARG;
+  if (scaled && (precision != PSD_PREC_FP32 || !params)) return PSD_ERR_INVALID_ARG;
   if ((grouped || pair_out) && (split || f8 || epi == 3)) return PSD_ERR_INVALID_ARG;
   if (cta_pair && (f8 || precision == PSD_PREC_FP32)) return PSD_ERR_INVALID_ARG;
   if (grouped && cta_pair) return PSD_ERR_INVALID_ARG;
@@ -559,9 +562,11 @@ psd_status_t psd_symm_product(int64_t n, const void* A, const void* B, int64_t l
     ps.d_state = reinterpret_cast<DevState*>(sm + o_state);
     ps.d_block = reinterpret_cast<BlockRec*>(sm + o_block);
   }
-  const int64_t tkey = cta_pair ? -n : n;  // the pair form's 256-row tiles under -n
+  // the pair form's 256-row tiles under -n, the FP32 path's of their own width under -n - kMaxOrder
+  const int64_t tkey = scaled ? -n - kMaxOrder : cta_pair ? -n : n;
+  const int width = scaled ? pair_tile_width(n) : 256;
   if (!ps.tiles.count(tkey)) {
-    std::vector<int4> tl = cta_pair ? make_tile_list_pair(n) : make_tile_list(n);
+    std::vector<int4> tl = scaled || cta_pair ? make_tile_list_pair(n, 0, 8, width) : make_tile_list(n);
     int4* d = nullptr;
     if (cudaMalloc(&d, sizeof(int4) * tl.size()) != cudaSuccess) return PSD_ERR_NO_MEMORY;
     cudaMemcpy(d, tl.data(), sizeof(int4) * tl.size(), cudaMemcpyHostToDevice);
@@ -570,6 +575,7 @@ psd_status_t psd_symm_product(int64_t n, const void* A, const void* B, int64_t l
   }
   const int dtype = precision == PSD_PREC_BF16    ? DT_BF16
                     : precision == PSD_PREC_MIXED ? DT_F16X2
+                    : scaled                      ? DT_F16X2
                     : precision == PSD_PREC_FP32  ? DT_TF32X3
                     : f8                          ? DT_E4M3
                                                   : DT_F16;
@@ -597,12 +603,12 @@ psd_status_t psd_symm_product(int64_t n, const void* A, const void* B, int64_t l
     set_lambda_kernel<<<1, 1, 0, s>>>(ps.d_state, params[0]);
     g.ep.absmax = nullptr;
   }
-  if (f8) {
+  if (f8 || scaled) {
     const double* sc = params + (epi == 0 ? 0 : epi == 1 ? 3 : 1);
     g.ep.in_scale = static_cast<float>(sc[0]);
     g.ep.y_scale = static_cast<float>(sc[1]);
     g.ep.out_scale = static_cast<float>(sc[2]);
-    g.ep.absmax = nullptr;
+    if (f8) g.ep.absmax = nullptr;
   }
   BlockRec br{};
   br.off = 0;
@@ -616,7 +622,15 @@ psd_status_t psd_symm_product(int64_t n, const void* A, const void* B, int64_t l
   }
   if (enqueue_set_block(ps.d_block, br, s) != cudaSuccess) return PSD_ERR_CUDA;
   cudaError_t e;
-  if (cta_pair && !split) {
+  if (scaled) {
+    g.tile_w = width;
+    CUtensorMap tm[4];
+    const uint8_t* parts[4] = {static_cast<const uint8_t*>(A), static_cast<const uint8_t*>(A) + pair,
+                               static_cast<const uint8_t*>(B), static_cast<const uint8_t*>(B) + pair};
+    for (int i = 0; i < 4; ++i)
+      if (!encode_tmap(&tm[i], dtype, parts[i], n, ld, i < 2 ? 128 : g.b_rows(), kRowBytesF32)) return PSD_ERR_CUDA;
+    e = launch_symgemm_f32(epi, tm, g, num_sms(), s);
+  } else if (cta_pair && !split) {
     CUtensorMap ta, tb;
     if (!encode_tmap(&ta, dtype, A, n, ld, 128) || !encode_tmap(&tb, dtype, B, n, ld, 128)) return PSD_ERR_CUDA;
     const uint32_t fmt = dtype == DT_BF16 ? 1u : 0u;
