@@ -279,20 +279,24 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 // Tensor memory of a CTA pair from start to end: every thread of both CTAs calls
-// both functions, warp 1 of each CTA allocates and frees.  An allocation is one
+// the three functions, warp 1 of each CTA allocates and frees.  An allocation is one
 // operation of two CTAs that blocks without a limit, so each step of one CTA that
 // the other's may depend on has a cluster barrier between them:
 //   before the allocation: both CTAs run (and have initialised their mbarriers);
 //     without it the leader's allocation can begin while the peer has not been
-//     started on its SM;
+//     started on its SM (tmem_pair_enter arrives, so that the CTA's own setup
+//     hides the barrier);
 //   before the permit is given up: both allocations are made;
 //   before the release: both CTAs have finished with tensor memory;
 //   after it: neither CTA leaves its SM while the other's release is under way.
 // Returns the address of the allocation (the same in both CTAs).
+__device__ __forceinline__ void tmem_pair_enter() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t tmem_pair_setup(volatile uint32_t* holder, uint32_t ncols) {
   const bool alloc_warp = (threadIdx.x >> 5) == 1;
   __syncwarp();
-  cluster_sync_all();
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   if (alloc_warp) tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(holder)), ncols);
   tc_fence_before();
   cluster_sync_all();

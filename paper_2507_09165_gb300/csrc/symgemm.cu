@@ -574,6 +574,7 @@ __global__ void __launch_bounds__(threads16(EW), 1)
   static_assert(OUTK != 1 && (EPI != EPI_FINAL || OUTK == 0), "pair form: 16-bit operands, no e4m3 output");
   static_assert(EW == 4 || EW == 8, "4 or 8 epilogue warps");
   constexpr int kStagesP = stages_pair(EW);
+  tmem_pair_enter();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));

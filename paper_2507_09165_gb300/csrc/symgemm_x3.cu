@@ -347,6 +347,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int kBBytes = X3Cfg<B1, PAIR>::kBBytes;
   constexpr bool kSW64 = X3Cfg<B1, PAIR>::kSW64;
   auto desc = [](uint32_t a) { return kSW64 ? sw64_kmajor_desc(a) : sw128_kmajor_desc(a); };
+  if constexpr (PAIR) tmem_pair_enter();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));

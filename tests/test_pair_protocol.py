@@ -42,7 +42,8 @@ def _order(body, *steps):
 
 def test_both_ctas_run_before_the_allocation_and_have_it_before_the_permit_goes():
     body = _body(_sources()["ptx.cuh"], "tmem_pair_setup")
-    _order(body, "cluster_sync_all()", "tmem_alloc_pair(", "cluster_sync_all()", "tmem_relinquish_pair(")
+    _order(body, "barrier.cluster.wait", "tmem_alloc_pair(", "cluster_sync_all()", "tmem_relinquish_pair(")
+    assert "barrier.cluster.arrive" in _body(_sources()["ptx.cuh"], "tmem_pair_enter")
 
 
 def test_no_cta_leaves_while_the_other_releases():
@@ -60,9 +61,10 @@ def test_kernels_on_pairs_use_nothing_else():
             assert raw not in code, (name, raw)
         if "mma_commit_pair(" in code:
             kernels += 1
-            assert code.count("tmem_pair_setup(") == 1 and code.count("tmem_pair_teardown(") == 1, name
+            for step in ("enter", "setup", "teardown"):
+                assert code.count("tmem_pair_%s(" % step) == 1, name
             # the producer waits for the ring's last commits between the tiles and the release
-            tail = _order(code, "tmem_pair_setup(", "tma_load_2d_pair(")
+            tail = _order(code, "tmem_pair_enter(", "tmem_pair_setup(", "tma_load_2d_pair(")
             m = re.search(r"for \(int q = 0; ok && q < kStages\w*; \+\+q\) \{\s*"
                           r"ok = wait_bounded\(empty_bar\(s\), ph \^ 1u, abort_flag\);", tail)
             assert m and m.start() < tail.index("tmem_pair_teardown("), name
