@@ -30,9 +30,9 @@ METRIC = "ms per n=10k PSD projection at rel err ≤1e-3 vs FP32 path; tensor-pi
 # one ncu capture of the bench's own roofline launch, n = 10,000), valid only while the kernel's
 # sources are the ones captured (sha256 over the files below); null otherwise.
 ROOFLINE_TRAFFIC = {
-    "mixed": {"bytes": 2117522688 + 381887744,
+    "mixed": {"bytes": 2037175808 + 381580288,
               "sources": ("paper_2507_09165_gb300/csrc/symgemm_x3.cu", "paper_2507_09165_gb300/csrc/ptx.cuh"),
-              "sha256": "4df80dbaa3b2fbc1dcc36d6d68e3344d1b60ed30f4da79b31f7d584e8cd7a311",
+              "sha256": "dc2a560c16b1452706429f42bff807abe8f0214a2f7bc0a901d8f71c75ec8b2c",
               "profile": "profiles/symgemm_x3_pair_traffic_n10000.md"},
 }
 
@@ -43,14 +43,18 @@ ROOFLINE_TRAFFIC = {
 # Valid only while the sources of the projection's kernels and launch sequence are the ones
 # captured (sha256 over TENSOR_PIPE_SOURCES; the batched, server, deflation and no-allocation
 # translation units do not take part in a single projection).
-TENSOR_PIPE_SOURCES = ("chain.h", "internal.h", "normbound.cu", "psdproj.cu", "ptx.cuh", "symgemm.cu",
+TENSOR_PIPE_SOURCES = ("chain.h", "epilogue.cuh", "internal.h", "normbound.cu", "normbound.cuh",
+                       "normbound_cluster.cuh", "psdproj.cu", "ptx.cuh", "symgemm.cu", "symgemm_f32.cu",
                        "symgemm_x3.cu", "tridiag.cuh")
 TENSOR_PIPE = {
-    "mixed": {"projection_pct": 76.46, "products_pct": 87.16,
-              "sha256": "454acbe484f18579ca1009885be5105da92691aab1572739f8c6b05776700208",
+    "mixed": {"projection_pct": 76.52, "products_pct": 85.59,
+              "sha256": "eb4e14bee9b36157bbff5d5a02a4413d4b5dc77287d8eb8470075a189b7396ab",
               "profile": "profiles/tensor_pipe_n10000.md"},
-    "fp16": {"projection_pct": 71.10, "products_pct": 83.85,
-             "sha256": "454acbe484f18579ca1009885be5105da92691aab1572739f8c6b05776700208",
+    "fp16": {"projection_pct": 70.85, "products_pct": 81.82,
+             "sha256": "eb4e14bee9b36157bbff5d5a02a4413d4b5dc77287d8eb8470075a189b7396ab",
+             "profile": "profiles/tensor_pipe_n10000.md"},
+    "fp32": {"projection_pct": 80.33, "products_pct": 83.39,
+             "sha256": "eb4e14bee9b36157bbff5d5a02a4413d4b5dc77287d8eb8470075a189b7396ab",
              "profile": "profiles/tensor_pipe_n10000.md"},
 }
 

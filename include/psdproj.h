@@ -67,7 +67,9 @@ typedef enum {
                          is three FP16 tensor-core products of hi/lo split
                          operands (about 22 bits: FP16 pairs of the values times
                          a power of two; the splitting of Ootomo & Yokota 2022),
-                         FP32 sums rounded to nearest every 128 terms */
+                         FP32 sums rounded to nearest every 128 terms; entries of
+                         X below 2^-17 of the bound keep fewer bits (a step of
+                         2^-39 of the bound) */
   PSD_PREC_FP16 = 1,  /* f~*_half (Table 2), T = 7, 22 products, FP16 operands,
                          FP32 accumulation in tensor memory */
   PSD_PREC_BF16 = 2,  /* as FP16 with BF16 operands */

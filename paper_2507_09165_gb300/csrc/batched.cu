@@ -51,7 +51,7 @@ struct BatchPlan {
   int nsymv = 0;
   int4* d_cast = nullptr;
   int ncast = 0;
-  double* d_cres = nullptr;  // 4 per tile position: shares of <out, X - out> (final product)
+  double* d_cres = nullptr;  // shares of <out, X - out> (final product): 4, 8 or 16 per tile position
   int* d_cidx = nullptr;     // per block, in its own tile order: positions in the tile list
   int2* d_crange = nullptr;  // per block: (first entry of d_cidx, count)
   uint8_t* small = nullptr;

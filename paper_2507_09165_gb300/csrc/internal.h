@@ -77,9 +77,8 @@ struct BlockRec {
   int64_t db, dc, dy;
   // EPI_FINAL with EpiParams::cres unset: if set, the shares of <out, X - out>
   // of the tile at launch position t go to cres at the tile's position in the
-  // request's own tile list, t + cres_shift (a served request), EW per 128-row
-  // tile (EW epilogue warps); on SM pairs 2 EW per tile: EW (2 (t + cres_shift) +
-  // rank) + warp.
+  // request's own tile list, t + cres_shift (a served request; one-SM kernel, EW
+  // per 128-row tile, EW epilogue warps).
   double* cres;
   int64_t cres_shift;
 };

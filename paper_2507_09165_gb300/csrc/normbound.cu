@@ -726,8 +726,8 @@ struct GridBarrier {
 };
 
 // The whole bound in one launch: the phases of the multi-launch path in the
-// same order, separated by grid barriers instead of kernel boundaries (about
-// 150 of them, each a few microseconds shorter than a kernel boundary, and no
+// same order, separated by grid barriers instead of kernel boundaries (108 of
+// them, each a few microseconds shorter than a kernel boundary, and no
 // launch of a small FP64 vector kernel waits on an empty GPU).
 //
 // RESIDENT: at most two tiles per CTA, loaded once -- the first into registers,

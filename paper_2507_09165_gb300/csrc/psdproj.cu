@@ -131,7 +131,7 @@ struct Plan {
   int ntiles_bal = 0;
   int tile_w = 0;
   int ncompl = 0;  // complementarity shares the final product writes (4 per one-SM tile, 16 per pair tile)
-  double* d_compl = nullptr;  // 4 per tile: shares of <out, X - out> from the final product
+  double* d_compl = nullptr;  // the shares of <out, X - out> from the final product
   cudaGraphExec_t exec = nullptr;
   bool graph_tried = false;
   int launches = 0;  // kernel launches of one projection (graph nodes + argument block)

@@ -547,15 +547,14 @@ __global__ void __launch_bounds__(threads16(EW), 1)
 // 256 x 256 blocks of the upper triangle, diagonal blocks in full (chunks
 // below the diagonal are computed but not written).  Epilogues: copy,
 // polynomial and scale with a 16-bit or FP16-pair output, and the final
-// product (FP32 output; with 4 epilogue warps per CTA, the eight of a pair
-// tile write the complementarity shares of the two 128-row tiles of the
-// one-SM form, in its order: slots 8 t + 4 rank + warp quarter).
-// EW epilogue warps per CTA: 4 with a 6-stage ring (single matrices, long
-// K), or 8 with a 5-stage ring (the blocks of a block-diagonal cone: K <=
-// 1024, where one warp per 32-lane quarter no longer drains a tile within
-// the next tile's main loop); with 8, a quarter's two warps take alternate
-// 32-column chunks and FINAL writes 16 shares per pair tile (2 EW t + EW rank
-// + warp).
+// product (FP32 output, 2 EW complementarity shares per tile: 2 EW t + EW rank +
+// warp; with EW = 4 the warp is its quarter).
+// EW epilogue warps per CTA: 4 with a 6-stage ring (the stage products of single
+// matrices, long K), or 8 with a 5-stage ring (the blocks of a block-diagonal cone:
+// K <= 1024, where one warp per 32-lane quarter no longer drains a tile within the
+// next tile's main loop; and the final product, which reads X and writes both
+// triangles in FP32); with 8, a quarter's two warps take alternate 32-column chunks.
+// Setup and release of tensor memory: tmem_pair_setup, tmem_pair_teardown (ptx.cuh).
 constexpr int kBHalfBytes = kBM * kRowBytes16;          // 16 KB: 128 rows of B
 constexpr int kStageBytesP = kABytes16 + kBHalfBytes;  // 32 KB
 __host__ __device__ constexpr int stages_pair(int ew) { return ew == 4 ? 6 : 5; }
@@ -756,13 +755,9 @@ __global__ void __launch_bounds__(threads16(EW), 1)
       if (!wait_bounded(tfull_bar(acc), acc_ph, abort_flag)) break;
       tc_fence_after();
       const float lam = EPI == EPI_FINAL ? static_cast<float>(br.st->lambda) : 0.f;
-      // shares at the launch position t, or (a served request) at its tile's
-      // position in the request's own list, t + cres_shift
       double* cdst = nullptr;
-      if (EPI == EPI_FINAL)
-        cdst = p.ep.cres ? p.ep.cres + 2 * EW * static_cast<int64_t>(t) + EW * static_cast<int>(rank)
-               : br.cres ? br.cres + 2 * EW * (static_cast<int64_t>(t) + br.cres_shift) + EW * static_cast<int>(rank)
-                         : nullptr;
+      if (EPI == EPI_FINAL && p.ep.cres)
+        cdst = p.ep.cres + 2 * EW * static_cast<int64_t>(t) + EW * static_cast<int>(rank);
       ComplAcc cacc;
       ComplAcc* cap = cdst ? &cacc : nullptr;
 #pragma unroll 1
